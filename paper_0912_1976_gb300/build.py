@@ -19,6 +19,7 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler",
           "-I", os.path.join(ROOT, "include")]
 UNITS = {
     "setup.cu": ["-fmad=false"],
+    "dense.cu": [],
     "layout.cu": [],
     "solve.cu": [],
     "batch.cu": [],

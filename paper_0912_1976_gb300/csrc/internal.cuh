@@ -317,6 +317,11 @@ int persist_profile(vemg_hierarchy *h, int cap, int *count, int *op, int *level,
 void assemble(const vemg_mesh *mesh, vemg_csr *A_out, cudaStream_t s);
 void load_vector(const vemg_mesh *mesh, const double *f, double *b, cudaStream_t s);
 void setup(vemg_hierarchy *h, const vemg_csr *A, const vemg_mesh *mesh, cudaStream_t s);
+// dense.cu
+constexpr int kDenseTile = 32;
+inline int dense_padded(int n) { return (n + kDenseTile - 1) / kDenseTile * kDenseTile; }
+void dense_spd_inverse(int n, double *D, double *G, int *err, cudaStream_t s);
+void dense_project(int n, double *G, const double *v, cudaStream_t s);
 // layout.cu
 void build_solve_layout(vemg_hierarchy *h, cudaStream_t s);
 // solve.cu

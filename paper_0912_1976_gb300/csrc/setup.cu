@@ -1578,123 +1578,33 @@ static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
 // ------------------------------------------------------------------------------------------
 // coarsest level: dense inverse (projected onto the complement of constants if singular)
 
-__global__ void k_dense_fill(int n, const int *__restrict__ rp, const int *__restrict__ ci,
-                             const double *__restrict__ v, double *D) {
+// D (np x np, np >= n): the level's matrix plus sigma v v^T (v null: the constants), and the identity in
+// the rows and columns past n. One block per row.
+__global__ void k_dense_fill(int n, int np, const int *__restrict__ rp, const int *__restrict__ ci,
+                             const double *__restrict__ v, double sigma, const double *__restrict__ nu, double *D) {
     int i = blockIdx.x;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) D[(int64_t)i * n + j] = 0.0;
-    __syncthreads();
-    for (int k = rp[i] + threadIdx.x; k < rp[i + 1]; k += blockDim.x) D[(int64_t)i * n + ci[k]] = v[k];
-}
-
-// in-place right-looking Cholesky (lower) of D + sigma 1 1^T, one block
-__global__ void k_dense_cholesky(int n, double *D, double sigma, int *err) {
-    if (sigma != 0.0)
-        for (int k = threadIdx.x; k < n * n; k += blockDim.x) D[k] = D[k] + sigma;
-    __syncthreads();
-    __shared__ double piv;
-    for (int j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            double djj = D[(int64_t)j * n + j];
-            if (!(djj > 0.0)) {
-                atomicCAS(err, 0, VEMG_EBREAKDOWN);
-                djj = 1.0;
-            }
-            piv = sqrt(djj);
-            D[(int64_t)j * n + j] = piv;
-        }
-        __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) D[(int64_t)i * n + j] /= piv;
-        __syncthreads();
-        int m = n - j - 1;
-        for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-            int i = j + 1 + t / m, k = j + 1 + t % m;
-            if (k <= i) D[(int64_t)i * n + k] -= D[(int64_t)i * n + j] * D[(int64_t)k * n + j];
-        }
-        __syncthreads();
-    }
-}
-
-// column c of the inverse: solve L L^T x = e_c; one thread per column
-__global__ void k_dense_inverse_cols(int n, const double *__restrict__ L, double *G) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    // forward: L y = e_c (stored in column c of G)
-    for (int i = 0; i < n; ++i) {
-        double s = (i == c) ? 1.0 : 0.0;
-        for (int k = 0; k < i; ++k) s -= L[(int64_t)i * n + k] * G[(int64_t)k * n + c];
-        G[(int64_t)i * n + c] = s / L[(int64_t)i * n + i];
-    }
-    for (int i = n - 1; i >= 0; --i) {
-        double s = G[(int64_t)i * n + c];
-        for (int k = i + 1; k < n; ++k) s -= L[(int64_t)k * n + i] * G[(int64_t)k * n + c];
-        G[(int64_t)i * n + c] = s / L[(int64_t)i * n + i];
-    }
-}
-
-// G := Q G Q, Q = I - 1 1^T / n (G symmetric)
-__global__ void k_project_dense(int n, double *G) {
-    __shared__ double rowmean[1024];
-    __shared__ double total;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double s = 0.0;
-        for (int j = 0; j < n; ++j) s += G[(int64_t)i * n + j];
-        rowmean[i] = s / n;
+    double *row = D + (int64_t)i * np;
+    for (int j = threadIdx.x; j < np; j += blockDim.x) {
+        double d = i == j ? 1.0 : 0.0;
+        if (i < n && j < n) d = nu ? sigma * nu[i] * nu[j] : sigma;
+        row[j] = d;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += rowmean[i];
-        total = s / n;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-        int i = t / n, j = t % n;
-        G[t] = G[t] - rowmean[i] - rowmean[j] + total;
-    }
+    if (i >= n) return;
+    for (int k = rp[i] + threadIdx.x; k < rp[i + 1]; k += blockDim.x) row[ci[k]] += v[k];
 }
 
-__global__ void k_trace(int n, const int *__restrict__ rp, const int *__restrict__ ci,
-                        const double *__restrict__ v, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// sum of the diagonal in row order (the order of the definition: sigma enters every element of D, and
+// a last-bit change of it would show in the inverse, magnified by the condition number). One block
+// loads the diagonal, one thread adds it up.
+__global__ void __launch_bounds__(1024) k_trace(int n, const double *__restrict__ diag, double *out) {
+    __shared__ double sh[1024];
+    if (threadIdx.x < n) sh[threadIdx.x] = diag[threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     double s = 0.0;
-    for (int i = 0; i < n; ++i)
-        for (int k = rp[i]; k < rp[i + 1]; ++k)
-            if (ci[k] == i) s += v[k];
+    for (int i = 0; i < n; ++i) s += sh[i];
     *out = s;
-}
-
-// D += sigma nu nu^T (the rank-one regularisation of a singular chain with nullspace nu)
-__global__ void k_dense_rank1(int n, double *D, double sigma, const double *__restrict__ nu) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * n; t += gridDim.x * blockDim.x) {
-        int i = t / n, j = t % n;
-        D[t] += sigma * nu[i] * nu[j];
-    }
-}
-
-// G := Q G Q, Q = I - nu nu^T / (nu^T nu) (G symmetric); one block
-__global__ void k_project_dense_nu(int n, double *G, const double *__restrict__ nu) {
-    __shared__ double gnu[1024];
-    __shared__ double nn, nugnu;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double s = 0.0;
-        for (int j = 0; j < n; ++j) s += G[(int64_t)i * n + j] * nu[j];
-        gnu[i] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int i = 0; i < n; ++i) {
-            a += nu[i] * nu[i];
-            b += nu[i] * gnu[i];
-        }
-        nn = a;
-        nugnu = b;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-        int i = t / n, j = t % n;
-        G[t] = G[t] - (gnu[i] * nu[j] + nu[i] * gnu[j]) / nn + nu[i] * nu[j] * nugnu / (nn * nn);
-    }
 }
 
 static void coarse_inverse(Arena &ar, Chain &C, cudaStream_t s) {
@@ -1705,7 +1615,7 @@ static void coarse_inverse(Arena &ar, Chain &C, cudaStream_t s) {
     double sigma = 0.0;
     if (C.singular) {
         Scratch<double> tr(1);
-        k_trace<<<1, 32, 0, s>>>(n, L.A.rp, L.A.ci, L.A.v, tr);
+        k_trace<<<1, 1024, 0, s>>>(n, L.diag, tr);
         VEMG_CHECK_LAUNCH();
         double t = 0.0;
         VEMG_CHECK_CUDA(cudaMemcpyAsync(&t, tr.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1721,27 +1631,15 @@ static void coarse_inverse(Arena &ar, Chain &C, cudaStream_t s) {
             sigma = t / ((double)n * (double)n);
         }
     }
-    Scratch<double> D((int64_t)n * n);
+    const int np = dense_padded(n);
+    Scratch<double> D((int64_t)np * np);
     Scratch<int> err(1);
     VEMG_CHECK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    k_dense_fill<<<n, 128, 0, s>>>(n, L.A.rp, L.A.ci, L.A.v, D);
-    VEMG_CHECK_LAUNCH();
-    if (C.nu) {
-        k_dense_rank1<<<grid_for((int64_t)n * n, 256), 256, 0, s>>>(n, D, sigma, C.nu);
-        VEMG_CHECK_LAUNCH();
-    }
-    k_dense_cholesky<<<1, 1024, 0, s>>>(n, D, C.nu ? 0.0 : sigma, err);
+    k_dense_fill<<<np, 128, 0, s>>>(n, np, L.A.rp, L.A.ci, L.A.v, sigma, C.nu, D);
     VEMG_CHECK_LAUNCH();
     C.G = ar.alloc<double>((int64_t)n * n);
-    k_dense_inverse_cols<<<grid_for(n, 64), 64, 0, s>>>(n, D, C.G);
-    VEMG_CHECK_LAUNCH();
-    if (C.singular && C.nu) {
-        k_project_dense_nu<<<1, 1024, 0, s>>>(n, C.G, C.nu);
-        VEMG_CHECK_LAUNCH();
-    } else if (C.singular) {
-        k_project_dense<<<1, 1024, 0, s>>>(n, C.G);
-        VEMG_CHECK_LAUNCH();
-    }
+    dense_spd_inverse(n, D, C.G, err, s);
+    if (C.singular) dense_project(n, C.G, C.nu, s);
     if (int e = read_flag(err, s)) throw Error{e};
 }
 

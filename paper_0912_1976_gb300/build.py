@@ -35,7 +35,7 @@ def _nvcc():
 
 
 def _sources():
-    return [os.path.join(CSRC, u) for u in UNITS] + [os.path.join(CSRC, "internal.cuh"),
+    return [os.path.join(CSRC, u) for u in UNITS] + [os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "sell.cuh"),
                                                     os.path.join(ROOT, "include", "vemg.h")]
 
 

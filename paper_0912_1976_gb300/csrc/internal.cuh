@@ -44,6 +44,32 @@ inline int grid_for(int64_t n, int block) { return (int)((n + block - 1) / block
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// FP32 <-> FP64 in integer arithmetic: the conversion instructions run on the FP64 pipe, which takes a
+// warp 64 cycles for any instruction on this GPU (two lanes per cycle and SM), as long as a
+// multiply-add; these take a few integer instructions at full rate. The same bits as the conversions:
+// every case that is not an ordinary normal number (zeros, subnormals, infinities, NaN, results at the
+// ends of the FP32 range) takes the instruction.
+__device__ __forceinline__ double cvt_f64(float f) {
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ float cvt_f32(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), m = hi & 0x7fffffffu;
+    if (m - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)d;   // outside 2^-126 <= |d| < 2^127
+    unsigned v = ((m - 0x38000000u) << 3) | (lo >> 29);
+    v += (lo & 0x1fffffffu) + (v & 1u) > 0x10000000u;                    // to nearest, ties to even
+    return __uint_as_float((hi & 0x80000000u) | v);
+}
+template <class T>
+__device__ __forceinline__ T cvt(double a) { return sizeof(T) == sizeof(float) ? (T)cvt_f32(a) : (T)a; }
+template <class T>
+__device__ __forceinline__ T cvt(float a) { return sizeof(T) == sizeof(float) ? (T)a : (T)cvt_f64(a); }
+
+// a + b on the FP64 pipe as a multiply-add with a one that the compiler cannot see (the same bits): an
+// addition issues at 1.68 lanes per cycle and SM, a multiply-add at 2.0 (measured)
+__device__ __forceinline__ double dadd(double a, double b, double one) { return __fma_rn(b, one, a); }
+
 // ------------------------------------------------------------------------------------------
 // programmatic dependent launch: a kernel launched with pdl_launch may start while the kernel
 // before it on the stream finishes; pdl_begin() at its top waits until that kernel has completed
@@ -76,7 +102,8 @@ inline void pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStre
 void *dev_alloc_raw(size_t bytes);
 void dev_free_raw(void *p);
 
-// An owner of device allocations; freed together.
+// An owner of device allocations; freed together. Blocks start on 256-byte boundaries whatever the
+// allocator returns (the kernels load vectors 16 bytes at a time).
 struct Arena {
     std::vector<void *> ptrs;
     size_t bytes = 0;
@@ -85,9 +112,14 @@ struct Arena {
         size_t b = (size_t)(count > 0 ? count : 1) * sizeof(T);
         b = (b + 255) & ~(size_t)255;
         void *p = dev_alloc_raw(b);
+        if ((uintptr_t)p & 255) {
+            dev_free_raw(p);
+            b += 256;
+            p = dev_alloc_raw(b);
+        }
         ptrs.push_back(p);
         bytes += b;
-        return (T *)p;
+        return (T *)(((uintptr_t)p + 255) & ~(uintptr_t)255);
     }
     void release() {
         for (void *p : ptrs) dev_free_raw(p);
@@ -179,22 +211,28 @@ struct Probe {
     int64_t launches = 0;
 };
 
-// Sliced ELL with slices of 32 rows (one warp, one thread per row). Entry k of the row in lane
-// l of slice s is at off[s] + 32 k + l; unused entries hold value 0 and a column inside the
-// matrix. Slices never straddle the row groups given at construction (colours).
+// Sliced ELL (one warp per slice). Two kinds:
+// the outer operators (A, E~ in FP64): slices of 32 rows, one thread per row, entry k of the row in lane
+// l of slice s at off[s] + 32 k + l; unused entries hold value 0 and a column inside the matrix;
+// the chains' operators (rl set): 32 >> lsh rows per slice, 1 << lsh lanes per row (sell.cuh).
+// Slices never straddle the row groups given at construction (colours).
 struct Sell {
     int n = 0, m = 0;         // rows, columns
     int nslices = 0;
     int *row0 = nullptr;      // first row of each slice
     int *nrow = nullptr;      // rows in each slice (<= 32)
     int *off = nullptr;       // element offset of each slice
-    int *width = nullptr;     // stored entries per row of each slice
+    int *width = nullptr;     // stored entries per lane of each slice
     int *col = nullptr;
     void *v = nullptr;        // double or float values
     bool fp32 = false;
     int64_t nnz = 0;          // stored (unpadded) entries
     int64_t padded = 0;       // stored entries including padding
     void *vh = nullptr;       // BF16 copy of the FP32 values (BF16 precision), else null
+    int lsh = 0;              // log2 of the lanes per row
+    int4 *meta = nullptr;     // row0, nrow, off of each slice
+    unsigned *rl = nullptr;   // per row: lower entries | entries << 16, or the two words (rl_wide)
+    int rl_wide = 0;
 };
 
 // One multigrid level in solve order: rows grouped by colour (colour-major, ascending natural
@@ -202,10 +240,11 @@ struct Sell {
 struct SLevel {
     int n = 0, ncolours = 0;
     Sell A;                        // off-diagonal entries (SOR sweeps, residual)
-    void *diag = nullptr, *dinv = nullptr;
+    void *dinv = nullptr;
     std::vector<int> cslice;       // host: slice range of each colour (ncolours + 1)
     std::vector<int> crow;         // host: row range of each colour (ncolours + 1)
     std::vector<int64_t> cnnz;     // host: stored off-diagonal entries of each colour
+    std::vector<int64_t> clow;     // host: those of earlier colours (what a sweep from zero reads)
     Sell P, PT;                    // prolongation (fine rows) and restriction (coarse rows)
     void *x = nullptr, *b = nullptr, *r = nullptr;
 };

@@ -25,9 +25,9 @@
 // Coherence: data a phase writes is read by other CTAs in later phases of the same kernel, so
 // every such read goes to L2 (ld.global.cg) and every such write is an st.global.cg; operators
 // and the outer residual, which the kernel never writes, go through the read-only path.
-#include <map>
+#include <algorithm>
 
-#include "internal.cuh"
+#include "sell.cuh"
 
 namespace vemg {
 
@@ -40,16 +40,15 @@ enum : int { PH_SOR = 0, PH_RES, PH_SPMV, PH_SPMV_ADD, PH_RESTRICT_F64, PH_DENSE
 struct PPhase {
     int op;
     int s0, s1;          // slice range (sliced-ELL phases)
-    int lim;             // SOR from zero: first row of the colour (columns >= lim are zero); else -1
+    int range;           // the part of each row that the phase takes (sell.cuh)
     int b_outer;         // the right-hand side is the FP64 outer residual r + b_off
     int b_off;
     int n;               // PH_DENSE: rows of the dense inverse
     int level;           // multigrid level of the phase (for profiles)
-    const int4 *meta;    // per slice: first row, rows, element offset, width
-    const int *col;
+    SellView S;
     const void *v;       // values (XT; double for PH_RESTRICT_F64; the dense inverse for PH_DENSE)
-    const void *d;       // PH_SOR: inverse diagonal; PH_RES: diagonal
-    const void *b;       // right-hand side (PH_SOR, PH_RES, PH_DENSE) or SpMV input
+    const void *d;       // PH_SOR: inverse diagonal
+    const void *b;       // right-hand side (PH_SOR, PH_DENSE) or SpMV input
     void *x;             // PH_SOR: solution; PH_RES: iterate; SpMV / dense: output
     void *r;             // PH_RES: residual output
 };
@@ -117,18 +116,16 @@ __device__ bool bar_wait(const unsigned long long *ctr, unsigned long long targe
     return s_ok != 0;
 }
 
-// the operator data of one row's first kPU entries, loaded ahead of the phase
+// the operator data of a lane's first kPU entries, loaded ahead of the phase
 template <class XT>
 struct Pre {
     int s;          // slice, or -1
-    int i, o, w;    // row, element offset of the row, stored entries
-    int c[kPU];
-    XT a[kPU];
-    XT d;           // inverse diagonal (SOR) or diagonal (residual)
+    LaneRow a;
+    RowHead<XT, kPU> h;
+    XT d;           // inverse diagonal (SOR)
     double bo;      // outer right-hand side entry, when the phase reads the outer residual
 };
 
-template <class XT>
 __device__ __forceinline__ bool sell_op(int op) {
     return op == PH_SOR || op == PH_RES || op == PH_SPMV || op == PH_SPMV_ADD;
 }
@@ -137,43 +134,14 @@ template <class XT>
 __device__ __forceinline__ void prefetch(const PPhase &p, const double *__restrict__ r, int gw, int lane,
                                          Pre<XT> &q) {
     // every field is written on every path, so nothing of the previous phase stays live
-    int s = p.s0 + gw;
-    int4 m = make_int4(0, 0, 0, 0);
-    bool on = sell_op<XT>(p.op) && s < p.s1;
-    if (on) m = __ldg(p.meta + s);
-    on = on && lane < m.y;
+    const int s = p.s0 + gw;
+    const bool on = sell_op(p.op) && s < p.s1;
     q.s = on ? s : -1;
-    q.i = m.x + lane;
-    q.o = m.z + lane;
-    q.w = on ? m.w : 0;
-    const XT *v = (const XT *)p.v;
-#pragma unroll
-    for (int u = 0; u < kPU; ++u) {
-        q.c[u] = u < q.w ? __ldg(p.col + q.o + 32 * u) : 0;
-        q.a[u] = u < q.w ? __ldg(v + q.o + 32 * u) : (XT)0;
-    }
-    q.d = on && (p.op == PH_SOR || p.op == PH_RES) ? __ldg((const XT *)p.d + q.i) : (XT)0;
-    q.bo = on && p.b_outer && (p.op == PH_SOR || p.op == PH_RES) ? __ldg(r + p.b_off + q.i) : 0.0;
-}
-
-// entries [k0, w) of a row dotted with x (x through L2), continuing the sum acc
-template <class VT, class XT, class AT, int B>
-__device__ __forceinline__ AT prow_from(AT acc, const int *__restrict__ col, const VT *__restrict__ v, int o, int w,
-                                        const XT *x, int lim, int k0) {
-    for (; k0 < w; k0 += B) {
-        int c[B];
-        VT a[B];
-#pragma unroll
-        for (int u = 0; u < B; ++u) {
-            int k = k0 + u;
-            c[u] = k < w ? __ldg(col + o + 32 * k) : 0;
-            a[u] = k < w ? __ldg(v + o + 32 * k) : (VT)0;
-        }
-#pragma unroll
-        for (int u = 0; u < B; ++u)
-            if (k0 + u < w && (lim < 0 || c[u] < lim)) acc = fmadd((AT)a[u], (AT)ldcg(x + c[u]), acc);
-    }
-    return acc;
+    if (on) q.a = lane_row(p.S, s, lane, p.range);
+    else q.a = LaneRow{0, 0, 0, 0, false, false};
+    load_head(q.h, p.S.col, (const XT *)p.v, q.a, q.a.t0);
+    q.d = q.a.first && p.op == PH_SOR ? __ldg((const XT *)p.d + q.a.r) : (XT)0;
+    q.bo = q.a.first && p.b_outer && p.op == PH_SOR ? __ldg(r + p.b_off + q.a.r) : 0.0;
 }
 
 template <class XT>
@@ -181,87 +149,50 @@ __device__ __forceinline__ XT rhs(const PPhase &p, const double *__restrict__ r,
     return p.b_outer ? (XT)__ldg(r + p.b_off + i) : ldcg((const XT *)p.b + i);
 }
 
-// one row of a sliced-ELL phase; `first` holds its first kPU entries when pre != nullptr
-template <class XT>
-__device__ __forceinline__ void sell_row_op(const PPhase &p, const double *__restrict__ r, int i, int o, int w,
-                                            const Pre<XT> *pre) {
-    const XT *v = (const XT *)p.v;
+// one slice of a sliced-ELL phase, the lane's first entries loaded; all lanes of the warp call it
+template <class XT, int U>
+__device__ __forceinline__ void slice_op(const PPhase &p, const double *__restrict__ r, const LaneRow &a,
+                                         RowHead<XT, U> &h, XT d, XT b) {
     const XT *x = (const XT *)(p.op == PH_SPMV || p.op == PH_SPMV_ADD ? p.b : p.x);
-    const int lim = p.op == PH_SOR ? p.lim : -1;
-    XT acc = (XT)0;
-    if (!(p.op == PH_SOR && lim == 0)) {
-        if (pre) {
-#pragma unroll
-            for (int u = 0; u < kPU; ++u)
-                if (u < w && (lim < 0 || pre->c[u] < lim)) acc = fmadd(pre->a[u], ldcg(x + pre->c[u]), acc);
-            if (w > kPU) acc = prow_from<XT, XT, XT, 8>(acc, p.col, v, o, w, x, lim, kPU);
-        } else {
-            acc = prow_from<XT, XT, XT, kPU>(acc, p.col, v, o, w, x, lim, 0);
-        }
-    }
+    const XT acc = row_sum(lane_sum<true, XT>(h, p.S.col, (const XT *)p.v, a, x), p.S.lsh);
+    if (!a.first) return;
     switch (p.op) {
-        case PH_SOR: {
-            XT d = pre ? pre->d : __ldg((const XT *)p.d + i);
-            XT b = pre && p.b_outer ? (XT)pre->bo : rhs<XT>(p, r, i);
-            stcg((XT *)p.x + i, (b - acc) * d);
-            break;
-        }
-        case PH_RES: {
-            XT d = pre ? pre->d : __ldg((const XT *)p.d + i);
-            XT b = pre && p.b_outer ? (XT)pre->bo : rhs<XT>(p, r, i);
-            XT t = fmadd(d, ldcg((const XT *)p.x + i), acc);
-            stcg((XT *)p.r + i, b - t);
-            break;
-        }
-        case PH_SPMV: stcg((XT *)p.x + i, acc); break;
-        case PH_SPMV_ADD: stcg((XT *)p.x + i, ldcg((const XT *)p.x + i) + acc); break;
+        case PH_SOR: stcg((XT *)p.x + a.r, (b - acc) * d); break;
+        case PH_RES: stcg((XT *)p.r + a.r, (XT)0 - acc); break;
+        case PH_SPMV: stcg((XT *)p.x + a.r, acc); break;
+        case PH_SPMV_ADD: stcg((XT *)p.x + a.r, ldcg((const XT *)p.x + a.r) + acc); break;
         default: break;
     }
 }
 
-// PRE: the warp's first slice of the phase was prefetched into `pre` (the grid kernel); the
-// single-CTA tail kernel runs without prefetch
+// PRE: the warp's first slice of the phase was prefetched into `pre`
 template <class XT, bool PRE>
-__device__ void run_phase(const PPhase &p, const double *__restrict__ r, int gw, int nw, int lane,
-                          const Pre<XT> &pre) {
-    if (sell_op<XT>(p.op)) {
+__device__ void run_phase(const PPhase &p, const double *__restrict__ r, int gw, int nw, int lane, Pre<XT> &pre) {
+    if (sell_op(p.op)) {
         int s = p.s0 + gw;
         if (PRE && s < p.s1 && pre.s == s) {
-            sell_row_op<XT>(p, r, pre.i, pre.o, pre.w, &pre);
-            s += nw;
-        } else if (PRE && s < p.s1) {
-            // no prefetched row for this lane (a short slice): nothing to do in this slice
+            XT b = (XT)0;
+            if (p.op == PH_SOR && pre.a.first) b = p.b_outer ? (XT)pre.bo : ldcg((const XT *)p.b + pre.a.r);
+            slice_op<XT>(p, r, pre.a, pre.h, pre.d, b);
             s += nw;
         }
         for (; s < p.s1; s += nw) {
-            int4 m = __ldg(p.meta + s);
-            if (lane >= m.y) continue;
-            sell_row_op<XT>(p, r, m.x + lane, m.z + lane, m.w, nullptr);
+            const LaneRow a = lane_row(p.S, s, lane, p.range);
+            RowHead<XT, kPU> h;
+            load_head(h, p.S.col, (const XT *)p.v, a, a.t0);
+            const bool sor = p.op == PH_SOR && a.first;
+            slice_op<XT>(p, r, a, h, sor ? __ldg((const XT *)p.d + a.r) : (XT)0, sor ? rhs<XT>(p, r, a.r) : (XT)0);
         }
         return;
     }
     if (p.op == PH_RESTRICT_F64) {   // E~^T r of the outer FP64 residual, accumulated in FP64
         const double *v = (const double *)p.v;
-        XT *y = (XT *)p.x;
         for (int s = p.s0 + gw; s < p.s1; s += nw) {
-            int4 m = __ldg(p.meta + s);
-            if (lane >= m.y) continue;
-            double acc = 0.0;
-            int o = m.z + lane, w = m.w;
-            for (int k0 = 0; k0 < w; k0 += kPU) {
-                int c[kPU];
-                double a[kPU];
-#pragma unroll
-                for (int u = 0; u < kPU; ++u) {
-                    int k = k0 + u;
-                    c[u] = k < w ? __ldg(p.col + o + 32 * k) : 0;
-                    a[u] = k < w ? __ldg(v + o + 32 * k) : 0.0;
-                }
-#pragma unroll
-                for (int u = 0; u < kPU; ++u)
-                    if (k0 + u < w) acc = fmadd(a[u], __ldg(r + c[u]), acc);
-            }
-            stcg(y + m.x + lane, (XT)acc);
+            const LaneRow a = lane_row(p.S, s, lane, ROW_ALL);
+            RowHead<double, 8> h;
+            load_head(h, p.S.col, v, a, 0);
+            const double acc = row_sum(lane_sum<false, double>(h, p.S.col, v, a, r), p.S.lsh);
+            if (a.first) stcg((XT *)p.x + a.r, (XT)acc);
         }
         return;
     }
@@ -446,43 +377,20 @@ int barrier_selftest(int claimed, int launched, cudaStream_t s) {
 // ------------------------------------------------------------------------------------------
 // host side: the program
 
-__global__ void k_pack_meta(int ns, const int *__restrict__ row0, const int *__restrict__ nrow,
-                            const int *__restrict__ off, const int *__restrict__ width, int4 *meta) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < ns) meta[s] = make_int4(row0[s], nrow[s], off[s], width[s]);
-}
-
 namespace {
 
 struct Builder {
-    Arena &ar;
-    cudaStream_t st;
     std::vector<PPhase> ph;
-    std::map<const int *, const int4 *> metas;
     double bytes = 0.0;
     size_t xs = 8;
 
-    Builder(Arena &a, cudaStream_t s) : ar(a), st(s) {}
-
-    const int4 *meta_of(const Sell &S) {
-        auto it = metas.find(S.row0);
-        if (it != metas.end()) return it->second;
-        int4 *m = ar.alloc<int4>(std::max(S.nslices, 1));
-        if (S.nslices > 0) {
-            k_pack_meta<<<grid_for(S.nslices, 256), 256, 0, st>>>(S.nslices, S.row0, S.nrow, S.off, S.width, m);
-            VEMG_CHECK_LAUNCH();
-        }
-        metas[S.row0] = m;
-        return m;
-    }
     PPhase sell_phase(int op, const Sell &S, int s0, int s1) {
         PPhase p{};
         p.op = op;
         p.s0 = s0;
         p.s1 = s1;
-        p.lim = -1;
-        p.meta = meta_of(S);
-        p.col = S.col;
+        p.range = ROW_ALL;
+        p.S = view(S);
         p.v = S.v;
         return p;
     }
@@ -502,14 +410,14 @@ struct Builder {
             int s0 = L.cslice[c], s1 = L.cslice[c + 1];
             if (s1 == s0) continue;
             PPhase p = sell_phase(PH_SOR, L.A, s0, s1);
-            p.lim = from_zero ? L.crow[c] : -1;
+            p.range = from_zero ? ROW_LOWER : ROW_ALL;
             p.d = L.dinv;
             set_b(p, b, outer_off);
             p.x = x;
             p.level = lev;
             ph.push_back(p);
             int rows = L.crow[c + 1] - L.crow[c];
-            bytes += (p.lim == 0 ? 0.0 : (double)L.cnnz[c] * (xs + 4.0)) + (double)rows * 3.0 * xs +
+            bytes += (double)(from_zero ? L.clow[c] : L.cnnz[c]) * (xs + 4.0) + (double)rows * 3.0 * xs +
                      (double)xs * L.n / L.ncolours;
         }
     }
@@ -544,13 +452,12 @@ struct Builder {
         }
         sweep(L, b, outer_off, x, true, true);
         PPhase p = sell_phase(PH_RES, L.A, 0, L.A.nslices);
-        p.d = L.diag;
-        set_b(p, b, outer_off);
+        p.range = ROW_UPPER;
         p.x = x;
         p.r = L.r;
         p.level = l;
         ph.push_back(p);
-        bytes += (double)L.A.nnz * (xs + 4.0) + (double)L.n * 5.0 * xs;
+        bytes += 0.5 * (double)L.A.nnz * (xs + 4.0) + (double)L.n * 2.0 * xs;
         const SLevel &N = C.lv[l + 1];
         spmv(L.PT, L.r, N.b, false);
         vcycle(C, l + 1, N.b, -1, N.x);
@@ -574,7 +481,7 @@ void build_persist(vemg_hierarchy *h, cudaStream_t s) {
     const bool fp32 = h->precision != VEMG_PREC_FP64;
     const bool coarse = h->opts.cycle == VEMG_CYCLE_HYBRID;
     bool two = !single_chain(h);
-    Builder B(h->arena, s);
+    Builder B;
     B.xs = fp32 ? 4 : 8;
     std::vector<int2> ranges;   // phase ranges per group
     if (coarse) {
@@ -697,7 +604,7 @@ static void build_tail(Arena &ar, SChain &C, bool fp32, int tail_rows, int ncta,
             break;
         }
     if (l0 < 0) return;
-    Builder B(ar, s);
+    Builder B;
     B.xs = fp32 ? 4 : 8;
     for (;;) {   // the single-CTA tail starts deeper while its phases do not fit in shared memory
         B.ph.clear();

@@ -10,7 +10,7 @@
 // the outer loop is flexible CG (Notay's FCG(1)), since the preconditioner is then not exactly
 // symmetric (section 5.5 on nested inexact inner solves).
 //
-// Operators are sliced ELL in solve order (layout.cu); one thread per row, 32 rows per warp.
+// Operators are sliced ELL in solve order (layout.cu, sell.cuh).
 // Reductions are deterministic (fixed grid, fixed order). One solve runs as three CUDA graphs:
 // the first iteration, a WHILE conditional node whose body is one further iteration (the
 // condition is set on the device from the residual norm), and the exit work.
@@ -20,16 +20,14 @@
 
 #include <type_traits>
 
-#include <cuda_bf16.h>
-
-#include "internal.cuh"
+#include "sell.cuh"
 
 namespace vemg {
 
 static constexpr int kRedBlocks = 608;  // 4 x 152 SMs
 static constexpr int kRedThreads = 256;
 static constexpr int kSellBlock = 128;  // 4 slices per block
-static constexpr int kRows = 1;         // rows per thread and loop trip in the streaming kernels (1: k_combine fits 4 blocks per SM)
+static constexpr int kVecBlocks = 304;  // 2 x 152 SMs: the streaming kernels' most
 static constexpr int kEmax = 4;         // E~ rows with at most this many entries take the fast path
 
 // ------------------------------------------------------------------------------------------
@@ -107,162 +105,113 @@ static double sell_bytes(int64_t nnz, double vb, int64_t rows, double per_row) {
 // ------------------------------------------------------------------------------------------
 // sliced-ELL kernels
 
-// entries of a sliced-ELL row loaded per chunk (before their gathers)
+// entries of an outer operator's row loaded per chunk (before their gathers)
 static constexpr int kU = 16;
 
-// the V-cycle kernels' chunk: 8 entries with FP64 values (16 FP64 values and their columns held
-// 80 registers and measured 11% slower per FP64-cycle solve), 16 with FP32 or BF16 values
-template <class VT>
-__host__ __device__ constexpr int cycle_chunk() {
-    return sizeof(VT) == sizeof(double) ? 8 : kU;
-}
-
-// BF16 values widen to FP32 before they meet the vector; FP32 and FP64 values pass through
-__device__ __forceinline__ float float_or_self(__nv_bfloat16 a) { return __bfloat162float(a); }
-__device__ __forceinline__ float float_or_self(float a) { return a; }
-__device__ __forceinline__ double float_or_self(double a) { return a; }
-
-// The first U entries of a sliced-ELL row (column indices and values), loaded before the
-// kernel waits for its predecessor: the operators are setup data that no solve kernel writes,
-// so these loads overlap the previous kernel and only the gathers of x remain after the wait.
-template <class VT, int U = kU>
-struct RowHead {
+// Dot product of one row of an outer operator with x, U entries at a time (column indices and values
+// first, then the gathers), so that a row costs two dependent memory round trips per U entries instead
+// of two per entry. The first U stand outside the loop: most rows have no more, and with them inside
+// it k_spmv_pq took 164 instead of 97 us on the 256 x 256 x 32 mesh. The products are added in the
+// row's stored order whatever U is.
+template <class VT, int U>
+struct Chunk {
     int c[U];
     VT a[U];
-};
-
-template <class VT, int U>
-__device__ __forceinline__ void load_head(RowHead<VT, U> &h, const int *__restrict__ col, const VT *__restrict__ v,
-                                          int o, int w) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        h.c[u] = u < w ? __ldg(col + o + 32 * u) : 0;
-        h.a[u] = u < w ? __ldg(v + o + 32 * u) : VT{};
-    }
-}
-
-// Dot product of one sliced-ELL row with x: the head's entries, then the rest of the row U
-// entries at a time (column indices and values first, then the gathers), so that a row costs
-// two dependent memory round trips per U entries instead of two per entry. lim >= 0 skips
-// columns >= lim. The products are added in the row's stored order whatever U is.
-template <class VT, class XT, class AT, int U>
-__device__ __forceinline__ AT sell_row(const RowHead<VT, U> &h, const int *__restrict__ col, const VT *__restrict__ v,
-                                       int o, int w, const XT *x, int lim) {
-    AT acc = 0;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if (u < w && (lim < 0 || h.c[u] < lim)) acc = fmadd((AT)(float_or_self(h.a[u])), (AT)x[h.c[u]], acc);
-    for (int k0 = U; k0 < w; k0 += U) {
-        int c[U];
-        VT a[U];
+    __device__ __forceinline__ void load(const int *__restrict__ col, const VT *__restrict__ v, int o, int n) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            int k = k0 + u;
-            c[u] = k < w ? __ldg(col + o + 32 * k) : 0;
-            a[u] = k < w ? __ldg(v + o + 32 * k) : VT{};
+            c[u] = u < n ? __ldg(col + o + 32 * u) : 0;
+            a[u] = u < n ? __ldg(v + o + 32 * u) : VT{};
         }
+    }
+    template <class AT, class XT>
+    __device__ __forceinline__ AT add(AT acc, const XT *x, int n) const {
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (k0 + u < w && (lim < 0 || c[u] < lim)) acc = fmadd((AT)(float_or_self(a[u])), (AT)x[c[u]], acc);
+            if (u < n) acc = fmadd((AT)a[u], (AT)x[c[u]], acc);
+        return acc;
+    }
+};
+
+template <class VT, class XT, class AT, int U = kU>
+__device__ __forceinline__ AT sell_row(const int *__restrict__ col, const VT *__restrict__ v, int o, int w,
+                                       const XT *x) {
+    Chunk<VT, U> h;
+    h.load(col, v, o, w);
+    AT acc = h.add((AT)0, x, w);
+    for (int k0 = U; k0 < w; k0 += U) {
+        Chunk<VT, U> g;
+        g.load(col, v, o + 32 * k0, w - k0);
+        acc = g.add(acc, x, w - k0);
     }
     return acc;
 }
 
-template <class VT, class XT, class AT, int U = kU>
-__device__ __forceinline__ AT sell_row(const int *__restrict__ col, const VT *__restrict__ v, int o, int w,
-                                       const XT *x, int lim) {
-    RowHead<VT, U> h;
-    load_head(h, col, v, o, w);
-    return sell_row<VT, XT, AT, U>(h, col, v, o, w, x, lim);
-}
-
-// y = A x (add: y += A x) over the slices [s0, s1); accumulation in AT. With x0: the restriction
-// into a level whose V-cycle starts with a sweep from x = 0 also does that sweep's first colour
-// (rows below lim0): x0_i = y_i / A_ii, the same product the colour's own launch would form.
-template <class VT, class XT, class YT, class AT>
-__global__ void __launch_bounds__(kSellBlock) k_sell_spmv(int s0, int s1, const int *__restrict__ row0,
-                                                          const int *__restrict__ nrow, const int *__restrict__ off,
-                                                          const int *__restrict__ width, const int *__restrict__ col,
-                                                          const VT *__restrict__ v, const XT *__restrict__ x,
-                                                          YT *__restrict__ y, int add, const YT *__restrict__ dinv0,
-                                                          YT *__restrict__ x0, int lim0) {
-    int s = s0 + (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    int lane = threadIdx.x & 31;
-    const bool active = s < s1 && lane < nrow[s];
-    constexpr int U = cycle_chunk<VT>();
-    RowHead<VT, U> h;
-    int o = 0, w = 0, r = 0;
-    YT d0 = 0;
-    if (active) {
-        o = off[s] + lane;
-        w = width[s];
-        r = row0[s] + lane;
-        if (x0 && r < lim0) d0 = dinv0[r];
-        load_head(h, col, v, o, w);
+// y = A x (add: y += A x) over all slices of a transfer operator; accumulation in AT. With x0: the
+// restriction into a level whose V-cycle starts with a sweep from x = 0 also does that sweep's
+// first colour (rows below lim0): x0_i = y_i / A_ii, the same product the colour's own launch would form.
+template <class VT, class XT, class YT, class AT, int U>
+__global__ void __launch_bounds__(kSellBlock) k_sell_spmv(int nsl, SellView S, const VT *__restrict__ v,
+                                                          const XT *__restrict__ x, YT *__restrict__ y, int add,
+                                                          const YT *__restrict__ dinv0, YT *__restrict__ x0, int lim0) {
+    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= nsl) {
+        pdl_begin();
+        return;
     }
+    const LaneRow a = lane_row(S, s, lane, ROW_ALL);
+    RowHead<VT, U> h;
+    load_head(h, S.col, v, a, 0);
+    const bool fuse = a.first && x0 && a.r < lim0;
+    const YT d0 = fuse ? dinv0[a.r] : (YT)0;
     pdl_begin();
-    if (!active) return;
-    AT acc = sell_row<VT, XT, AT, U>(h, col, v, o, w, x, -1);
-    YT yr = add ? (YT)((AT)y[r] + acc) : (YT)acc;
-    y[r] = yr;
-    if (x0 && r < lim0) x0[r] = yr * d0;
+    const AT y0 = add && a.first ? (AT)y[a.r] : (AT)0;
+    const AT acc = row_sum(lane_sum<false, AT>(h, S.col, v, a, x), S.lsh);
+    if (!a.first) return;
+    const YT yr = (YT)(add ? y0 + acc : acc);
+    y[a.r] = yr;
+    if (fuse) x0[a.r] = yr * d0;
 }
 
 // SOR (omega = 1) on the rows of one colour (slices [s0, s1)):
-// x_i = (b_i - sum_{j != i} A_ij x_j) / A_ii. lim >= 0: sweep from x = 0, entries with column
-// >= lim (colours not yet visited) are zero and skipped; lim == 0 needs no entries at all.
-template <class VT, class XT, class BT>
-__global__ void __launch_bounds__(kSellBlock) k_sell_sor(int s0, int s1, const int *__restrict__ row0,
-                                                         const int *__restrict__ nrow, const int *__restrict__ off,
-                                                         const int *__restrict__ width, const int *__restrict__ col,
-                                                         const VT *__restrict__ v, const XT *__restrict__ dinv,
-                                                         const BT *__restrict__ b, XT *x, int lim) {
-    int s = s0 + (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    int lane = threadIdx.x & 31;
-    const bool active = s < s1 && lane < nrow[s];
-    constexpr int U = cycle_chunk<VT>();
-    RowHead<VT, U> h;
-    int o = 0, w = 0, r = 0;
-    XT di = 0;
-    if (active) {
-        o = off[s] + lane;
-        w = lim == 0 ? 0 : width[s];
-        r = row0[s] + lane;
-        di = dinv[r];
-        load_head(h, col, v, o, w);
+// x_i = (b_i - sum_{j != i} A_ij x_j) / A_ii. ROW_LOWER: in a sweep from x = 0, where the colours not
+// yet visited hold zeros.
+template <class VT, class XT, class BT, int U>
+__global__ void __launch_bounds__(kSellBlock) k_sell_sor(int s0, int s1, SellView S, const VT *__restrict__ v,
+                                                         const XT *__restrict__ dinv, const BT *__restrict__ b, XT *x,
+                                                         int range) {
+    const int s = s0 + (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= s1) {
+        pdl_begin();
+        return;
     }
+    const LaneRow a = lane_row(S, s, lane, range);
+    RowHead<VT, U> h;
+    load_head(h, S.col, v, a, 0);
+    const XT di = a.first ? dinv[a.r] : (XT)0;
     pdl_begin();
-    if (!active) return;
-    XT acc = sell_row<VT, XT, XT, U>(h, col, v, o, w, x, lim);
-    x[r] = ((XT)b[r] - acc) * di;
+    const XT bi = a.first ? cvt<XT>(b[a.r]) : (XT)0;
+    const XT acc = row_sum(lane_sum<false, XT>(h, S.col, v, a, x), S.lsh);
+    if (a.first) x[a.r] = (bi - acc) * di;
 }
 
-// r = b - D x - (A - D) x over all slices
-template <class VT, class XT, class BT>
-__global__ void __launch_bounds__(kSellBlock) k_sell_residual(int nsl, const int *__restrict__ row0,
-                                                              const int *__restrict__ nrow, const int *__restrict__ off,
-                                                              const int *__restrict__ width, const int *__restrict__ col,
-                                                              const VT *__restrict__ v, const XT *__restrict__ diag,
-                                                              const BT *__restrict__ b, const XT *__restrict__ x,
-                                                              XT *__restrict__ r) {
-    int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    int lane = threadIdx.x & 31;
-    const bool active = s < nsl && lane < nrow[s];
-    constexpr int U = cycle_chunk<VT>();
-    RowHead<VT, U> h;
-    int o = 0, w = 0, i = 0;
-    XT dg = 0;
-    if (active) {
-        o = off[s] + lane;
-        w = width[s];
-        i = row0[s] + lane;
-        dg = diag[i];
-        load_head(h, col, v, o, w);
+// The residual after a sweep from x = 0 in ascending colours: row i was solved against the colours
+// before its own, so what is left of b - A x is the part of the later ones, r_i = -sum_{j later} A_ij x_j:
+// half the entries, and neither b nor the diagonal.
+template <class VT, class XT, int U>
+__global__ void __launch_bounds__(kSellBlock) k_sell_residual(int nsl, SellView S, const VT *__restrict__ v,
+                                                              const XT *__restrict__ x, XT *__restrict__ r) {
+    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= nsl) {
+        pdl_begin();
+        return;
     }
+    const LaneRow a = lane_row(S, s, lane, ROW_UPPER);
+    RowHead<VT, U> h;
+    load_head(h, S.col, v, a, a.t0);
     pdl_begin();
-    if (!active) return;
-    XT acc = fmadd(dg, x[i], sell_row<VT, XT, XT, U>(h, col, v, o, w, x, -1));
-    r[i] = (XT)b[i] - acc;
+    const XT acc = row_sum(lane_sum<false, XT>(h, S.col, v, a, x), S.lsh);
+    if (a.first) r[a.r] = (XT)0 - acc;
 }
 
 // x = G b for the dense coarsest inverse (one warp per row; G and the sums in the cycle's
@@ -282,10 +231,36 @@ __global__ void k_dense_mv(int n, const XT *__restrict__ Gm, const BT *__restric
 // ------------------------------------------------------------------------------------------
 // launch wrappers
 
+// Entries a lane holds from before the dependency wait: registers against a second round trip of
+// the longer rows. 4, 8 or 16 by the mean share of a lane, with some room for the longer ones; 16 FP64
+// values and their columns hold 80 registers and measured 11% slower per FP64-cycle solve than 8.
+template <class VT, class F>
+static void by_head(double mean, F &&f) {
+    if (mean <= 3.5) f(std::integral_constant<int, 4>{});
+    else if (mean <= 8.0 || sizeof(VT) == sizeof(double)) f(std::integral_constant<int, 8>{});
+    else f(std::integral_constant<int, (sizeof(VT) == sizeof(double) ? 8 : 16)>{});
+}
+
+// the operator's values as the per-phase kernels read them: BF16 ones where it has them
+template <class VT, class F>
+static void by_value(const Sell &S, F &&f) {
+    if constexpr (sizeof(VT) == sizeof(float)) {
+        if (S.vh) {
+            f((const __nv_bfloat16 *)S.vh);
+            return;
+        }
+    }
+    f((const VT *)S.v);
+}
+
+// mean entries of a lane's share of a row
+static double lane_mean(const Sell &S, double entries, double rows) {
+    return entries / std::max(1.0, rows * (1 << S.lsh));
+}
+
 template <class VT, class XT, class YT, class AT>
 static void sell_spmv(const Sell &S, const XT *x, YT *y, int add, cudaStream_t s, const SLevel *first = nullptr) {
     if (S.nslices == 0) return;
-    int64_t threads = (int64_t)S.nslices * 32;
     // first: the level y feeds, whose from-zero sweep's first colour this launch also does
     const YT *d0 = first ? (const YT *)first->dinv : nullptr;
     YT *x0 = first ? (YT *)first->x : nullptr;
@@ -297,13 +272,13 @@ static void sell_spmv(const Sell &S, const XT *x, YT *y, int add, cudaStream_t s
                   sell_bytes(S.nnz, vb, S.n, (add ? 2.0 : 1.0) * sizeof(YT)) + (double)sizeof(XT) * S.m +
                       2.0 * sizeof(YT) * lim0,
                   s);
-    if (S.vh)   // BF16 values (FP32 vectors)
-        pdl_launch(k_sell_spmv<__nv_bfloat16, XT, YT, AT>, grid_for(threads, kSellBlock), kSellBlock, s, 0,
-                   S.nslices, S.row0, S.nrow, S.off, S.width, S.col, (const __nv_bfloat16 *)S.vh, x, y, add, d0, x0,
-                   lim0);
-    else
-        pdl_launch(k_sell_spmv<VT, XT, YT, AT>, grid_for(threads, kSellBlock), kSellBlock, s, 0, S.nslices,
-                   S.row0, S.nrow, S.off, S.width, S.col, (const VT *)S.v, x, y, add, d0, x0, lim0);
+    by_value<VT>(S, [&](auto *v) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(v)>>;
+        by_head<T>(lane_mean(S, (double)S.nnz, S.n), [&](auto u) {
+            pdl_launch(k_sell_spmv<T, XT, YT, AT, decltype(u)::value>, grid_for((int64_t)S.nslices * 32, kSellBlock),
+                       kSellBlock, s, S.nslices, view(S), v, x, y, add, d0, x0, lim0);
+        });
+    });
     SOLVE_LAUNCHED();
 }
 
@@ -321,36 +296,37 @@ static void sor_sweep(const SLevel &L, const BT *b, XT *x, bool forward, bool fr
         int c = forward ? cc : L.ncolours - 1 - cc;
         int s0 = L.cslice[c], s1 = L.cslice[c + 1];
         if (s1 == s0) continue;
-        int lim = from_zero ? L.crow[c] : -1;
+        const int range = from_zero ? ROW_LOWER : ROW_ALL;
+        const int64_t entries = from_zero ? L.clow[c] : L.cnnz[c];
         int rows = L.crow[c + 1] - L.crow[c];
-        // stored entries of the colour (none when lim == 0), b / dinv / x-write per row, and one
+        // the entries of the colour that the sweep takes, b / dinv / x-write per row, and one
         // read of the level's x shared among the sweep's colours
-        double bytes = sell_bytes(lim == 0 ? 0 : L.cnnz[c], value_bytes<XT>(L.A), rows, 3.0 * sizeof(XT)) +
+        double bytes = sell_bytes(entries, value_bytes<XT>(L.A), rows, 3.0 * sizeof(XT)) +
                        (double)sizeof(XT) * L.n / L.ncolours;
         ProbeScope ps(fine ? PROBE_SOR_FINE : PROBE_SOR, bytes, s);
-        int64_t threads = (int64_t)(s1 - s0) * 32;
-        if (L.A.vh)
-            pdl_launch(k_sell_sor<__nv_bfloat16, XT, BT>, grid_for(threads, kSellBlock), kSellBlock, s, s0, s1,
-                       L.A.row0, L.A.nrow, L.A.off, L.A.width, L.A.col, (const __nv_bfloat16 *)L.A.vh,
-                       (const XT *)L.dinv, b, x, lim);
-        else
-            pdl_launch(k_sell_sor<XT, XT, BT>, grid_for(threads, kSellBlock), kSellBlock, s, s0, s1, L.A.row0,
-                       L.A.nrow, L.A.off, L.A.width, L.A.col, (const XT *)L.A.v, (const XT *)L.dinv, b, x, lim);
+        by_value<XT>(L.A, [&](auto *v) {
+            using T = std::remove_const_t<std::remove_pointer_t<decltype(v)>>;
+            by_head<T>(lane_mean(L.A, (double)entries, rows), [&](auto u) {
+                pdl_launch(k_sell_sor<T, XT, BT, decltype(u)::value>, grid_for((int64_t)(s1 - s0) * 32, kSellBlock),
+                           kSellBlock, s, s0, s1, view(L.A), v, (const XT *)L.dinv, b, x, range);
+            });
+        });
         SOLVE_LAUNCHED();
     }
 }
 
-template <class XT, class BT>
-static void residual(const SLevel &L, const BT *b, const XT *x, XT *r, cudaStream_t s) {
-    ProbeScope ps(PROBE_RESIDUAL, sell_bytes(L.A.nnz, value_bytes<XT>(L.A), L.n, 5.0 * sizeof(XT)), s);
-    int64_t threads = (int64_t)L.A.nslices * 32;
-    if (L.A.vh)
-        pdl_launch(k_sell_residual<__nv_bfloat16, XT, BT>, grid_for(threads, kSellBlock), kSellBlock, s,
-                   L.A.nslices, L.A.row0, L.A.nrow, L.A.off, L.A.width, L.A.col, (const __nv_bfloat16 *)L.A.vh,
-                   (const XT *)L.diag, b, x, r);
-    else
-        pdl_launch(k_sell_residual<XT, XT, BT>, grid_for(threads, kSellBlock), kSellBlock, s, L.A.nslices,
-                   L.A.row0, L.A.nrow, L.A.off, L.A.width, L.A.col, (const XT *)L.A.v, (const XT *)L.diag, b, x, r);
+// r = b - A x where x is a sweep from zero in ascending colours
+template <class XT>
+static void residual(const SLevel &L, const XT *x, XT *r, cudaStream_t s) {
+    const double entries = 0.5 * (double)L.A.nnz;   // of later colours (the pattern is symmetric)
+    ProbeScope ps(PROBE_RESIDUAL, sell_bytes((int64_t)entries, value_bytes<XT>(L.A), L.n, 2.0 * sizeof(XT)), s);
+    by_value<XT>(L.A, [&](auto *v) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(v)>>;
+        by_head<T>(lane_mean(L.A, entries, L.n), [&](auto u) {
+            pdl_launch(k_sell_residual<T, XT, decltype(u)::value>, grid_for((int64_t)L.A.nslices * 32, kSellBlock),
+                       kSellBlock, s, L.A.nslices, view(L.A), v, x, r);
+        });
+    });
     SOLVE_LAUNCHED();
 }
 
@@ -390,7 +366,7 @@ static void vcycle_level(const SChain &C, int l, const BT *b, XT *x, cudaStream_
         return;
     }
     sor_sweep<XT, BT>(L, b, x, true, true, fine, s, first_done);
-    residual<XT, BT>(L, b, x, (XT *)L.r, s);
+    residual<XT>(L, (const XT *)x, (XT *)L.r, s);
     const SLevel &N = C.lv[l + 1];
     const bool fuse = fused_first(C, l + 1);
     sell_spmv<XT, XT, XT, XT>(L.PT, (const XT *)L.r, (XT *)N.b, 0, s, fuse ? &N : nullptr);
@@ -406,7 +382,7 @@ template <class XT, class BT>
 static void vcycle_down(const SChain &C, const BT *b, XT *x, cudaStream_t s) {
     const SLevel &L = C.lv[0];
     sor_sweep<XT, BT>(L, b, x, true, true, C.is_bar, s);
-    residual<XT, BT>(L, b, x, (XT *)L.r, s);
+    residual<XT>(L, (const XT *)x, (XT *)L.r, s);
     sell_spmv<XT, XT, XT, XT>(L.PT, (const XT *)L.r, (XT *)C.lv[1].b, 0, s);
 }
 
@@ -419,7 +395,14 @@ static void vcycle_up(const SChain &C, const BT *b, XT *x, cudaStream_t s) {
 
 // ------------------------------------------------------------------------------------------
 // deterministic block reductions: every block writes its partial sums, the last block to finish
-// adds them in block order (fixed grid, fixed order: the same bits on every run)
+// adds them in block order (a grid fixed by n, a fixed order: the same bits on every run).
+//
+// Every FP64 instruction holds one of an SM's four schedulers for 64 cycles, so a reduction costs by
+// the instructions of its warps: one warp per sum adds the block's values up from shared memory, eight
+// a lane, instead of every warp its own 32 (12 instructions a sum and block, not 40). For the same
+// reason the grid grows with n only up to two blocks per SM (one row a thread until there), and a
+// small problem takes few blocks: 2,601 rows with 608 blocks spent 40 of an iteration's 81 us in
+// the reductions of three kernels.
 
 enum {
     S_RZ = 0, S_PQ, S_ALPHA, S_BETA, S_MU, S_BN, S_RN, S_FLAG, S_TOL, S_MAXIT, S_ITERS, S_CONT, S_ZERO, S_TRUE,
@@ -429,46 +412,43 @@ enum { C_SPMV = 0, C_XR, C_Z, C_SUMB, C_PREP, C_SUMX, C_TRUE, C_COUNT };
 
 int solve_scalar_iters() { return S_ITERS; }
 
+static int vec_blocks(int64_t n) { return (int)std::min<int64_t>(kVecBlocks, std::max<int64_t>(1, (n + kRedThreads - 1) / kRedThreads)); }
+
 template <int NS>
 __device__ bool finish_block(double (&acc)[NS], double *part, unsigned *counter, double (&tot)[NS]) {
-    __shared__ double sh[NS][kRedThreads / 32];
+    static_assert(NS <= kRedThreads / 32, "a warp per sum");
+    __shared__ double sh[NS][kRedThreads];
     __shared__ bool last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = gridDim.x;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        double v = acc[s];
+    for (int s = 0; s < NS; ++s) sh[s][threadIdx.x] = acc[s];
+    __syncthreads();
+    if (warp < NS) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < kRedThreads / 32; ++k) v += sh[warp][32 * k + lane];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[s][warp] = v;
+        if (lane == 0) {
+            part[warp * kRedBlocks + blockIdx.x] = v;
+            __threadfence();
+        }
     }
     __syncthreads();
-    if (threadIdx.x < NS) {
-        double v = 0.0;
-        for (int w = 0; w < kRedThreads / 32; ++w) v += sh[threadIdx.x][w];
-        part[threadIdx.x * kRedBlocks + blockIdx.x] = v;
-        __threadfence();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == (unsigned)(kRedBlocks - 1);
+    if (threadIdx.x == 0) last = nb == 1 || atomicAdd(counter, 1u) == (unsigned)(nb - 1);
     __syncthreads();
     if (!last) return false;
     __threadfence();
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
+    if (warp < NS) {
         double v = 0.0;
-        for (int k = threadIdx.x; k < kRedBlocks; k += kRedThreads) v += __ldcg(part + s * kRedBlocks + k);
+        for (int k = lane; k < nb; k += 32) v += __ldcg(part + warp * kRedBlocks + k);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        __syncthreads();
-        if (lane == 0) sh[s][warp] = v;
+        if (lane == 0) sh[warp][0] = v;
     }
     __syncthreads();
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        double v = 0.0;
-        for (int w = 0; w < kRedThreads / 32; ++w) v += sh[s][w];
-        tot[s] = v;
-    }
+    for (int s = 0; s < NS; ++s) tot[s] = sh[s][0];
     if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
@@ -483,6 +463,11 @@ static SellArgs sargs(const Sell &S) {
     return SellArgs{S.nslices, S.row0, S.nrow, S.off, S.width, S.col, (const double *)S.v};
 }
 
+// the grid of a pass over an outer operator: a warp per slice until the chip is full
+static int row_blocks(const Sell &S) {
+    return std::min(kRedBlocks, std::max(1, grid_for((int64_t)S.nslices * 32, kRedThreads)));
+}
+
 // q = A p over all slices and (p, q); the last block sets alpha = rz / pq. At most 64 registers:
 // the whole grid (kRedBlocks = 4 per SM) is resident at once.
 __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152) k_spmv_pq(SellArgs A, const double *__restrict__ p,
@@ -491,12 +476,12 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152) k_spmv_pq(SellA
     pdl_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double acc[1] = {0.0};
-    for (int s = blockIdx.x * (kRedThreads / 32) + warp; s < A.nsl; s += kRedBlocks * (kRedThreads / 32)) {
+    for (int s = blockIdx.x * (kRedThreads / 32) + warp; s < A.nsl; s += gridDim.x * (kRedThreads / 32)) {
         if (lane < A.nrow[s]) {
             int r = A.row0[s] + lane;
-            double qv = sell_row<double, double, double>(A.col, A.v, A.off[s] + lane, A.width[s], p, -1);
+            double qv = sell_row<double, double, double>(A.col, A.v, A.off[s] + lane, A.width[s], p);
             q[r] = qv;
-            acc[0] += p[r] * qv;
+            acc[0] = fma(p[r], qv, acc[0]);
         }
     }
     double tot[1];
@@ -515,36 +500,42 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152) k_spmv_pq(SellA
 
 // x += alpha p, r -= alpha q; the last block sets ||r||, the iteration count and the continuation
 // test (and, inside the solve graph, the WHILE condition)
-__global__ void __launch_bounds__(kRedThreads) k_update_xr(int n, const double *__restrict__ p,
-                                                           const double *__restrict__ q, double *__restrict__ x,
-                                                           double *__restrict__ r, double *sc, double *part,
-                                                           unsigned *ctr, cudaGraphConditionalHandle handle,
-                                                           int use_cond) {
+// Bound by memory (48 bytes a row; vectors are 256-byte aligned, two rows a load, four a trip).
+__global__ void __launch_bounds__(kRedThreads, 2) k_update_xr(int n, const double *__restrict__ p,
+                                                              const double *__restrict__ q, double *__restrict__ x,
+                                                              double *__restrict__ r, double *sc, double *part,
+                                                              unsigned *ctr, cudaGraphConditionalHandle handle,
+                                                              int use_cond) {
     pdl_begin();
-    double a = sc[S_ALPHA];
+    const double a = sc[S_ALPHA];
     double acc[1] = {0.0};
-    constexpr int stride = kRedBlocks * kRedThreads;
-    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += kRows * stride) {
-        double pv[kRows], qv[kRows], xv[kRows], rv[kRows];
+    const int stride = gridDim.x * kRedThreads, n2 = n >> 1;
+    const double2 *p2 = (const double2 *)p, *q2 = (const double2 *)q;
+    double2 *x2 = (double2 *)x, *r2 = (double2 *)r;
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n2; i0 += 2 * stride) {
+        double2 pv[2], qv[2], xv[2], rv[2];
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            int i = i0 + u * stride;
-            bool ok = i < n;
-            pv[u] = ok ? p[i] : 0.0;
-            qv[u] = ok ? q[i] : 0.0;
-            xv[u] = ok ? x[i] : 0.0;
-            rv[u] = ok ? r[i] : 0.0;
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * stride;
+            if (i < n2) { pv[u] = p2[i]; qv[u] = q2[i]; xv[u] = x2[i]; rv[u] = r2[i]; }
         }
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            int i = i0 + u * stride;
-            if (i < n) {
-                x[i] = xv[u] + a * pv[u];
-                double ri = rv[u] - a * qv[u];
-                r[i] = ri;
-                acc[0] += ri * ri;
-            }
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= n2) continue;
+            x2[i] = make_double2(fma(a, pv[u].x, xv[u].x), fma(a, pv[u].y, xv[u].y));
+            const double2 ri = make_double2(fma(-a, qv[u].x, rv[u].x), fma(-a, qv[u].y, rv[u].y));
+            r2[i] = ri;
+            acc[0] = fma(ri.x, ri.x, acc[0]);
+            acc[0] = fma(ri.y, ri.y, acc[0]);
         }
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        const int i = n - 1;
+        x[i] = fma(a, p[i], x[i]);
+        const double ri = fma(-a, q[i], r[i]);
+        r[i] = ri;
+        acc[0] = fma(ri, ri, acc[0]);
     }
     double tot[1];
     if (!finish_block<1>(acc, part, ctr, tot) || threadIdx.x != 0) return;
@@ -562,85 +553,67 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(int n, const double *
 // top: z = x_bar) and the sums t0 = sum z, t1 = (r, z), t2 = sum r, t3 = (z, q), t4 = sum q.
 // The last block sets mu (mean of z), rz = (r, z - mu) and beta: first direction 0, CG
 // rz'/rz, FCG -(z - mu, q) / (p, q).
+//
+// FP64 bounds it, five sums a row (22 us of 2.2M rows; the bytes take 12): the sums are multiply-adds,
+// z's conversion integer arithmetic. z itself: with FP32 V-cycles (XT = float, FP32 copy evf of E~) it
+// is formed in FP32 and converted once, else in FP64.
 template <class XT>
-__global__ void __launch_bounds__(kRedThreads) k_combine(int nu, int mtop, SellArgs E, const float *__restrict__ evf,
-                                                         const XT *__restrict__ ys, const XT *__restrict__ xb,
-                                                         double *__restrict__ z, const double *__restrict__ r,
-                                                         const double *__restrict__ q, int neumann, int flexible,
-                                                         int first, double inv_n, double *sc, double *part,
-                                                         unsigned *ctr, const int *__restrict__ perr, double *coef) {
+__global__ void __launch_bounds__(kRedThreads, 2) k_combine(int nu, int mtop, SellArgs E, const float *__restrict__ evf,
+                                                            const XT *__restrict__ ys, const XT *__restrict__ xb,
+                                                            double *__restrict__ z, const double *__restrict__ r,
+                                                            const double *__restrict__ q, int neumann, int flexible,
+                                                            int first, double inv_n, double *sc, double *part,
+                                                            unsigned *ctr, const int *__restrict__ perr, double *coef,
+                                                            double one) {
     pdl_begin();
-    // FP32 V-cycles with an FP32 copy of E~ (evf): z_i = x_bar_i + sum_k e_k y_s(c_k) is formed in
-    // FP32 and converted once (FP64 instructions are scarce on this GPU); otherwise in FP64
-    using ZT = typename std::conditional<std::is_same<XT, float>::value, float, double>::type;
-    const bool lowz = std::is_same<XT, float>::value && evf != nullptr;
+    const XT *ev = sizeof(XT) == sizeof(float) ? (const XT *)evf : (const XT *)E.v;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    constexpr int stride = kRedBlocks * kRedThreads;
+    constexpr int R = sizeof(XT) == sizeof(float) ? 4 : 2;   // rows per thread and trip
+    const int stride = gridDim.x * kRedThreads;
     const bool dots_q = flexible && !first;
-    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < nu; i0 += kRows * stride) {
-        double zv[kRows], rv[kRows], qv[kRows];
-        ZT zl[kRows];
-        // loads of every row first (the E~ row entries, x_bar, r, q), then the gathers of y_s
-        int ec[kRows][kEmax];
-        double ev[kRows][kEmax];
-        ZT el[kRows][kEmax];
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < nu; i0 += R * stride) {
+        // loads of every row first (x_bar, r, q, the E~ row's entries), then the gathers of y_s
+        double rv[R], qv[R];
+        XT zl[R], el[R][kEmax];
+        int ec[R][kEmax], wd[R], of[R];
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            int i = i0 + u * stride;
-            zv[u] = 0.0;
-            zl[u] = (ZT)0;
-            rv[u] = 0.0;
-            qv[u] = 0.0;
-#pragma unroll
-            for (int k = 0; k < kEmax; ++k) { ec[u][k] = -1; ev[u][k] = 0.0; el[u][k] = (ZT)0; }
-            if (i >= nu) continue;
-            rv[u] = r[i];
-            if (dots_q) qv[u] = q[i];
-            if (i < mtop) continue;
-            if (mtop == 0) { zv[u] = (double)xb[i]; continue; }
-            int qq = i - mtop, sl = qq >> 5, ln = qq & 31;
-            int o = E.off[sl] + ln, w = E.width[sl];
-            if (lowz) zl[u] = (ZT)xb[qq];
-            else zv[u] = (double)xb[qq];
-            if (w <= kEmax) {
-#pragma unroll
-                for (int k = 0; k < kEmax; ++k)
-                    if (k < w) {
-                        ec[u][k] = __ldg(E.col + o + 32 * k);
-                        if (lowz) el[u][k] = (ZT)__ldg(evf + o + 32 * k);
-                        else ev[u][k] = __ldg(E.v + o + 32 * k);
-                    }
-            } else if (lowz) {
-                zl[u] += (ZT)sell_row<float, XT, float>(E.col, evf, o, w, ys, -1);
-            } else {
-                zv[u] += sell_row<double, XT, double>(E.col, E.v, o, w, ys, -1);
+        for (int u = 0; u < R; ++u) {
+            const int i = i0 + u * stride;
+            const bool ok = i < nu, low = ok && i >= mtop;
+            rv[u] = ok ? r[i] : 0.0;
+            qv[u] = ok && dots_q ? q[i] : 0.0;
+            zl[u] = low ? xb[i - mtop] : ok ? ys[i] : (XT)0;
+            wd[u] = of[u] = 0;
+            if (low && mtop > 0) {
+                const int sl = (i - mtop) >> 5;
+                of[u] = E.off[sl] + ((i - mtop) & 31);
+                wd[u] = E.width[sl];
             }
         }
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            int i = i0 + u * stride;
-            if (i >= nu) continue;
-            double zi;
-            if (lowz && i >= mtop && mtop > 0) {
-                ZT zf = zl[u];
+        for (int u = 0; u < R; ++u)
 #pragma unroll
-                for (int k = 0; k < kEmax; ++k)
-                    if (ec[u][k] >= 0) zf += el[u][k] * (ZT)ys[ec[u][k]];
-                zi = (double)zf;
-            } else {
-                zi = zv[u];
-                if (i < mtop) zi = (double)ys[i];
-#pragma unroll
-                for (int k = 0; k < kEmax; ++k)
-                    if (ec[u][k] >= 0) zi += ev[u][k] * (double)ys[ec[u][k]];
+            for (int k = 0; k < kEmax; ++k) {
+                const bool on = k < wd[u] && wd[u] <= kEmax;
+                ec[u][k] = on ? __ldg(E.col + of[u] + 32 * k) : -1;
+                el[u][k] = on ? __ldg(ev + of[u] + 32 * k) : (XT)0;
             }
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= nu) continue;
+            if (wd[u] > kEmax) zl[u] += sell_row<XT, XT, XT>(E.col, ev, of[u], wd[u], ys);
+#pragma unroll
+            for (int k = 0; k < kEmax; ++k)
+                if (ec[u][k] >= 0) zl[u] += el[u][k] * ys[ec[u][k]];
+            const double zi = cvt<double>(zl[u]);
             z[i] = zi;
-            acc[0] += zi;
-            acc[1] += rv[u] * zi;
-            acc[2] += rv[u];
+            acc[0] = dadd(acc[0], zi, one);
+            acc[1] = fma(rv[u], zi, acc[1]);
+            acc[2] = dadd(acc[2], rv[u], one);
             if (dots_q) {
-                acc[3] += zi * qv[u];
-                acc[4] += qv[u];
+                acc[3] = fma(zi, qv[u], acc[3]);
+                acc[4] = dadd(acc[4], qv[u], one);
             }
         }
     }
@@ -662,12 +635,17 @@ __global__ void __launch_bounds__(kRedThreads) k_combine(int nu, int mtop, SellA
     if (!first && k >= 1 && 2 * k - 1 < kCoefCap) coef[2 * k - 1] = beta;
 }
 
-// p = (z - mu) + beta p
+// p = (z - mu) + beta p, two rows a thread
 __global__ void k_update_p(int n, const double *__restrict__ sc, const double *__restrict__ z, double *__restrict__ p) {
     pdl_begin();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double mu = sc[S_MU], beta = sc[S_BETA];
-    if (i < n) p[i] = (z[i] - mu) + beta * p[i];
+    const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const double mu = sc[S_MU], beta = sc[S_BETA];
+    if (i + 1 < n) {
+        const double2 zv = *(const double2 *)(z + i), pv = *(const double2 *)(p + i);
+        *(double2 *)(p + i) = make_double2(fma(beta, pv.x, zv.x - mu), fma(beta, pv.y, zv.y - mu));
+    } else if (i < n) {
+        p[i] = fma(beta, p[i], z[i] - mu);
+    }
 }
 
 // sum of a vector; the last block stores the mean in sc[slot]
@@ -675,13 +653,13 @@ __global__ void __launch_bounds__(kRedThreads) k_mean(int n, const double *__res
                                                       double *sc, double *part, unsigned *ctr) {
     pdl_begin();
     double acc[1] = {0.0};
-    constexpr int stride = kRedBlocks * kRedThreads;
-    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += kRows * stride) {
-        double v[kRows];
+    const int stride = gridDim.x * kRedThreads;
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        double v[4];
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) v[u] = i0 + u * stride < n ? a[i0 + u * stride] : 0.0;
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u * stride < n ? a[i0 + u * stride] : 0.0;
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) acc[0] += v[u];
+        for (int u = 0; u < 4; ++u) acc[0] += v[u];
     }
     double tot[1];
     if (!finish_block<1>(acc, part, ctr, tot) || threadIdx.x != 0) return;
@@ -696,22 +674,21 @@ __global__ void __launch_bounds__(kRedThreads) k_prepare(int n, int neumann, dou
     pdl_begin();
     double mu = neumann ? sc[S_BMEAN] : 0.0;
     double acc[1] = {0.0};
-    constexpr int stride = kRedBlocks * kRedThreads;
-    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += kRows * stride) {
-        double v[kRows];
+    const int stride = gridDim.x * kRedThreads;
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        double v[4];
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) v[u] = i0 + u * stride < n ? b[i0 + u * stride] : 0.0;
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u * stride < n ? b[i0 + u * stride] : 0.0;
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            int i = i0 + u * stride;
-            if (i < n) {
-                double bi = v[u] - mu;
-                b[i] = bi;
-                r[i] = bi;
-                x[i] = 0.0;
-                p[i] = 0.0;
-                acc[0] += bi * bi;
-            }
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= n) continue;
+            const double bi = v[u] - mu;
+            b[i] = bi;
+            r[i] = bi;
+            x[i] = 0.0;
+            p[i] = 0.0;
+            acc[0] = fma(bi, bi, acc[0]);
         }
     }
     double tot[1];
@@ -737,10 +714,10 @@ __global__ void __launch_bounds__(kRedThreads) k_true_res(SellArgs A, const doub
     pdl_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double acc[1] = {0.0};
-    for (int s = blockIdx.x * (kRedThreads / 32) + warp; s < A.nsl; s += kRedBlocks * (kRedThreads / 32)) {
+    for (int s = blockIdx.x * (kRedThreads / 32) + warp; s < A.nsl; s += gridDim.x * (kRedThreads / 32)) {
         if (lane < A.nrow[s]) {
             int r = A.row0[s] + lane;
-            double d = b[r] - sell_row<double, double, double>(A.col, A.v, A.off[s] + lane, A.width[s], x, -1);
+            double d = b[r] - sell_row<double, double, double>(A.col, A.v, A.off[s] + lane, A.width[s], x);
             acc[0] += d * d;
         }
     }
@@ -830,10 +807,10 @@ static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, 
                                  (double)sizeof(XT) * mt
                            : 0.0),
                   s);
-    pdl_launch(k_combine<XT>, kRedBlocks, kRedThreads, s, h->nu, mt, sargs(h->Enon), (const float *)h->Enon_vf, ys, xb, z, r,
+    pdl_launch(k_combine<XT>, vec_blocks(h->nu), kRedThreads, s, h->nu, mt, sargs(h->Enon), (const float *)h->Enon_vf, ys, xb, z, r,
                                                      h->q, neu, flex, first, 1.0 / (double)h->nu, h->scal,
                                                      h->red + 5 * kRedBlocks * C_Z, h->ctr + C_Z,
-                                                     persist ? persist_err(h) : nullptr, h->coef);
+                                                     persist ? persist_err(h) : nullptr, h->coef, 1.0);
     SOLVE_LAUNCHED();
 }
 
@@ -845,7 +822,7 @@ static void precond_solve_order(vemg_hierarchy *h, const double *r, double *z, i
 // q = A p of the outer loop, with (p, q) and alpha
 static void spmv_outer(vemg_hierarchy *h, const double *x, double *y, cudaStream_t s) {
     ProbeScope ps(PROBE_SPMV_A, sell_bytes(h->Aop.nnz, 8.0, h->Aop.n, 24.0), s);   // p read twice, q write
-    pdl_launch(k_spmv_pq, kRedBlocks, kRedThreads, s, sargs(h->Aop), x, y, h->scal, h->red + 5 * kRedBlocks * C_SPMV,
+    pdl_launch(k_spmv_pq, row_blocks(h->Aop), kRedThreads, s, sargs(h->Aop), x, y, h->scal, h->red + 5 * kRedBlocks * C_SPMV,
                                                  h->ctr + C_SPMV, h->coef);
     SOLVE_LAUNCHED();
 }
@@ -890,17 +867,17 @@ static void phase_pre(vemg_hierarchy *h, cudaStream_t s) {
     const bool neu = h->bc == VEMG_NEUMANN;
     const int nu = h->nu;
     if (neu) {
-        pdl_launch(k_mean, kRedBlocks, kRedThreads, s, nu, h->b, 1.0 / (double)nu, S_BMEAN, h->scal, part_of(h, C_SUMB),
+        pdl_launch(k_mean, vec_blocks(nu), kRedThreads, s, nu, h->b, 1.0 / (double)nu, S_BMEAN, h->scal, part_of(h, C_SUMB),
                                                   h->ctr + C_SUMB);
         SOLVE_LAUNCHED();
     }
-    pdl_launch(k_prepare, kRedBlocks, kRedThreads, s, nu, neu, h->b, h->r, h->x, h->p, h->scal, part_of(h, C_PREP),
+    pdl_launch(k_prepare, vec_blocks(nu), kRedThreads, s, nu, neu, h->b, h->r, h->x, h->p, h->scal, part_of(h, C_PREP),
                                                  h->ctr + C_PREP);
     SOLVE_LAUNCHED();
     precond_solve_order(h, h->r, h->z, 1, s);
     {
         ProbeScope ps(PROBE_VECTOR, 24.0 * nu, s);   // z, p read; p written
-        pdl_launch(k_update_p, grid_for(nu, 256), 256, s, nu, h->scal, h->z, h->p);
+        pdl_launch(k_update_p, grid_for(nu, 512), 256, s, nu, h->scal, h->z, h->p);
         SOLVE_LAUNCHED();
     }
 }
@@ -909,7 +886,7 @@ static void phase_pre(vemg_hierarchy *h, cudaStream_t s) {
 static void phase_step(vemg_hierarchy *h, cudaStream_t s, cudaGraphConditionalHandle hd, int use_cond) {
     spmv_outer(h, h->p, h->q, s);
     ProbeScope ps(PROBE_VECTOR, 48.0 * h->nu, s);   // p, q, x, r read; x, r written
-    pdl_launch(k_update_xr, kRedBlocks, kRedThreads, s, h->nu, h->p, h->q, h->x, h->r, h->scal, part_of(h, C_XR),
+    pdl_launch(k_update_xr, vec_blocks(h->nu), kRedThreads, s, h->nu, h->p, h->q, h->x, h->r, h->scal, part_of(h, C_XR),
                                                    h->ctr + C_XR, hd, use_cond);
     SOLVE_LAUNCHED();
 }
@@ -918,7 +895,7 @@ static void phase_step(vemg_hierarchy *h, cudaStream_t s, cudaGraphConditionalHa
 static void phase_direction(vemg_hierarchy *h, cudaStream_t s) {
     precond_solve_order(h, h->r, h->z, 0, s);
     ProbeScope ps(PROBE_VECTOR, 24.0 * h->nu, s);   // z, p read; p written
-    pdl_launch(k_update_p, grid_for(h->nu, 256), 256, s, h->nu, h->scal, h->z, h->p);
+    pdl_launch(k_update_p, grid_for(h->nu, 512), 256, s, h->nu, h->scal, h->z, h->p);
     SOLVE_LAUNCHED();
 }
 
@@ -926,13 +903,13 @@ static void phase_post(vemg_hierarchy *h, cudaStream_t s) {
     const bool neu = h->bc == VEMG_NEUMANN;
     const int nu = h->nu;
     if (neu) {
-        pdl_launch(k_mean, kRedBlocks, kRedThreads, s, nu, h->x, 1.0 / (double)nu, S_XMEAN, h->scal, part_of(h, C_SUMX),
+        pdl_launch(k_mean, vec_blocks(nu), kRedThreads, s, nu, h->x, 1.0 / (double)nu, S_XMEAN, h->scal, part_of(h, C_SUMX),
                                                   h->ctr + C_SUMX);
         SOLVE_LAUNCHED();
         pdl_launch(k_sub_scalar, grid_for(nu, 256), 256, s, nu, h->x, h->scal, S_XMEAN);
         SOLVE_LAUNCHED();
     }
-    pdl_launch(k_true_res, kRedBlocks, kRedThreads, s, sargs(h->Aop), h->x, h->b, h->scal, part_of(h, C_TRUE),
+    pdl_launch(k_true_res, row_blocks(h->Aop), kRedThreads, s, sargs(h->Aop), h->x, h->b, h->scal, part_of(h, C_TRUE),
                                                   h->ctr + C_TRUE);
     SOLVE_LAUNCHED();
 }

@@ -208,7 +208,8 @@ typedef struct vemg_engine vemg_engine;
 /* Launch shapes of the batched solve's row kernels (the paper has no counterpart: an autotuner of
    this implementation). Three classes: 0 = colour sweeps, 1 = the other V-cycle operations,
    2 = the outer FP64 operations (A p, the true residual, E~ and E~^T). Each has kw lanes per row
-   (4, 8, 16 or 32; each lane takes the columns lane, lane + kw, ...) and warps per block (2, 4, 8).
+   (4, 8, 16 or 32; each lane takes up to 16 bytes of neighbouring columns at a time) and warps per
+   block (2, 4, 8).
    The first batched solve (or engine) of a width K times every candidate shape on this
    hierarchy's finest level and outer operator and keeps the fastest of each class; the results do
    not depend on the shapes. vemg_batch_tuning reports the batch width and the shapes in use with

@@ -2,10 +2,9 @@
 // batch.cu -- many right-hand sides in one solve.
 //
 // K systems A x_c = b_c share one hierarchy. Vectors are interleaved (row-major n x K, K a power
-// of two): x[i*K + c], in the natural (internal) ordering of each level. The operators are the
-// setup's natural-order CSR matrices: a group of KW = min(K, 32) lanes works on one row, the lanes
-// load KW consecutive entries of the row at once and pass them round by warp shuffles, so each
-// matrix entry is read once for all columns and the gathers x[j*K + c] are KW consecutive words.
+// of two): x[i*K + c], in the natural (internal) ordering of each level. A group of KW lanes works on
+// one row, each lane on V neighbouring columns per load (16 bytes where the batch is wide enough), so
+// each matrix entry is read once for all columns and a gather of x[j*K ..] is one wide load per lane.
 // Natural order keeps a row's neighbours close in memory, so the gathers stay in L2 even when the
 // K-column vectors are far larger than L2 (the colour-major order of the one-column solve does
 // not: each colour's pass would sweep the whole vector). Colour sweeps walk the level's list of
@@ -16,24 +15,18 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include <type_traits>
 
-#include "internal.cuh"
+#include "sell.cuh"
 
 namespace vemg {
 
-static constexpr int kBT = 512;        // their threads
-static constexpr int kBU = 8;          // entries loaded per round trip in a batched row
+static constexpr int kBT = 512;        // threads of the streaming kernels
 static constexpr int kMaxK = 128;      // widest batch
 static constexpr int kSellWarps = 4;   // warps per block of the batched row kernels (untuned default)
 static constexpr int kMaxWarps = 8;    // most warps per block the autotuner tries
-// columns a lane of a batched row kernel takes per pass when the batch is wide enough (K >= that
-// many times the lanes per row): 8 with FP32 accumulators, 4 with FP64 ones (8 FP64 accumulators
-// spill). Narrower batches take one column per pass: unused accumulator slots cost registers and
-// code size, which slowed the 8-column engines of the serving stream by about 2x.
-template <class AT>
-__host__ __device__ constexpr int cols_per_lane() { return sizeof(AT) == 4 ? 8 : 4; }
 
 static thread_local int64_t *b_count = nullptr;
 struct BTune;
@@ -62,14 +55,28 @@ static constexpr int kStallIters = 30;
 // global scalars after the per-column block (g[slot])
 enum { G_TOL = 0, G_MAXIT, G_CONT, G_ITERS, G_COUNT };
 
+// One operator as the batched row kernels read it: entries of row r at rp[r] - r * diag, a row
+// without its diagonal having one fewer (diag = 1). The chains' operators have their own copies:
+// FP32 values packed with their columns (ent: 8 bytes an entry, one load), and in a level's matrix the
+// diagonal left out and the entries of earlier colours first (lo[r] of them), so that a sweep from
+// x = 0 reads only those and the residual after it only the others (as in the one-column solve).
+struct BRows {
+    const int *rp = nullptr, *ci = nullptr;
+    const void *v = nullptr;
+    const int2 *ent = nullptr;
+    const int *lo = nullptr;
+    const int4 *info = nullptr;   // a level's matrix: row, first entry, lower entries, entries; in sweep order
+    int diag = 0;
+    int qsh = 0;            // log2 of the parts a row is split into (parts_shift)
+    double mean = 0.0;      // mean entries per row
+};
+
 // one multigrid level as the batched cycle sees it
 struct BLevel {
     int n = 0, ncolours = 0;
-    const int *rp = nullptr, *ci = nullptr, *colour = nullptr, *crow = nullptr;
-    const void *v = nullptr, *dinv = nullptr;
+    const void *dinv = nullptr;
     std::vector<int> cptr;
-    const int *prp = nullptr, *pci = nullptr, *trp = nullptr, *tci = nullptr;
-    const void *pv = nullptr, *tv = nullptr;
+    BRows A, P, PT;
 };
 
 struct BChain {
@@ -81,11 +88,6 @@ struct BChain {
     const float *Gf = nullptr;   // FP32 copy (FP32 cycles)
 };
 
-struct CsrP {
-    const int *rp, *ci;
-    const void *v;
-};
-
 struct BatchGraphs {
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -94,9 +96,9 @@ struct BatchGraphs {
 };
 
 // Launch shapes of the batched row kernels, by class: 0 = colour sweeps, 1 = the other V-cycle
-// operations (residuals, restrictions, prolongations), 2 = the outer FP64 operations (A p, the
-// true residual, E~ and E~^T). kw: lanes per row (each lane takes columns lane, lane + kw, ...),
-// warps: warps per block. Chosen per batch width by timing the candidates (autotune below); the
+// operations (residuals, restrictions, prolongations, E~ in FP32), 2 = the outer FP64 operations (A p,
+// the true residual, E~ and E~^T). kw: lanes per row (each lane takes 16 bytes of neighbouring
+// columns at a time), warps: warps per block. Chosen per batch width by timing the candidates (autotune below); the
 // per-column arithmetic is the same for every shape.
 struct BTune {
     int kw[3] = {0, 0, 0}, warps[3] = {0, 0, 0};   // 0: the untuned default
@@ -115,12 +117,12 @@ struct BatchWork {
     BatchGraphs *graphs = nullptr;
     Arena arena;
     BChain *bsurf = nullptr, *bbar = nullptr;
-    CsrP Aout{};
+    BRows Aout, E, ET;   // the outer operators, FP64 (E: FP32 with FP32 V-cycles)
     const int *caller_of = nullptr;   // caller id of each unknown (internal order)
-    // FP32 V-cycles: E~'s values in FP32 (the prolongation z = E~ y_s is formed in FP32) and an
-    // FP32 copy of the A_bar part of the outer residual (the finest level's right-hand side,
-    // converted once per application instead of on every read)
-    float *Ev32 = nullptr, *Rb32 = nullptr;
+    // FP32 V-cycles: an FP32 copy of the A_bar part of the outer residual (the finest level's
+    // right-hand side, converted once per application instead of on every read); E~'s values are
+    // FP32 too (the prolongation z = E~ y_s is formed in FP32)
+    float *Rb32 = nullptr;
     ~BatchWork() {
         delete bsurf;
         delete bbar;
@@ -130,203 +132,229 @@ struct BatchWork {
 static double *gsc(BatchWork *w) { return w->sc + B_COUNT * w->K; }
 
 // ------------------------------------------------------------------------------------------
-// batched CSR row operations (natural order)
+// batched row operations (natural order)
 
 // BOP_SPMV_PLUS: y = b_part + A x, where rows r >= cur start from b[(r - cur) K + c] (and the
-// others from 0): z = [0; x_bar] + E~ y_s formed in the accumulator type, converted once
-enum { BOP_SPMV = 0, BOP_SPMV_ADD = 1, BOP_SOR = 2, BOP_RES = 3, BOP_SPMV_PLUS = 4 };
+// others from 0): z = [0; x_bar] + E~ y_s formed in the accumulator type, converted once.
+// BOP_UPPER: the residual after a sweep from zero in ascending colours, y = -(entries of later colours) x
+enum { BOP_SPMV = 0, BOP_SPMV_ADD = 1, BOP_SOR = 2, BOP_RES = 3, BOP_SPMV_PLUS = 4, BOP_UPPER = 5 };
 
-__global__ void k_bto_float(int64_t n, const double *__restrict__ a, float *__restrict__ b) {
-    pdl_begin();
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) b[i] = (float)a[i];
+
+// V neighbouring columns, in loads and stores of up to 16 bytes (p is aligned to V elements: V
+// divides K and the vectors start on 256-byte boundaries)
+template <int V, class T>
+__device__ __forceinline__ void load_cols(const T *p, T (&o)[V]) {
+    constexpr int B = V * (int)sizeof(T);
+    if constexpr (B >= 16) {
+#pragma unroll
+        for (int k = 0; k < B / 16; ++k) {
+            const float4 f = *(const float4 *)((const char *)p + 16 * k);
+            memcpy((char *)o + 16 * k, &f, 16);
+        }
+    } else if constexpr (B == 8) {
+        const float2 f = *(const float2 *)p;
+        memcpy(o, &f, 8);
+    } else {
+        o[0] = *p;
+    }
 }
-
-// Rows idx in [0, nrows): row = rows ? rows[idx] : r0 + idx, a group of KW lanes per row, columns
-// c = lane % KW + j KW. SOR skips the diagonal entry and, when sweeping from x = 0 (cur >= 0), every
-// entry whose column has colour >= cur (not yet visited: zero). RES keeps the diagonal: y = b - A x.
-template <int OP, class VT, class XT, class BT, class YT, class AT, int KW, int CPL>
-__global__ void __launch_bounds__(32 * kMaxWarps) k_bcsr(int nrows, const int *__restrict__ rows, int r0, CsrP A,
-                                                         const VT *__restrict__ dg, const BT *__restrict__ b,
-                                                         const XT *x, YT *y, int K, const int *__restrict__ colour,
-                                                         int cur) {
-    constexpr int RW = 32 / KW;
-    int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (w * RW >= nrows) {   // warp-uniform
-        pdl_begin();
-        return;
-    }
-    int idx = w * RW + lane / KW;
-    bool valid = idx < nrows;
-    int r = valid ? (rows ? rows[idx] : r0 + idx) : 0;
-    int lo = valid ? A.rp[r] : 0, wd = valid ? A.rp[r + 1] - lo : 0;
-    const VT *v = (const VT *)A.v;
-    const int gl = lane % KW, gb = lane - gl;
-    const bool skip_all = OP == BOP_SOR && cur == 0;
-    int wmax = __reduce_max_sync(0xffffffffu, (unsigned)wd);
-    // the row's first KW entries are setup data: loaded before waiting on the previous kernel
-    int cc0 = -1;
-    VT vv0 = (VT)0;
-    if (!skip_all) {
-        cc0 = gl < wd ? __ldg(A.ci + lo + gl) : -1;
-        vv0 = gl < wd ? __ldg(v + lo + gl) : (VT)0;
-        if (OP == BOP_SOR && cc0 >= 0 && (cc0 == r || (cur > 0 && __ldg(colour + cc0) >= cur))) cc0 = -1;
-    }
-    pdl_begin();
-    // a lane takes the columns c0, c0 + KW, ..., CPL of them per pass, so that each entry of the
-    // row issues CPL independent loads of its neighbour's x row. K, KW and CPL are powers of two
-    // and K is a multiple of CPL * KW (or CPL = 1), so every column c0 + u KW of a pass exists and
-    // every lane of the warp makes the same number of passes (the shuffles need all 32).
-    for (int c0 = gl; c0 < K; c0 += CPL * KW) {
-        AT acc[CPL];
+template <int V, class T>
+__device__ __forceinline__ void store_cols(T *p, const T (&o)[V]) {
+    constexpr int B = V * (int)sizeof(T);
+    if constexpr (B >= 16) {
 #pragma unroll
-        for (int u = 0; u < CPL; ++u)
-            acc[u] = (OP == BOP_SPMV_PLUS && valid && r >= cur) ? (AT)b[(int64_t)(r - cur) * K + c0 + u * KW] : (AT)0;
-        if (!skip_all) {
-            for (int k0 = 0; k0 < wmax; k0 += KW) {
-                int k = k0 + gl;
-                int cc = cc0;
-                VT vv = vv0;
-                if (k0 > 0) {
-                    cc = k < wd ? __ldg(A.ci + lo + k) : -1;
-                    vv = k < wd ? __ldg(v + lo + k) : (VT)0;
-                    if (OP == BOP_SOR && cc >= 0 && (cc == r || (cur > 0 && __ldg(colour + cc) >= cur))) cc = -1;
-                }
-                int nj = min(KW, wmax - k0);
-#pragma unroll
-                for (int jj = 0; jj < KW; ++jj) {
-                    if (jj < nj) {
-                        int cj = __shfl_sync(0xffffffffu, cc, gb + jj);
-                        VT vj = __shfl_sync(0xffffffffu, vv, gb + jj);
-                        if (cj >= 0) {
-                            const XT *xr = x + (int64_t)cj * K;
-#pragma unroll
-                            for (int u = 0; u < CPL; ++u) acc[u] += (AT)vj * (AT)xr[c0 + u * KW];
-                        }
-                    }
-                }
-            }
+        for (int k = 0; k < B / 16; ++k) {
+            float4 f;
+            memcpy(&f, (const char *)o + 16 * k, 16);
+            *(float4 *)((char *)p + 16 * k) = f;
         }
-        if (!valid) continue;
-#pragma unroll
-        for (int u = 0; u < CPL; ++u) {
-            const int c = c0 + u * KW;
-            int64_t e = (int64_t)r * K + c;
-            if (OP == BOP_SPMV || OP == BOP_SPMV_PLUS) y[e] = (YT)acc[u];
-            else if (OP == BOP_SPMV_ADD) y[e] = (YT)((AT)y[e] + acc[u]);
-            else if (OP == BOP_SOR) y[e] = (YT)(((AT)b[e] - acc[u]) * (AT)dg[r]);
-            else y[e] = (YT)((AT)b[e] - acc[u]);
-        }
+    } else if constexpr (B == 8) {
+        float2 f;
+        memcpy(&f, o, 8);
+        *(float2 *)p = f;
+    } else {
+        *p = o[0];
     }
 }
 
-// one lane per row and column group (K = 1, 2): entries loaded kBU at a time
-template <int OP, class VT, class XT, class BT, class YT, class AT, int KW>
-__global__ void __launch_bounds__(32 * kMaxWarps) k_bcsr_narrow(int nrows, const int *__restrict__ rows, int r0,
-                                                                CsrP A, const VT *__restrict__ dg,
-                                                                const BT *__restrict__ b, const XT *x, YT *y, int K,
-                                                                const int *__restrict__ colour, int cur) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int idx = (int)(t / KW), c = (int)(t % KW);
-    if (idx >= nrows) {
+// up to kBU entries of a row
+static constexpr int kBU = 4;
+template <bool PACK, class VT>
+struct Entries {
+    int c[kBU];
+    VT v[kBU];
+    __device__ __forceinline__ void load(const BRows &A, int at, int step, int n) {
+#pragma unroll
+        for (int u = 0; u < kBU; ++u) {
+            c[u] = 0;
+            v[u] = (VT)0;
+            if (u < n) {
+                if constexpr (PACK) {
+                    const int2 e = __ldg(A.ent + at + u * step);
+                    c[u] = e.x;
+                    v[u] = __int_as_float(e.y);
+                } else {
+                    c[u] = __ldg(A.ci + at + u * step);
+                    v[u] = __ldg((const VT *)A.v + at + u * step);
+                }
+            }
+        }
+    }
+};
+
+// Rows idx in [0, nrows) (info: in sweep order, else in row order). A warp holds 32 / (KW Q) rows,
+// KW = 1 << kwsh lanes by Q = 1 << A.qsh parts a row: lane l takes the columns (l mod KW) V + j KW V .. + V
+// in pass j, part q the entries q, q + Q, ... of the row, and the parts are added by a fixed xor tree.
+// The sum of a column thus depends on Q and not on the launch shape. K is a multiple of KW V.
+//
+// Latency of the gathers bounds it: 16-byte loads, four entries' gathers before their multiply-adds
+// and the next four entries under way meanwhile, in at most 64 registers (four blocks of 8 warps per
+// SM). The finest sweep's largest colour on the 384 x 384 x 24 mesh with 64 columns: 331 us (422 with one
+// column per load). Eight columns a lane with eight entries held took 102 registers and 446 us; three,
+// five or six blocks per SM, or two entries at a time, were slower for one batch width or another. The
+// outer product is bound by the FP64 pipe instead (54.5M entries x 64 columns: 5.5 of its 6.3 ms).
+template <int OP, bool PACK, class VT, class XT, class BT, class YT, class AT, int V>
+__global__ void __launch_bounds__(32 * kMaxWarps, 4) k_brow(int nrows, const int4 *__restrict__ info, BRows A, int range,
+                                                            const XT *__restrict__ dg, const BT *__restrict__ b,
+                                                            const XT *x, YT *y, int K, int kwsh, int cur) {
+    const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    const int gsh = kwsh + A.qsh, rw = 32 >> gsh, kw = 1 << kwsh, Q = 1 << A.qsh;
+    if ((int64_t)w * rw >= nrows) {   // warp-uniform
         pdl_begin();
         return;
     }
-    int r = rows ? rows[idx] : r0 + idx;
-    int lo = A.rp[r], hi = A.rp[r + 1];
-    const VT *v = (const VT *)A.v;
+    const int idx = w * rw + (lane >> gsh), gl = lane & (kw - 1), part = (lane >> kwsh) & (Q - 1);
+    const bool valid = idx < nrows, out = valid && part == 0;
+    int r = 0, at = 0, n = 0;   // row, first entry and entries of this part
+    if (valid) {
+        int lo = 0, len;
+        if (info) {
+            const int4 m = __ldg(info + idx);
+            r = m.x;
+            at = m.y;
+            lo = m.z;
+            len = m.w;
+        } else {
+            r = idx;
+            const int o = __ldg(A.rp + r);
+            len = __ldg(A.rp + r + 1) - o - A.diag;
+            if (range != ROW_ALL) lo = __ldg(A.lo + r);
+            at = o - r * A.diag;
+        }
+        const int e0 = range == ROW_UPPER ? lo : 0, e1 = range == ROW_LOWER ? lo : len;
+        at += e0 + part;
+        n = (e1 - e0 - part + Q - 1) >> A.qsh;
+    }
+    Entries<PACK, VT> h;
+    h.load(A, at, Q, n);
+    const XT d = OP == BOP_SOR && out ? __ldg(dg + r) : (XT)0;
     pdl_begin();
-    AT acc = (OP == BOP_SPMV_PLUS && r >= cur) ? (AT)b[(int64_t)(r - cur) * K + c] : (AT)0;
-    if (!(OP == BOP_SOR && cur == 0)) {
-        for (int k0 = lo; k0 < hi; k0 += kBU) {
-            int cc[kBU];
-            VT a[kBU];
+    for (int c0 = gl * V; c0 < K; c0 += kw * V) {
+        AT acc[V];
 #pragma unroll
-            for (int u = 0; u < kBU; ++u) {
-                int k = k0 + u;
-                cc[u] = k < hi ? __ldg(A.ci + k) : -1;
-                a[u] = k < hi ? __ldg(v + k) : (VT)0;
-                if (OP == BOP_SOR && cc[u] >= 0 && (cc[u] == r || (cur > 0 && __ldg(colour + cc[u]) >= cur))) cc[u] = -1;
-            }
+        for (int i = 0; i < V; ++i) acc[i] = (AT)0;
+        BT bv[V];
+        if ((OP == BOP_SOR || OP == BOP_RES) && out) load_cols<V>(b + (int64_t)r * K + c0, bv);
+        if (OP == BOP_SPMV_PLUS && out && r >= cur) {
+            load_cols<V>(b + (int64_t)(r - cur) * K + c0, bv);
+#pragma unroll
+            for (int i = 0; i < V; ++i) acc[i] = (AT)bv[i];
+        }
+        const XT *xc = x + c0;
+        for (int t = 0; t < n; t += kBU) {
+            XT g[kBU][V];
 #pragma unroll
             for (int u = 0; u < kBU; ++u)
-                if (cc[u] >= 0) acc += (AT)a[u] * (AT)x[(int64_t)cc[u] * K + c];
+                if (t + u < n) load_cols<V>(xc + (int64_t)h.c[u] * K, g[u]);
+            Entries<PACK, VT> cu = h;
+            // the next entries of the row, or its first ones again for the next pass
+            if (t + kBU < n) h.load(A, at + (t + kBU) * Q, Q, n - t - kBU);
+            else if (n > kBU) h.load(A, at, Q, n);
+#pragma unroll
+            for (int u = 0; u < kBU; ++u)
+                if (t + u < n)
+#pragma unroll
+                    for (int i = 0; i < V; ++i) acc[i] = fmadd((AT)cu.v[u], (AT)g[u][i], acc[i]);
         }
+        for (int o = 1 << (gsh - 1); A.qsh > 0 && o >= kw; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < V; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+        if (!out) continue;
+        const int64_t e = (int64_t)r * K + c0;
+        YT res[V];
+        if (OP == BOP_SPMV_ADD) load_cols<V>((const YT *)y + e, res);
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const AT s = acc[i];
+            if (OP == BOP_SPMV || OP == BOP_SPMV_PLUS) res[i] = cvt<YT>(s);
+            else if (OP == BOP_SPMV_ADD) res[i] = (YT)((AT)res[i] + s);
+            else if (OP == BOP_SOR) res[i] = (YT)((cvt<AT>(bv[i]) - s) * (AT)d);
+            else if (OP == BOP_RES) res[i] = (YT)((AT)bv[i] - s);
+            else res[i] = (YT)((AT)0 - s);
+        }
+        store_cols<V>(y + e, res);
     }
-    int64_t e = (int64_t)r * K + c;
-    if (OP == BOP_SPMV || OP == BOP_SPMV_PLUS) y[e] = (YT)acc;
-    else if (OP == BOP_SPMV_ADD) y[e] = (YT)((AT)y[e] + acc);
-    else if (OP == BOP_SOR) y[e] = (YT)(((AT)b[e] - acc) * (AT)dg[r]);
-    else y[e] = (YT)((AT)b[e] - acc);
 }
 
-// cls: the launch-shape class of the call (BTune); kw, nw > 0 force a shape (autotuning)
-template <int OP, class VT, class XT, class BT, class YT, class AT>
-static void bcsr(CsrP A, int nrows, const int *rows, int r0, const VT *dg, const BT *b, const XT *x, YT *y, int K,
-                 const int *colour, int cur, cudaStream_t s, int cls = 1, int kw = 0, int nw = 0) {
+// V: the columns of a 16-byte load of x, where a lane has that many. kw, nw > 0 force a shape
+// (autotuning); cls: the launch-shape class (BTune). info: the rows of a colour, else all rows.
+template <int OP, bool PACK, class VT, class XT, class BT, class YT, class AT>
+static void brow(const BRows &A, int nrows, const int4 *info, int range, const XT *dg, const BT *b, const XT *x, YT *y,
+                 int K, int cur, cudaStream_t s, int cls = 1, int kw = 0, int nw = 0) {
     if (nrows <= 0) return;
     if (kw <= 0 && b_tune && b_tune->kw[cls] > 0) {
         kw = b_tune->kw[cls];
         nw = b_tune->warps[cls];
     }
-    int KW = std::min(K, kw > 0 ? kw : 32);
+    constexpr int VM = 16 / (int)sizeof(XT);
     const int wpb = nw > 0 ? nw : kSellWarps;
-    dim3 blk(32 * wpb);
-    if (KW < 4) {
-        int64_t t = (int64_t)nrows * KW;
-        if (KW == 1)
-            pdl_launch(k_bcsr_narrow<OP, VT, XT, BT, YT, AT, 1>, grid_for(t, 32 * wpb), blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-        else
-            pdl_launch(k_bcsr_narrow<OP, VT, XT, BT, YT, AT, 2>, grid_for(t, 32 * wpb), blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-        BATCH_LAUNCHED();
-        return;
-    }
-    int RW = 32 / KW;
-    int64_t warps = (nrows + RW - 1) / RW;
-    int grid = (int)((warps + wpb - 1) / wpb);
-    constexpr int C = cols_per_lane<AT>();
-    const bool wide = K >= C * KW;   // then K is a multiple of C * KW (both powers of two)
-    switch (KW) {
-        case 4:
-            if (wide) pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 4, C>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            else pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 4, 1>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            break;
-        case 8:
-            if (wide) pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 8, C>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            else pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 8, 1>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            break;
-        case 16:
-            if (wide) pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 16, C>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            else pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 16, 1>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            break;
-        default:
-            if (wide) pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 32, C>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            else pdl_launch(k_bcsr<OP, VT, XT, BT, YT, AT, 32, 1>, grid, blk, s, nrows, rows, r0, A, dg, b, x, y, K, colour, cur);
-            break;
-    }
+    if (kw <= 0) kw = K < 4 ? 1 : 32;
+    const int KW = std::min(K, kw), V = std::min(K / KW, VM);
+    int kwsh = 0;
+    while ((1 << kwsh) < KW) ++kwsh;
+    const int64_t per = 32 >> (kwsh + A.qsh), warps = (nrows + per - 1) / per;
+    auto go = [&](auto v) {
+        pdl_launch(k_brow<OP, PACK, VT, XT, BT, YT, AT, decltype(v)::value>, (int)((warps + wpb - 1) / wpb), 32 * wpb,
+                   s, nrows, info, A, range, dg, b, x, y, K, kwsh, cur);
+    };
+    if (V == 1) go(std::integral_constant<int, 1>{});
+    else if (V < VM) go(std::integral_constant<int, 2>{});
+    else go(std::integral_constant<int, VM>{});
     BATCH_LAUNCHED();
 }
 
-// x = G b on the coarsest level, one thread per (row, column)
+// x = G b on the coarsest level: one block per row, its threads K columns by 256 / K parts of the row
+static constexpr int kDenseThreads = 256;
 template <class XT, class BT>
-__global__ void k_bdense(int n, const XT *__restrict__ G, const BT *__restrict__ b, XT *__restrict__ x, int K) {
+__global__ void __launch_bounds__(kDenseThreads) k_bdense(int n, const XT *__restrict__ G, const BT *__restrict__ b,
+                                                          XT *__restrict__ x, int K) {
     pdl_begin();
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n * K) return;
-    int r = (int)(t >> (__ffs(K) - 1)), c = (int)(t & (K - 1));
+    __shared__ XT sh[kDenseThreads];
+    const int r = blockIdx.x, t = threadIdx.x, c = t & (K - 1), part = t / K, parts = kDenseThreads / K;
     XT s = 0;
-    for (int j = 0; j < n; ++j) s += G[(int64_t)r * n + j] * (XT)b[(int64_t)j * K + c];
-    x[t] = (XT)s;
+#pragma unroll 8
+    for (int j = part; j < n; j += parts) s = fmadd(__ldg(G + (int64_t)r * n + j), cvt<XT>(b[(int64_t)j * K + c]), s);
+    sh[t] = s;
+    for (int o = kDenseThreads / 2; o >= K; o >>= 1) {
+        __syncthreads();
+        if (t < o) sh[t] += sh[t + o];
+    }
+    __syncthreads();
+    if (t < K) x[(int64_t)r * K + t] = sh[t];
 }
+
+// the chains' operators in FP32 are packed
+template <class XT>
+constexpr bool packed() { return sizeof(XT) == sizeof(float); }
 
 template <class XT, class BT>
 static void bsweep(const BLevel &L, const BT *b, XT *x, bool forward, bool from_zero, int K, cudaStream_t s) {
-    CsrP A{L.rp, L.ci, L.v};
     for (int cc = 0; cc < L.ncolours; ++cc) {
         int c = forward ? cc : L.ncolours - 1 - cc;
         int nrows = L.cptr[c + 1] - L.cptr[c];
-        bcsr<BOP_SOR, XT, XT, BT, XT, XT>(A, nrows, L.crow + L.cptr[c], 0, (const XT *)L.dinv, b, x, x, K, L.colour,
-                                         from_zero ? c : -1, s, 0);
+        brow<BOP_SOR, packed<XT>(), XT, XT, BT, XT, XT>(L.A, nrows, L.A.info + L.cptr[c],
+                                                        from_zero ? ROW_LOWER : ROW_ALL, (const XT *)L.dinv, b, x, x,
+                                                        K, -1, s, 0);
     }
 }
 
@@ -336,9 +364,8 @@ static void bvcycle(const BChain &C, BatchWork *W, int ch, int l, const BT *b, X
     const int K = W->K;
     if (l == C.nlev - 1) {
         if (C.direct) {
-            int64_t t = (int64_t)C.nc * K;
             const XT *G = sizeof(XT) == sizeof(float) ? (const XT *)C.Gf : (const XT *)C.G;
-            pdl_launch(k_bdense<XT, BT>, grid_for(t, 256), 256, s, C.nc, G, b, x, K);
+            pdl_launch(k_bdense<XT, BT>, C.nc, kDenseThreads, s, C.nc, G, b, x, K);
             BATCH_LAUNCHED();
             return;
         }
@@ -346,30 +373,33 @@ static void bvcycle(const BChain &C, BatchWork *W, int ch, int l, const BT *b, X
         bsweep<XT, BT>(L, b, x, false, false, K, s);
         return;
     }
+    constexpr bool P = packed<XT>();
     XT *r = (XT *)W->lr[ch][l];
     XT *nb = (XT *)W->lb[ch][l + 1], *nx = (XT *)W->lx[ch][l + 1];
     const BLevel &N = C.lv[l + 1];
+    const XT *none = nullptr;
     bsweep<XT, BT>(L, b, x, true, true, K, s);
-    bcsr<BOP_RES, XT, XT, BT, XT, XT>(CsrP{L.rp, L.ci, L.v}, L.n, nullptr, 0, (const XT *)nullptr, b, x, r, K,
-                                      nullptr, -1, s);
-    bcsr<BOP_SPMV, XT, XT, XT, XT, XT>(CsrP{L.trp, L.tci, L.tv}, N.n, nullptr, 0, (const XT *)nullptr,
-                                       (const XT *)nullptr, r, nb, K, nullptr, -1, s);
+    brow<BOP_UPPER, P, XT, XT, XT, XT, XT>(L.A, L.n, nullptr, ROW_UPPER, none, none, x, r, K, -1, s);
+    brow<BOP_SPMV, P, XT, XT, XT, XT, XT>(L.PT, N.n, nullptr, ROW_ALL, none, none, r, nb, K, -1, s);
     bvcycle<XT, XT>(C, W, ch, l + 1, (const XT *)nb, nx, s);
-    bcsr<BOP_SPMV_ADD, XT, XT, XT, XT, XT>(CsrP{L.prp, L.pci, L.pv}, L.n, nullptr, 0, (const XT *)nullptr,
-                                           (const XT *)nullptr, nx, x, K, nullptr, -1, s);
+    brow<BOP_SPMV_ADD, P, XT, XT, XT, XT, XT>(L.P, L.n, nullptr, ROW_ALL, none, none, nx, x, K, -1, s);
     bsweep<XT, BT>(L, b, x, false, false, K, s);
 }
 
 // ------------------------------------------------------------------------------------------
-// per-column deterministic reductions in two stages. Stage 1 (streaming kernels): each block
-// covers kBT * kBE consecutive elements of the n x K block; thread t always holds column
-// t % K (K divides kBT), loads its kBE elements first, and the block writes one partial per
+// per-column deterministic reductions in two stages. Stage 1 (streaming kernels): the blocks
+// stride over the n x K block by kBT * kBE elements; thread t always holds column
+// t % K (K divides kBT), loads a trip's elements first, and the block writes one partial per
 // column and sum. Stage 2 (k_bstage2): one block per column adds the block partials in fixed
 // order and applies the scalar step of that column; the last column block sets the globals.
 
-static constexpr int kBE = 8;   // elements per thread in stage 1
+static constexpr int kBE = 4;   // elements per thread and trip in stage 1
 
-static int stage1_blocks(int64_t N) { return (int)((N + (int64_t)kBT * kBE - 1) / ((int64_t)kBT * kBE)); }
+// blocks of stage 1: two per SM (fewer for a small batch), each in trips of kBT * kBE elements; partials
+// stay few for stage 2 (one block per 4,096 elements wrote and read 150 MB of them at n K = 2.4e8)
+static int stage1_blocks(int64_t N) {
+    return (int)std::min<int64_t>(304, (N + (int64_t)kBT * kBE - 1) / ((int64_t)kBT * kBE));
+}
 
 template <int NS>
 __device__ void bblock_partials(double (&acc)[NS], int K, double *part) {
@@ -401,52 +431,54 @@ __global__ void __launch_bounds__(kBT) k_bsums(int64_t N, int K, BSums d, double
     double acc[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) acc[s] = 0.0;
-    int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x;
-    double va[NS][kBE], vb[NS][kBE];
+    for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
+        double va[NS][kBE], vb[NS][kBE];
 #pragma unroll
-    for (int j = 0; j < kBE; ++j) {
-        int64_t e = base + (int64_t)j * kBT;
+        for (int j = 0; j < kBE; ++j) {
+            int64_t e = base + (int64_t)j * kBT;
 #pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            va[s][j] = e < N ? d.a[s][e] : 0.0;
-            vb[s][j] = (e < N && d.b[s]) ? d.b[s][e] : 1.0;
+            for (int s = 0; s < NS; ++s) {
+                va[s][j] = e < N ? d.a[s][e] : 0.0;
+                vb[s][j] = (e < N && d.b[s]) ? d.b[s][e] : 1.0;
+            }
         }
+#pragma unroll
+        for (int j = 0; j < kBE; ++j)
+#pragma unroll
+            for (int s = 0; s < NS; ++s) acc[s] = fma(va[s][j], vb[s][j], acc[s]);
     }
-#pragma unroll
-    for (int j = 0; j < kBE; ++j)
-#pragma unroll
-        for (int s = 0; s < NS; ++s) acc[s] = fma(va[s][j], vb[s][j], acc[s]);
     bblock_partials<NS>(acc, K, part);
 }
 
 // the preconditioner's sums over z, r (and q): s0 = sum z, s1 = sum r z, s2 = sum r
-// [, s3 = sum z q, s4 = sum q]; each vector is loaded once per element (the generic kernel
-// above would load z three times and hold 80 values per thread). Same order of accumulation.
+// [, s3 = sum z q, s4 = sum q]; each vector is loaded once per element. FP64 bounds it: five
+// multiply-adds an element (one: 1.0, see dadd).
 template <int NS>
 __global__ void __launch_bounds__(kBT, 2) k_bsums_zrq(int64_t N, int K, const double *__restrict__ z,
                                                       const double *__restrict__ r, const double *__restrict__ q,
-                                                      double *part) {
+                                                      double *part, double one) {
     pdl_begin();
     double acc[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) acc[s] = 0.0;
-    int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x;
-    double vz[kBE], vr[kBE], vq[kBE];
+    for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
+        double vz[kBE], vr[kBE], vq[kBE];
 #pragma unroll
-    for (int j = 0; j < kBE; ++j) {
-        int64_t e = base + (int64_t)j * kBT;
-        vz[j] = e < N ? z[e] : 0.0;
-        vr[j] = e < N ? r[e] : 0.0;
-        vq[j] = (NS == 5 && e < N) ? q[e] : 0.0;
-    }
+        for (int j = 0; j < kBE; ++j) {
+            int64_t e = base + (int64_t)j * kBT;
+            vz[j] = e < N ? z[e] : 0.0;
+            vr[j] = e < N ? r[e] : 0.0;
+            vq[j] = (NS == 5 && e < N) ? q[e] : 0.0;
+        }
 #pragma unroll
-    for (int j = 0; j < kBE; ++j) {
-        acc[0] += vz[j] * 1.0;
-        acc[1] += vr[j] * vz[j];
-        acc[2] += vr[j] * 1.0;
-        if (NS == 5) {
-            acc[3] += vz[j] * vq[j];
-            acc[4] += vq[j] * 1.0;
+        for (int j = 0; j < kBE; ++j) {
+            acc[0] = dadd(acc[0], vz[j], one);
+            acc[1] = fma(vr[j], vz[j], acc[1]);
+            acc[2] = dadd(acc[2], vr[j], one);
+            if (NS == 5) {
+                acc[3] = fma(vz[j], vq[j], acc[3]);
+                acc[4] = dadd(acc[4], vq[j], one);
+            }
         }
     }
     bblock_partials<NS>(acc, K, part);
@@ -579,27 +611,31 @@ __global__ void k_bprepare(int64_t N, int K, int neumann, double *__restrict__ b
 }
 
 // X += alpha P, R -= alpha Q per column, the FP32 copy of R's A_bar part, and the stage-1 sums
-// of R * R: the elements of a thread and the order of its sum are those of k_bsums, so the
-// partials are the same bits as a separate pass would give
-__global__ void __launch_bounds__(kBT) k_bupdate_xr(int64_t N, int K, const double *__restrict__ p,
-                                                    const double *__restrict__ q, double *__restrict__ x,
-                                                    double *__restrict__ r, const double *__restrict__ sc,
-                                                    float *__restrict__ rb32, int64_t off32, double *part) {
+// of R * R (elements of a thread and order as in k_bsums)
+__global__ void __launch_bounds__(kBT, 2) k_bupdate_xr(int64_t N, int K, const double *__restrict__ p,
+                                                       const double *__restrict__ q, double *__restrict__ x,
+                                                       double *__restrict__ r, const double *__restrict__ sc,
+                                                       float *__restrict__ rb32, int64_t off32, double *part) {
     pdl_begin();
     double acc[1] = {0.0};
-    const int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x;
-    const double a = sc[B_ALPHA * K + (int)(base & (K - 1))];   // kBT is a multiple of K: one column
+    const double a = sc[B_ALPHA * K + (int)(threadIdx.x & (K - 1))];   // kBT is a multiple of K: one column
+    for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
+        double vp[kBE], vq[kBE], vx[kBE], vr[kBE];
 #pragma unroll
-    for (int j = 0; j < kBE; ++j) {
-        const int64_t e = base + (int64_t)j * kBT;
-        double rn = 0.0;
-        if (e < N) {
-            x[e] = fma(a, p[e], x[e]);
-            rn = fma(-a, q[e], r[e]);
-            r[e] = rn;
-            if (rb32 && e >= off32) rb32[e - off32] = (float)rn;
+        for (int j = 0; j < kBE; ++j) {
+            const int64_t e = base + (int64_t)j * kBT;
+            if (e < N) { vp[j] = p[e]; vq[j] = q[e]; vx[j] = x[e]; vr[j] = r[e]; }
         }
-        acc[0] = fma(rn, rn, acc[0]);
+#pragma unroll
+        for (int j = 0; j < kBE; ++j) {
+            const int64_t e = base + (int64_t)j * kBT;
+            if (e >= N) continue;
+            x[e] = fma(a, vp[j], vx[j]);
+            const double rn = fma(-a, vq[j], vr[j]);
+            r[e] = rn;
+            if (rb32 && e >= off32) rb32[e - off32] = cvt_f32(rn);
+            acc[0] = fma(rn, rn, acc[0]);
+        }
     }
     bblock_partials<1>(acc, K, part);
 }
@@ -610,7 +646,7 @@ __global__ void k_badd(int64_t N, const XT *__restrict__ x, double *__restrict__
     pdl_begin();
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= N) return;
-    z[e] = assign ? (double)x[e] : z[e] + (double)x[e];
+    z[e] = assign ? cvt<double>(x[e]) : z[e] + cvt<double>(x[e]);
 }
 
 // P = (Z - mu) + beta P per column
@@ -620,7 +656,7 @@ __global__ void k_bupdate_p(int64_t N, int K, const double *__restrict__ sc, con
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= N) return;
     int c = (int)(e & (K - 1));
-    p[e] = (z[e] - sc[B_MU * K + c]) + sc[B_BETA * K + c] * p[e];
+    p[e] = fma(sc[B_BETA * K + c], p[e], z[e] - sc[B_MU * K + c]);
 }
 
 __global__ void k_bsub_mean(int64_t N, int K, double *__restrict__ x, const double *__restrict__ sc, int slot) {
@@ -679,9 +715,9 @@ static void bprecond(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
         VEMG_CHECK_CUDA(cudaEventRecord(h->ev_fork, s));
         VEMG_CHECK_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
         // surface branch: r_c = E~^T r in FP64, one V-cycle on E~^T A E~
-        bcsr<BOP_SPMV, double, double, double, XT, double>(CsrP{h->ET.rp, h->ET.ci, h->ET.v}, h->mtop, nullptr, 0,
-                                                           (const double *)nullptr, (const double *)nullptr, W->R,
-                                                           b0, K, nullptr, -1, h->side, 2);
+        brow<BOP_SPMV, false, double, double, double, XT, double>(W->ET, h->mtop, nullptr, ROW_ALL,
+                                                                  (const double *)nullptr, (const double *)nullptr,
+                                                                  W->R, b0, K, -1, h->side, 2);
         bvcycle<XT, XT>(*W->bsurf, W, 0, 0, (const XT *)b0, x0, h->side);
         VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
         const int64_t nbk = (int64_t)(h->n - mt) * K;
@@ -693,14 +729,15 @@ static void bprecond(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
         VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
         // z = E~ y_s + [0; x_bar]: with FP32 V-cycles formed in FP32 from x_bar on and converted
         // once into the FP64 z; with FP64 ones in FP64
-        if (std::is_same<XT, float>::value && W->Ev32) {
-            bcsr<BOP_SPMV_PLUS, float, XT, XT, double, float>(CsrP{h->E.rp, h->E.ci, W->Ev32}, h->n, nullptr, 0,
-                                                             (const float *)nullptr, (const XT *)xb, x0, W->Z, K,
-                                                             nullptr, mt, s, 2);
+        if constexpr (std::is_same<XT, float>::value) {
+            brow<BOP_SPMV_PLUS, false, float, float, float, double, float>(W->E, h->n, nullptr, ROW_ALL,
+                                                                           (const float *)nullptr, xb, x0, W->Z, K,
+                                                                           mt, s, 1);
         } else {
-            bcsr<BOP_SPMV, double, XT, double, double, double>(CsrP{h->E.rp, h->E.ci, h->E.v}, h->n, nullptr, 0,
-                                                               (const double *)nullptr, (const double *)nullptr, x0,
-                                                               W->Z, K, nullptr, -1, s, 2);
+            brow<BOP_SPMV, false, double, double, double, double, double>(W->E, h->n, nullptr, ROW_ALL,
+                                                                          (const double *)nullptr,
+                                                                          (const double *)nullptr, x0, W->Z, K, -1, s,
+                                                                          2);
             pdl_launch(k_badd<XT>, grid_for(nbk, 256), 256, s, nbk, (const XT *)xb, W->Z + (int64_t)mt * K, 0);
             BATCH_LAUNCHED();
         }
@@ -742,10 +779,10 @@ static void bprecond_any(vemg_hierarchy *h, BatchWork *W, int first, cudaStream_
     const int ns = flex ? 5 : 3;
     if (flex)
         pdl_launch(k_bsums_zrq<5>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
-                   (const double *)W->Q, W->part);
+                   (const double *)W->Q, W->part, 1.0);
     else
         pdl_launch(k_bsums_zrq<3>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
-                   (const double *)nullptr, W->part);
+                   (const double *)nullptr, W->part, 1.0);
     BATCH_LAUNCHED();
     bstage2(h, W, ST_BETA, ns, N, first, s);
 }
@@ -771,8 +808,9 @@ static void bphase_pre(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
 static void bphase_step(vemg_hierarchy *h, BatchWork *W, cudaStream_t s, cudaGraphConditionalHandle hd, int use_cond) {
     const int K = W->K;
     const int64_t N = (int64_t)h->nu * K;
-    bcsr<BOP_SPMV, double, double, double, double, double>(W->Aout, h->nu, nullptr, 0, (const double *)nullptr,
-                                                           (const double *)nullptr, W->P, W->Q, K, nullptr, -1, s, 2);
+    brow<BOP_SPMV, false, double, double, double, double, double>(W->Aout, h->nu, nullptr, ROW_ALL,
+                                                                  (const double *)nullptr, (const double *)nullptr,
+                                                                  W->P, W->Q, K, -1, s, 2);
     {
         BSums d{{W->P}, {W->Q}, 1};
         bsums(W, N, d, s);
@@ -802,8 +840,9 @@ static void bphase_post(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
         BATCH_LAUNCHED();
     }
     // true residual into Q
-    bcsr<BOP_RES, double, double, double, double, double>(W->Aout, h->nu, nullptr, 0, (const double *)nullptr, W->B,
-                                                          W->X, W->Q, K, nullptr, -1, s, 2);
+    brow<BOP_RES, false, double, double, double, double, double>(W->Aout, h->nu, nullptr, ROW_ALL,
+                                                                 (const double *)nullptr, W->B, W->X, W->Q, K, -1, s,
+                                                                 2);
     BSums d{{W->Q}, {W->Q}, 1};
     bsums(W, N, d, s);
     bstage2(h, W, ST_TRUE, 1, N, 0, s);
@@ -906,36 +945,116 @@ static const void *values(Arena &ar, const double *v, int64_t n, bool fp32, cuda
     return f;
 }
 
-static BChain *build_bchain(const Chain &C, bool fp32, Arena &ar, cudaStream_t s) {
-    BChain *B = new BChain();
-    B->nlev = C.nlev;
-    B->direct = C.direct;
-    B->nc = C.nc;
-    B->G = C.G;
-    if (C.direct && fp32) B->Gf = (const float *)values(ar, C.G, (int64_t)C.nc * C.nc, true, s);
-    for (int l = 0; l < C.nlev; ++l) {
-        const Level &L = C.lv[l];
-        BLevel &T = B->lv[l];
-        T.n = L.A.n;
-        T.ncolours = L.ncolours;
-        T.rp = L.A.rp;
-        T.ci = L.A.ci;
-        T.colour = L.colour;
-        T.crow = L.crow;
-        T.cptr = L.cptr;
-        T.v = values(ar, L.A.v, L.A.nnz, fp32, s);
-        void *di = fp32 ? (void *)ar.alloc<float>(L.A.n) : (void *)ar.alloc<double>(L.A.n);
-        k_recip<<<grid_for(L.A.n, 256), 256, 0, s>>>(L.A.n, L.diag, di, fp32);
-        VEMG_CHECK_LAUNCH();
-        T.dinv = di;
-        if (l + 1 < C.nlev) {
-            T.prp = L.P.rp;
-            T.pci = L.P.ci;
-            T.pv = values(ar, L.P.v, L.P.nnz, fp32, s);
-            T.trp = L.PT.rp;
-            T.tci = L.PT.ci;
-            T.tv = values(ar, L.PT.v, L.PT.nnz, fp32, s);
+// A chain operator's copy (BRows). colour: a level's matrix, its diagonal left out and the entries of
+// earlier colours first.
+__global__ void k_brows_fill(int n, const int *__restrict__ rp, const int *__restrict__ ci, const double *__restrict__ v,
+                             const int *__restrict__ colour, int2 *ent, int *oci, double *ov, int *lo) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    const int c0 = colour ? colour[r] : 0;
+    int64_t o = (int64_t)rp[r] - (colour ? r : 0);
+    for (int pass = colour ? 0 : 1; pass < 2; ++pass) {
+        for (int k = rp[r]; k < rp[r + 1]; ++k) {
+            const int j = ci[k];
+            if (colour && (j == r || (colour[j] < c0) != (pass == 0))) continue;
+            if (ent) {
+                ent[o] = make_int2(j, __float_as_int((float)v[k]));
+            } else {
+                oci[o] = j;
+                ov[o] = v[k];
+            }
+            ++o;
         }
+        if (pass == 0) lo[r] = (int)(o - ((int64_t)rp[r] - r));
+    }
+}
+
+__global__ void k_brows_info(int n, const int *__restrict__ crow, const int *__restrict__ rp, const int *__restrict__ lo,
+                             int4 *info) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int r = crow[i];
+    info[i] = make_int4(r, rp[r] - r, lo[r], rp[r + 1] - rp[r] - 1);
+}
+
+// Parts a row is split into: where the rows of one launch do not fill half the chip (152 SMs x 2048
+// threads), a launch lasts as long as a row's chain of loads, which parts of about four entries cut. A
+// warp must hold a row's parts at every launch shape, up to 32 lanes a row; the lanes that the widest
+// loads would take count here, so that the parts (and with them the sums' order) do not depend on the
+// shape.
+static int parts_shift(int K, bool fp32, double rows, double mean) {
+    const double lanes = std::max(1, K / (fp32 ? 4 : 2));
+    int qsh = 0;
+    while (std::min(K, 32) << (qsh + 1) <= 32 && mean > 4.0 * (1 << qsh) && rows * lanes * (2 << qsh) <= 152.0 * 1024.0)
+        ++qsh;
+    return qsh;
+}
+
+static BRows outer_rows(const DCsr &A, const void *v) {
+    BRows R;
+    R.rp = A.rp;
+    R.ci = A.ci;
+    R.v = v;
+    R.mean = (double)A.nnz / std::max(A.n, 1);
+    return R;
+}
+
+static BRows chain_rows(Arena &ar, const DCsr &A, const int *colour, const int *crow, double rows, int K, bool fp32, cudaStream_t s) {
+    BRows R;
+    const int64_t nnz = (int64_t)A.nnz - (colour ? A.n : 0);
+    R.rp = A.rp;
+    R.diag = colour != nullptr;
+    R.mean = (double)nnz / std::max(A.n, 1);
+    R.qsh = parts_shift(K, fp32, rows, R.mean);
+    int2 *ent = fp32 ? ar.alloc<int2>(nnz) : nullptr;
+    int *ci = fp32 ? nullptr : ar.alloc<int>(nnz), *lo = colour ? ar.alloc<int>(A.n) : nullptr;
+    double *v = fp32 ? nullptr : ar.alloc<double>(nnz);
+    if (A.n > 0) {
+        k_brows_fill<<<grid_for(A.n, 128), 128, 0, s>>>(A.n, A.rp, A.ci, A.v, colour, ent, ci, v, lo);
+        VEMG_CHECK_LAUNCH();
+    }
+    R.ent = ent;
+    R.ci = ci;
+    R.v = v;
+    R.lo = lo;
+    if (colour) {
+        int4 *info = ar.alloc<int4>(A.n);
+        if (A.n > 0) {
+            k_brows_info<<<grid_for(A.n, 256), 256, 0, s>>>(A.n, crow, A.rp, lo, info);
+            VEMG_CHECK_LAUNCH();
+        }
+        R.info = info;
+    }
+    return R;
+}
+
+static BChain *build_bchain(const Chain &C, int K, bool fp32, Arena &ar, cudaStream_t s) {
+    BChain *B = new BChain();
+    try {
+        B->nlev = C.nlev;
+        B->direct = C.direct;
+        B->nc = C.nc;
+        B->G = C.G;
+        if (C.direct && fp32) B->Gf = (const float *)values(ar, C.G, (int64_t)C.nc * C.nc, true, s);
+        for (int l = 0; l < C.nlev; ++l) {
+            const Level &L = C.lv[l];
+            BLevel &T = B->lv[l];
+            T.n = L.A.n;
+            T.ncolours = L.ncolours;
+            T.cptr = L.cptr;
+            T.A = chain_rows(ar, L.A, L.colour, L.crow, (double)L.A.n / std::max(L.ncolours, 1), K, fp32, s);
+            void *di = fp32 ? (void *)ar.alloc<float>(L.A.n) : (void *)ar.alloc<double>(L.A.n);
+            k_recip<<<grid_for(L.A.n, 256), 256, 0, s>>>(L.A.n, L.diag, di, fp32);
+            VEMG_CHECK_LAUNCH();
+            T.dinv = di;
+            if (l + 1 < C.nlev) {
+                T.P = chain_rows(ar, L.P, nullptr, nullptr, L.A.n, K, fp32, s);
+                T.PT = chain_rows(ar, L.PT, nullptr, nullptr, C.lv[l + 1].A.n, K, fp32, s);
+            }
+        }
+    } catch (...) {
+        delete B;
+        throw;
     }
     return B;
 }
@@ -968,7 +1087,6 @@ static void autotune_t(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     int cbig = 0;
     for (int c = 1; c < L.ncolours; ++c)
         if (L.cptr[c + 1] - L.cptr[c] > L.cptr[cbig + 1] - L.cptr[cbig]) cbig = c;
-    const CsrP A{L.rp, L.ci, L.v};
     cudaEvent_t e0, e1;
     VEMG_CHECK_CUDA(cudaEventCreate(&e0));
     VEMG_CHECK_CUDA(cudaEventCreate(&e1));
@@ -982,16 +1100,17 @@ static void autotune_t(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
                 for (int wp : {2, 4, 8}) {
                     auto run = [&]() {
                         if (cls == 0)
-                            bcsr<BOP_SOR, XT, XT, XT, XT, XT>(A, L.cptr[cbig + 1] - L.cptr[cbig], L.crow + L.cptr[cbig], 0,
-                                                               (const XT *)L.dinv, lb, lx, lx, K, L.colour, -1, s, 0,
-                                                               kw, wp);
+                            brow<BOP_SOR, packed<XT>(), XT, XT, XT, XT, XT>(
+                                L.A, L.cptr[cbig + 1] - L.cptr[cbig], L.A.info + L.cptr[cbig], ROW_ALL,
+                                (const XT *)L.dinv, lb, lx, lx, K, -1, s, 0, kw, wp);
                         else if (cls == 1)
-                            bcsr<BOP_RES, XT, XT, XT, XT, XT>(A, L.n, nullptr, 0, (const XT *)nullptr, lb, lx, lr, K,
-                                                               nullptr, -1, s, 1, kw, wp);
+                            brow<BOP_UPPER, packed<XT>(), XT, XT, XT, XT, XT>(L.A, L.n, nullptr, ROW_UPPER,
+                                                                             (const XT *)nullptr, lb, lx, lr, K, -1,
+                                                                             s, 1, kw, wp);
                         else
-                            bcsr<BOP_SPMV, double, double, double, double, double>(
-                                W->Aout, h->nu, nullptr, 0, (const double *)nullptr, (const double *)nullptr, W->P,
-                                W->Q, K, nullptr, -1, s, 2, kw, wp);
+                            brow<BOP_SPMV, false, double, double, double, double, double>(
+                                W->Aout, h->nu, nullptr, ROW_ALL, (const double *)nullptr, (const double *)nullptr,
+                                W->P, W->Q, K, -1, s, 2, kw, wp);
                     };
                     run();
                     VEMG_CHECK_CUDA(cudaEventRecord(e0, s));
@@ -1045,14 +1164,14 @@ BatchWork *new_batch_work(vemg_hierarchy *h, int K, cudaStream_t s) {
     const bool fp32 = h->precision != VEMG_PREC_FP64;
     size_t es = fp32 ? sizeof(float) : sizeof(double);
     const Chain *chains[2] = {&h->surf, single_chain(h) ? &the_chain(h) : &h->bar};
-    if (!single_chain(h)) W->bsurf = build_bchain(h->surf, fp32, ar, s);
-    W->bbar = build_bchain(*chains[1], fp32, ar, s);
+    if (!single_chain(h)) W->bsurf = build_bchain(h->surf, K, fp32, ar, s);
+    W->bbar = build_bchain(*chains[1], K, fp32, ar, s);
     if (h->bc == VEMG_NEUMANN) {
-        W->Aout = CsrP{h->A.rp, h->A.ci, h->A.v};
+        W->Aout = outer_rows(h->A, h->A.v);
         W->caller_of = h->new2old;
     } else {
         const DCsr &A0 = h->bar.lv[0].A;
-        W->Aout = CsrP{A0.rp, A0.ci, A0.v};
+        W->Aout = outer_rows(A0, A0.v);
         W->caller_of = h->new2old + h->mtop;
     }
     for (int ch = 0; ch < 2; ++ch)
@@ -1062,11 +1181,10 @@ BatchWork *new_batch_work(vemg_hierarchy *h, int K, cudaStream_t s) {
             W->lb[ch][l] = ar.alloc<char>((int64_t)es * m);
             W->lr[ch][l] = ar.alloc<char>((int64_t)es * m);
         }
-    if (fp32 && !single_chain(h)) {
-        W->Ev32 = ar.alloc<float>(h->E.nnz);
-        k_bto_float<<<grid_for(h->E.nnz, 256), 256, 0, s>>>(h->E.nnz, (const double *)h->E.v, W->Ev32);
-        VEMG_CHECK_LAUNCH();
-        W->Rb32 = ar.alloc<float>((int64_t)(h->n - h->mtop) * K);
+    if (!single_chain(h)) {
+        W->ET = outer_rows(h->ET, h->ET.v);
+        W->E = outer_rows(h->E, values(ar, h->E.v, h->E.nnz, fp32, s));
+        if (fp32) W->Rb32 = ar.alloc<float>((int64_t)(h->n - h->mtop) * K);
     }
     W->sc = ar.alloc<double>(B_COUNT * K + G_COUNT);
     W->part = ar.alloc<double>((int64_t)5 * stage1_blocks(N) * K);

@@ -22,31 +22,29 @@ __global__ void k_inverse_perm(int n, const int *__restrict__ s2n, int *n2s) {
     if (i < n) n2s[s2n[i]] = i;
 }
 
+// steps of each slice (one warp per slice) and the elements they take
 __global__ void k_sell_width(int nslices, const int *__restrict__ row0, const int *__restrict__ nrow,
                              const int *__restrict__ s2n, const int *__restrict__ rp, int split, int lsh, int *width,
-                             int *longest) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
+                             int *elements, int *longest) {
+    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (s >= nslices) return;
-    int w = 0;
-    for (int l = 0; l < nrow[s]; ++l) {
-        int r = row0[s] + l;
-        int i = s2n ? s2n[r] : r;
-        w = max(w, rp[i + 1] - rp[i] - split);
+    unsigned len = 0;
+    if (lane < nrow[s]) {
+        const int r = row0[s] + lane, i = s2n ? s2n[r] : r;
+        len = (unsigned)max(rp[i + 1] - rp[i] - split, 0);
     }
-    width[s] = (max(w, 0) + (1 << lsh) - 1) >> lsh;
+    const int w = (int)__reduce_max_sync(0xffffffffu, len);
+    if (lane != 0) return;
+    width[s] = (w + (1 << lsh) - 1) >> lsh;
+    elements[s] = 32 * width[s];
     if (w > 0xffff) atomicMax(longest, w);
-}
-
-__global__ void k_scale32(int n, const int *__restrict__ w, int *o) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) o[i] = 32 * w[i];
 }
 
 template <class VT>
 __global__ void k_sell_fill(int nslices, const int *__restrict__ row0, const int *__restrict__ nrow,
                             const int *__restrict__ off, const int *__restrict__ width, const int *__restrict__ s2n,
                             const int *__restrict__ n2s, const int *__restrict__ rp, const int *__restrict__ ci,
-                            const double *__restrict__ v, int *col, VT *val) {
+                            const double *__restrict__ v, int *col, VT *val, unsigned long long *cnt) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int s = (int)(t / 32), lane = (int)(t % 32);
     if (s >= nslices) return;
@@ -62,6 +60,8 @@ __global__ void k_sell_fill(int nslices, const int *__restrict__ row0, const int
             ++k;
         }
     }
+    const unsigned entries = __reduce_add_sync(0xffffffffu, (unsigned)k);
+    if (lane == 0) atomicAdd(cnt + 1, (unsigned long long)entries);   // one group
     for (; k < w; ++k) {
         col[o + 32 * k] = 0;
         val[o + 32 * k] = (VT)0;
@@ -71,13 +71,13 @@ __global__ void k_sell_fill(int nslices, const int *__restrict__ row0, const int
 // The chains' form (sell.cuh): the first thread of each row walks the row and deals its entries to
 // the row's lanes. split: the diagonal apart, the entries of earlier colours first (columns below
 // the row's own: a row has no entry in its own colour but the diagonal). Unused places hold zeros.
-// low: entries of earlier colours per colour of the rows (colour of a slice: gcol).
+// cnt: entries per group of the rows (group of a slice: gcol), of earlier colours and all.
 template <class VT>
 __global__ void k_sell_deal(int nslices, int lsh, const int *__restrict__ row0, const int *__restrict__ nrow,
                             const int *__restrict__ off, const int *__restrict__ width, const int *__restrict__ s2n,
                             const int *__restrict__ n2s, const int *__restrict__ rp, const int *__restrict__ ci,
                             const double *__restrict__ v, int split, int *col, VT *val, VT *dinv, int4 *meta,
-                            unsigned *rl, int rl_wide, const int *__restrict__ gcol, unsigned long long *low) {
+                            unsigned *rl, int rl_wide, const int *__restrict__ gcol, unsigned long long *cnt) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int s = (int)(t / 32), lane = (int)(t % 32);
     if (s >= nslices) return;
@@ -88,10 +88,9 @@ __global__ void k_sell_deal(int nslices, int lsh, const int *__restrict__ row0, 
         val[o + 32 * k + lane] = (VT)0;
     }
     __syncwarp();
-    unsigned nlow = 0;
+    unsigned nlow = 0, k = 0;
     if (lane < nrow[s] && lane < rows) {
         const int r = row0[s] + lane, i = s2n ? s2n[r] : r;
-        unsigned k = 0;
         for (int pass = split ? 0 : 1; pass < 2; ++pass) {
             for (int e = rp[i]; e < rp[i + 1]; ++e) {
                 const int c = ci[e];
@@ -115,9 +114,11 @@ __global__ void k_sell_deal(int nslices, int lsh, const int *__restrict__ row0, 
             rl[r] = nlow | k << 16;
         }
     }
-    if (!split) return;
     nlow = __reduce_add_sync(0xffffffffu, nlow);
-    if (lane == 0) atomicAdd(low + gcol[s], (unsigned long long)nlow);
+    k = __reduce_add_sync(0xffffffffu, k);
+    if (lane != 0) return;
+    if (nlow) atomicAdd(cnt + 2 * gcol[s], (unsigned long long)nlow);
+    atomicAdd(cnt + 2 * gcol[s] + 1, (unsigned long long)k);
 }
 
 // Lanes per row of a chain's operator, by the rows that one launch works on and their mean length.
@@ -130,21 +131,21 @@ static int lanes_shift(double rows, double mean) {
     return lsh;
 }
 
-static int scan_i32(const int *in, int *out, int n, cudaStream_t s) {
-    // small host-side scan (slice tables have at most a few hundred thousand entries)
-    std::vector<int> h(n), o(n + 1);
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(h.data(), in, sizeof(int) * n, cudaMemcpyDeviceToHost, s));
-    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    int64_t acc = 0;
-    for (int i = 0; i < n; ++i) {
-        o[i] = (int)acc;
-        acc += h[i];
+// slice s of the groups (group g: slices gs[g] .. gs[g + 1], rows from gr[g])
+__global__ void k_slices(int nslices, int ngroups, const int *__restrict__ gr, const int *__restrict__ gs, int rows,
+                         int *row0, int *nrow, int *gcol) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= nslices) return;
+    int lo = 0, hi = ngroups;   // the last group whose first slice is at most s (an empty group has none)
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (gs[mid] <= s) lo = mid;
+        else hi = mid;
     }
-    if (acc > 0x7fffffffLL) throw Error{VEMG_EINTERNAL};
-    o[n] = (int)acc;
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(out, o.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
-    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    return (int)acc;
+    const int r = gr[lo] + (s - gs[lo]) * rows;
+    row0[s] = r;
+    nrow[s] = min(rows, gr[lo + 1] - r);
+    gcol[s] = lo;
 }
 
 // Build the sliced ELL of the rows s2n[0..n) of the CSR matrix A (natural order), columns mapped
@@ -153,7 +154,8 @@ static int scan_i32(const int *in, int *out, int n, cudaStream_t s) {
 // else a chain's, with 1 << lsh lanes per row.
 static Sell build_sell(Arena &ar, const DCsr &A, int n, const int *s2n, const int *n2s, int ncols,
                        const std::vector<int> &groups, bool fp32, void **dinv, std::vector<int> *gslice,
-                       cudaStream_t s, int lsh = -1, std::vector<int64_t> *low = nullptr) {
+                       cudaStream_t s, int lsh = -1, std::vector<int64_t> *low = nullptr,
+                       std::vector<int64_t> *all = nullptr) {
     const bool split = dinv != nullptr;
     Sell S;
     S.n = n;
@@ -161,39 +163,33 @@ static Sell build_sell(Arena &ar, const DCsr &A, int n, const int *s2n, const in
     S.fp32 = fp32;
     S.lsh = lsh < 0 ? 0 : lsh;
     const int rows = 32 >> S.lsh;
-    std::vector<int> row0, nrow, gcol;
-    if (gslice) gslice->assign(1, 0);
-    for (size_t g = 0; g + 1 < groups.size(); ++g) {
-        for (int r = groups[g]; r < groups[g + 1]; r += rows) {
-            row0.push_back(r);
-            nrow.push_back(std::min(rows, groups[g + 1] - r));
-            gcol.push_back((int)g);
-        }
-        if (gslice) gslice->push_back((int)row0.size());
+    const int ngroups = std::max((int)groups.size() - 1, 0);
+    std::vector<int> table(2 * (size_t)(ngroups + 1), 0);   // first row, first slice of each group
+    for (int g = 0; g <= ngroups && !groups.empty(); ++g) {
+        table[g] = groups[g];
+        if (g > 0) table[ngroups + 1 + g] = table[ngroups + g] + (groups[g] - groups[g - 1] + rows - 1) / rows;
     }
-    S.nslices = (int)row0.size();
+    if (gslice) gslice->assign(table.begin() + ngroups + 1, table.end());
+    S.nslices = table.back();
     S.row0 = ar.alloc<int>(S.nslices);
     S.nrow = ar.alloc<int>(S.nslices);
     S.width = ar.alloc<int>(S.nslices);
     S.off = ar.alloc<int>(S.nslices + 1);
-    int longest = 0;
+    int longest = 0, total = 0;
+    Scratch<int> gtab((int64_t)table.size()), gcol(S.nslices);
     if (S.nslices) {
-        Scratch<int> lg(1);
+        Scratch<int> lg(1), w32(S.nslices);
         VEMG_CHECK_CUDA(cudaMemsetAsync(lg, 0, sizeof(int), s));
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(S.row0, row0.data(), sizeof(int) * S.nslices, cudaMemcpyHostToDevice, s));
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(S.nrow, nrow.data(), sizeof(int) * S.nslices, cudaMemcpyHostToDevice, s));
-        k_sell_width<<<grid_for(S.nslices, 128), 128, 0, s>>>(S.nslices, S.row0, S.nrow, s2n, A.rp, split ? 1 : 0,
-                                                              S.lsh, S.width, lg);
+        VEMG_CHECK_CUDA(cudaMemcpyAsync(gtab, table.data(), sizeof(int) * table.size(), cudaMemcpyHostToDevice, s));
+        k_slices<<<grid_for(S.nslices, 256), 256, 0, s>>>(S.nslices, ngroups, gtab, gtab.p + ngroups + 1, rows, S.row0,
+                                                          S.nrow, gcol);
+        VEMG_CHECK_LAUNCH();
+        k_sell_width<<<grid_for((int64_t)S.nslices * 32, 256), 256, 0, s>>>(S.nslices, S.row0, S.nrow, s2n, A.rp,
+                                                                            split ? 1 : 0, S.lsh, S.width, w32, lg);
         VEMG_CHECK_LAUNCH();
         VEMG_CHECK_CUDA(cudaMemcpyAsync(&longest, lg.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
+        total = scan_offsets(w32, S.off, S.nslices, s);   // synchronises
     }
-    Scratch<int> w32(S.nslices + 1);
-    if (S.nslices) {
-        k_scale32<<<grid_for(S.nslices, 256), 256, 0, s>>>(S.nslices, S.width, w32);
-        VEMG_CHECK_LAUNCH();
-    }
-    int total = scan_i32(w32, S.off, S.nslices, s);
     S.padded = total;
     S.col = ar.alloc<int>(total);
     if (fp32) S.v = ar.alloc<float>(total);
@@ -204,53 +200,44 @@ static Sell build_sell(Arena &ar, const DCsr &A, int n, const int *s2n, const in
         else di = ar.alloc<double>(n);
         *dinv = di;
     }
-    const int ngroups = (int)groups.size() - 1;
-    if (low) low->assign(std::max(ngroups, 0), 0);
     if (lsh >= 0) {
         S.rl_wide = longest > 0xffff;
         S.meta = ar.alloc<int4>(S.nslices);
         S.rl = ar.alloc<unsigned>((int64_t)n * (S.rl_wide ? 2 : 1));
     }
-    if (S.nslices && lsh >= 0) {
-        Scratch<int> gc(S.nslices);
-        Scratch<unsigned long long> lo(std::max(ngroups, 1));
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(gc, gcol.data(), sizeof(int) * S.nslices, cudaMemcpyHostToDevice, s));
-        VEMG_CHECK_CUDA(cudaMemsetAsync(lo, 0, sizeof(unsigned long long) * std::max(ngroups, 1), s));
+    // entries of each group: of earlier colours, and all
+    std::vector<unsigned long long> count(2 * (size_t)std::max(ngroups, 1), 0ull);
+    if (S.nslices) {
+        Scratch<unsigned long long> cnt((int64_t)count.size());
+        VEMG_CHECK_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * count.size(), s));
         const int grid = grid_for((int64_t)S.nslices * 32, 256);
-        if (fp32)
-            k_sell_deal<float><<<grid, 256, 0, s>>>(S.nslices, S.lsh, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp,
-                                                    A.ci, A.v, split, S.col, (float *)S.v, (float *)di,
-                                                    S.meta, S.rl, S.rl_wide, gc, lo);
-        else
-            k_sell_deal<double><<<grid, 256, 0, s>>>(S.nslices, S.lsh, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp,
-                                                     A.ci, A.v, split, S.col, (double *)S.v,
-                                                     (double *)di, S.meta, S.rl, S.rl_wide, gc, lo);
+        auto fill = [&](auto *v) {
+            using VT = std::remove_pointer_t<decltype(v)>;
+            if (lsh >= 0)
+                k_sell_deal<VT><<<grid, 256, 0, s>>>(S.nslices, S.lsh, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp,
+                                                     A.ci, A.v, split, S.col, v, (VT *)di, S.meta, S.rl, S.rl_wide,
+                                                     gcol, cnt);
+            else
+                k_sell_fill<VT><<<grid, 256, 0, s>>>(S.nslices, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp, A.ci,
+                                                     A.v, S.col, v, cnt);
+        };
+        if (fp32) fill((float *)S.v);
+        else fill((double *)S.v);
         VEMG_CHECK_LAUNCH();
-        std::vector<unsigned long long> hl(std::max(ngroups, 1));
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(hl.data(), lo.p, sizeof(unsigned long long) * hl.size(), cudaMemcpyDeviceToHost, s));
+        VEMG_CHECK_CUDA(cudaMemcpyAsync(count.data(), cnt.p, sizeof(unsigned long long) * count.size(),
+                                        cudaMemcpyDeviceToHost, s));
         VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-        if (low)
-            for (int g = 0; g < ngroups; ++g) (*low)[g] = (int64_t)hl[g];
-    } else if (S.nslices) {
-        const int grid = grid_for((int64_t)S.nslices * 32, 256);
-        if (fp32)
-            k_sell_fill<float><<<grid, 256, 0, s>>>(S.nslices, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp, A.ci,
-                                                    A.v, S.col, (float *)S.v);
-        else
-            k_sell_fill<double><<<grid, 256, 0, s>>>(S.nslices, S.row0, S.nrow, S.off, S.width, s2n, n2s, A.rp, A.ci,
-                                                     A.v, S.col, (double *)S.v);
-        VEMG_CHECK_LAUNCH();
     }
-    // stored entries (rows of s2n)
-    std::vector<int> hrp(A.n + 1);
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(hrp.data(), A.rp, sizeof(int) * (A.n + 1), cudaMemcpyDeviceToHost, s));
-    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    if (s2n) {
-        std::vector<int> hs(n);
-        VEMG_CHECK_CUDA(cudaMemcpy(hs.data(), s2n, sizeof(int) * n, cudaMemcpyDeviceToHost));
-        for (int r = 0; r < n; ++r) S.nnz += hrp[hs[r] + 1] - hrp[hs[r]] - (split ? 1 : 0);
-    } else {
-        S.nnz = (int64_t)hrp[n] - (split ? n : 0);
+    if (low) {
+        low->resize(ngroups);
+        all->resize(ngroups);
+    }
+    for (int g = 0; g < ngroups; ++g) {
+        S.nnz += (int64_t)count[2 * g + 1];
+        if (low) {
+            (*low)[g] = (int64_t)count[2 * g];
+            (*all)[g] = (int64_t)count[2 * g + 1];
+        }
     }
     return S;
 }
@@ -313,11 +300,9 @@ static void layout_chain(Arena &ar, const Chain &C, SChain &S, bool fp32, cudaSt
         T.n = L.A.n;
         T.ncolours = L.ncolours;
         T.crow = L.cptr;
-        T.cnnz.resize(L.ncolours);
-        for (int c = 0; c < L.ncolours; ++c) T.cnnz[c] = L.cnnz[c] - (L.cptr[c + 1] - L.cptr[c]);
         T.A = build_sell(ar, L.A, L.A.n, L.crow, inv[l], L.A.n, L.cptr, fp32, &T.dinv, &T.cslice, s,
                          lanes_shift((double)L.A.n / std::max(L.ncolours, 1), (double)L.A.nnz / std::max(L.A.n, 1) - 1.0),
-                         &T.clow);
+                         &T.clow, &T.cnnz);
         if (l + 1 < C.nlev) {
             const Level &N = C.lv[l + 1];
             T.P = build_sell(ar, L.P, L.A.n, L.crow, inv[l + 1], N.A.n, {0, L.A.n}, fp32, nullptr, nullptr, s,

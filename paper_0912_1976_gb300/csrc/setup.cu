@@ -100,6 +100,10 @@ static void scan64_inplace(int64_t *data, int64_t n, cudaStream_t s) {
     }
 }
 
+__global__ void k_scan_total(const int *__restrict__ in, int64_t *__restrict__ out, int64_t n) {
+    out[n] = n > 0 ? out[n - 1] + in[n - 1] : 0;
+}
+
 // out64[0..n] = exclusive scan of in[0..n-1], out64[n] = total. Returns the total.
 static int64_t scan_to64(const int *in, int64_t *out64, int64_t n, cudaStream_t s) {
     int64_t nb = (n + 1023) / 1024;
@@ -113,15 +117,10 @@ static int64_t scan_to64(const int *in, int64_t *out64, int64_t n, cudaStream_t 
             VEMG_CHECK_LAUNCH();
         }
     }
-    int64_t last_off = 0, total = 0;
-    int last_in = 0;
-    if (n > 0) {
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(&last_off, out64 + n - 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(&last_in, in + n - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-        VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-        total = last_off + last_in;
-    }
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(out64 + n, &total, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    int64_t total = 0;
+    k_scan_total<<<1, 1, 0, s>>>(in, out64, n);
+    VEMG_CHECK_LAUNCH();
+    VEMG_CHECK_CUDA(cudaMemcpyAsync(&total, out64 + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     return total;
 }
@@ -132,7 +131,7 @@ __global__ void k_narrow(const int64_t *__restrict__ in, int *__restrict__ out, 
 }
 
 // out[0..n] = exclusive scan of counts (int32 offsets); throws if the total needs 64 bits
-static int scan_offsets(const int *counts, int *out, int64_t n, cudaStream_t s) {
+int scan_offsets(const int *counts, int *out, int64_t n, cudaStream_t s) {
     Scratch<int64_t> t(n + 1);
     int64_t total = scan_to64(counts, t, n, s);
     if (total > 0x7fffffffLL) throw Error{VEMG_EINTERNAL};
@@ -468,6 +467,13 @@ void load_vector(const vemg_mesh *mesh, const double *f, double *b, cudaStream_t
 // ------------------------------------------------------------------------------------------
 // generic CSR operations
 
+// temporary arrays, released at scope exit
+struct TempArena : Arena {
+    TempArena() { temporary = true; }
+    ~TempArena() { release(); }
+    TempArena(const TempArena &) = delete;
+};
+
 static DCsr csr_alloc(Arena &ar, int n, int m, int nnz) {
     DCsr a;
     a.n = n;
@@ -613,13 +619,12 @@ __global__ void k_mirror_upper(int n, const int *__restrict__ rp, const int *__r
 
 // Galerkin product P^T (A P), then exact symmetrisation (section 5.1, Eq. reduced AMG)
 static DCsr galerkin(Arena &ar, const DCsr &A, const DCsr &P, const DCsr &PT, cudaStream_t s) {
-    Arena tmp;
+    TempArena tmp;
     DCsr AP = csr_spgemm(tmp, A, P, s);
     DCsr C = csr_spgemm(ar, PT, AP, s);
     k_mirror_upper<<<grid_for(C.n, 128), 128, 0, s>>>(C.n, C.rp, C.ci, C.v);
     VEMG_CHECK_LAUNCH();
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    tmp.release();
     return C;
 }
 
@@ -1266,7 +1271,7 @@ static DCsr csr_spgemm(Arena &ar, const DCsr &L, const DCsr &R, cudaStream_t s);
 // coarsening stops here).
 static int coarsen_linear(Arena &ar, Level &L, Level &N, double theta, double omega, cudaStream_t s) {
     const int n = L.A.n;
-    Arena tmp;
+    TempArena tmp;
     int nagg = 0;
     int *bagg = nullptr;
     Scratch<int> err(1);
@@ -1295,10 +1300,7 @@ static int coarsen_linear(Arena &ar, Level &L, Level &N, double theta, double om
         VEMG_CHECK_LAUNCH();
         nagg = sa_aggregate(tmp, L.A, d, theta, true, &bagg, s);
     }
-    if (nagg == 0) {
-        tmp.release();
-        return 0;
-    }
+    if (nagg == 0) return 0;
     int *agg = ar.alloc<int>(n);
     k_map_blocks<<<grid_for(n, 256), 256, 0, s>>>(n, L.blk, bagg, agg);
     VEMG_CHECK_LAUNCH();
@@ -1320,10 +1322,7 @@ static int coarsen_linear(Arena &ar, Level &L, Level &N, double theta, double om
     VEMG_CHECK_LAUNCH();
     Scratch<int64_t> col0(nagg + 1);
     const int64_t nc64 = scan_to64(kept, col0, nagg, s);
-    if (nc64 == 0 || nc64 * 10 > (int64_t)n * 9) {
-        tmp.release();
-        return 0;
-    }
+    if (nc64 == 0 || nc64 * 10 > (int64_t)n * 9) return 0;
     const int nc = (int)nc64;
     DCsr Pt;
     Pt.n = n;
@@ -1352,7 +1351,6 @@ static int coarsen_linear(Arena &ar, Level &L, Level &N, double theta, double om
     VEMG_CHECK_LAUNCH();
     L.agg = agg;
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    tmp.release();
     return nc;
 }
 
@@ -1385,7 +1383,8 @@ __global__ void k_offdiag_degree(int n, const int *__restrict__ rp, const int *_
 
 // The rounds work on worklists: a round touches only the nodes it handles and their
 // neighbours, so that a round costs about one small kernel launch (the peeling needs thousands
-// of rounds on the finest levels).
+// of rounds on the finest levels); each is launched while the one before it runs (programmatic
+// dependent launch).
 static constexpr int kRoundBlocks = 152, kRoundThreads = 256;
 static constexpr int kRing = 64;   // worklist sizes of the rounds, kept in a ring (> kRoundBatch + 2)
 
@@ -1401,6 +1400,7 @@ __global__ void __launch_bounds__(kRoundThreads) k_peel_round(const int *__restr
                                                              int *nring, const int *__restrict__ rp,
                                                              const int *__restrict__ ci, int *rank, int *deg, int k,
                                                              int round, int *removed) {
+    pdl_begin();
     const int cnt = nring[round % kRing];
     int *n_out = nring + (round + 1) % kRing;
     if (blockIdx.x == 0 && threadIdx.x == 0) nring[(round + 2) % kRing] = 0;
@@ -1458,6 +1458,7 @@ __global__ void __launch_bounds__(kRoundThreads) k_jp_round(const int *__restric
                                                            int round, const int *__restrict__ rp,
                                                            const int *__restrict__ ci, const int *__restrict__ rank,
                                                            int *pc, int *colour, int *maxc) {
+    pdl_begin();
     const int cnt = nring[round % kRing];
     int *n_out = nring + (round + 1) % kRing;
     if (blockIdx.x == 0 && threadIdx.x == 0) nring[(round + 2) % kRing] = 0;
@@ -1466,10 +1467,14 @@ __global__ void __launch_bounds__(kRoundThreads) k_jp_round(const int *__restric
     for (int q = w0; q < cnt; q += nw) {
         const int v = wl_in[q];
         const int lo = rp[v], hi = rp[v + 1];
+        // the lane's first neighbour stays in registers for the second walk of the row
+        const int j0 = lo + lane < hi ? ci[lo + lane] : v;
+        const int c0 = j0 != v ? colour[j0] : -1, r0 = j0 != v ? rank[j0] : 0, rv = rank[v];
         int col = -1;
         for (int base = 0; col < 0; base += 64) {
             unsigned long long used = 0ull;
-            for (int e = lo + lane; e < hi; e += 32) {
+            if (c0 - base >= 0 && c0 - base < 64) used = 1ull << (c0 - base);
+            for (int e = lo + lane + 32; e < hi; e += 32) {
                 int j = ci[e];
                 int c = j != v ? colour[j] - base : -1;
                 if (c >= 0 && c < 64) used |= 1ull << c;
@@ -1481,25 +1486,37 @@ __global__ void __launch_bounds__(kRoundThreads) k_jp_round(const int *__restric
         }
         if (lane == 0) {
             colour[v] = col;
-            atomicMax(maxc, col);
+            if (col > *(volatile int *)maxc) atomicMax(maxc, col);
         }
-        const uint64_t kv = colour_key(rank[v], v);
-        for (int e = lo + lane; e < hi; e += 32) {
+        const uint64_t kv = colour_key(rv, v);
+        if (j0 != v && colour_key(r0, j0) < kv && atomicSub(pc + j0, 1) == 1) push(wl_out, n_out, j0);
+        for (int e = lo + lane + 32; e < hi; e += 32) {
             int j = ci[e];
             if (j != v && colour_key(rank[j], j) < kv && atomicSub(pc + j, 1) == 1) push(wl_out, n_out, j);
         }
     }
 }
 
-__global__ void k_eq_flag(int n, const int *__restrict__ key, int c, int *flag) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = key[i] == c;
-}
+// Rows grouped by colour, ascending within a colour: a counting sort. A warp takes kGroupRows
+// consecutive rows; count c * nw + w is warp w's rows of colour c, so that the exclusive scan of the
+// counts is where each warp puts them.
+static constexpr int kGroupRows = 1024;
 
-__global__ void k_scatter_flagged(int n, const int *__restrict__ flag, const int *__restrict__ off, int base,
-                                  int *out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && flag[i]) out[base + off[i]] = i;
+template <bool SCATTER>
+__global__ void k_group(int n, int nw, const int *__restrict__ colour, int *cnt, int *out) {
+    const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (w >= nw) return;
+    for (int i0 = w * kGroupRows; i0 < (w + 1) * kGroupRows && i0 < n; i0 += 32) {
+        const int i = i0 + lane, c = i < n ? colour[i] : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, c);
+        const int lead = __ffs((int)same) - 1, before = __popc(same & ((1u << lane) - 1u));
+        int *place = cnt + (int64_t)c * nw + w;   // one leader per colour: no other lane or warp touches it
+        int at = c >= 0 && lane == lead ? __ldcg(place) : 0;
+        at = __shfl_sync(0xffffffffu, at, lead);
+        if (SCATTER && c >= 0) out[at + before] = i;
+        if (c >= 0 && lane == lead) __stcg(place, at + __popc(same));
+        __syncwarp();
+    }
 }
 
 static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
@@ -1531,9 +1548,8 @@ static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
             VEMG_CHECK_LAUNCH();
         }
         for (int u = 0; u < kRoundBatch; ++u, ++t)
-            k_peel_round<<<kRoundBlocks, kRoundThreads, 0, s>>>(wl[t & 1], wl[(t + 1) & 1], nring, L.A.rp, L.A.ci,
-                                                                rank, deg, k, t, removed);
-        VEMG_CHECK_LAUNCH();
+            pdl_launch(k_peel_round, kRoundBlocks, kRoundThreads, s, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p,
+                       (const int *)L.A.rp, (const int *)L.A.ci, rank.p, deg.p, k, t, removed.p);
     }
     // colouring in decreasing key order: Jones-Plassmann rounds on predecessor counts
     if (n > 0) {
@@ -1545,34 +1561,25 @@ static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
     for (int64_t batches = 0; n > 0; ++batches) {
         if (batches > (int64_t)n + 64) throw Error{VEMG_EINTERNAL};   // every batch colours a node
         for (int u = 0; u < kRoundBatch; ++u, ++t)
-            k_jp_round<<<kRoundBlocks, kRoundThreads, 0, s>>>(wl[t & 1], wl[(t + 1) & 1], nring, t, L.A.rp, L.A.ci,
-                                                              rank, pc, L.colour, maxc);
-        VEMG_CHECK_LAUNCH();
+            pdl_launch(k_jp_round, kRoundBlocks, kRoundThreads, s, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p, t,
+                       (const int *)L.A.rp, (const int *)L.A.ci, (const int *)rank.p, pc.p, L.colour, maxc.p);
         if (read_int(nring + t % kRing, s) == 0) break;   // every node coloured
     }
     L.ncolours = n > 0 ? read_int(maxc, s) + 1 : 0;
     L.crow = ar.alloc<int>(n);
-    L.cptr.assign(L.ncolours + 1, 0);
-    Scratch<int> flag(n), off(n + 1);
-    int base = 0;
-    for (int c = 0; c < L.ncolours; ++c) {
-        k_eq_flag<<<grid_for(n, 256), 256, 0, s>>>(n, L.colour, c, flag);
-        VEMG_CHECK_LAUNCH();
-        int cnt = scan_offsets(flag, off, n, s);
-        k_scatter_flagged<<<grid_for(n, 256), 256, 0, s>>>(n, flag, off, base, L.crow);
-        VEMG_CHECK_LAUNCH();
-        L.cptr[c] = base;
-        base += cnt;
-    }
-    L.cptr[L.ncolours] = base;
-    // entries per colour (for the algorithmic byte count of each sweep launch)
-    std::vector<int> hrp(n + 1), hrow(n);
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(hrp.data(), L.A.rp, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost, s));
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(hrow.data(), L.crow, sizeof(int) * n, cudaMemcpyDeviceToHost, s));
+    L.cptr.assign(L.ncolours + 1, n);
+    if (n == 0) return;
+    const int nw = (n + kGroupRows - 1) / kGroupRows, nc = L.ncolours;
+    Scratch<int> cnt((int64_t)nc * nw), off((int64_t)nc * nw + 1);
+    VEMG_CHECK_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)nc * nw, s));
+    k_group<false><<<grid_for((int64_t)nw * 32, 128), 128, 0, s>>>(n, nw, L.colour, cnt, nullptr);
+    VEMG_CHECK_LAUNCH();
+    scan_offsets(cnt, off, (int64_t)nc * nw, s);
+    VEMG_CHECK_CUDA(cudaMemcpy2DAsync(L.cptr.data(), sizeof(int), off.p, sizeof(int) * (size_t)nw, sizeof(int), nc,
+                                      cudaMemcpyDeviceToHost, s));
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    L.cnnz.assign(L.ncolours, 0);
-    for (int c = 0; c < L.ncolours; ++c)
-        for (int k = L.cptr[c]; k < L.cptr[c + 1]; ++k) L.cnnz[c] += hrp[hrow[k] + 1] - hrp[hrow[k]];
+    k_group<true><<<grid_for((int64_t)nw * 32, 128), 128, 0, s>>>(n, nw, L.colour, off, L.crow);
+    VEMG_CHECK_LAUNCH();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1688,15 +1695,9 @@ static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_
         k_diag<<<grid_for(n, 256), 256, 0, s>>>(n, L.A.rp, L.A.ci, L.A.v, d);
         VEMG_CHECK_LAUNCH();
         int *agg = nullptr;
-        Arena tmp;
-        int nagg = sa_aggregate(tmp, L.A, d, o.strength, singular, &agg, s);
-        if (nagg == 0 || (int64_t)nagg * 10 > (int64_t)n * 9) {
-            tmp.release();
-            break;
-        }
-        L.agg = ar.alloc<int>(n);
-        VEMG_CHECK_CUDA(cudaMemcpyAsync(L.agg, agg, sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
-        tmp.release();
+        int nagg = sa_aggregate(ar, L.A, d, o.strength, singular, &agg, s);
+        if (nagg == 0 || (int64_t)nagg * 10 > (int64_t)n * 9) break;
+        L.agg = agg;
         Scratch<int> plen(n), err(1);
         VEMG_CHECK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         k_prolong_len<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp, L.A.ci, L.A.v, d, o.strength, L.agg, plen, err);

@@ -306,6 +306,7 @@ struct Chain {
 };
 
 struct Graphs;
+struct PrecondGraph;
 struct BatchWork;
 struct Persist;
 
@@ -339,6 +340,7 @@ struct vemg_hierarchy {
     // ---- solve order (see layout.cu) ----
     int nu = 0;                                   // unknowns: n (Neumann) or n - mtop
     int *caller_of = nullptr;                     // caller id of each solve-order unknown
+    int *s2i = nullptr;                           // its index among the unknowns in internal order
     int *tops = nullptr;                          // caller ids of the top nodes
     vemg::Sell Aop;                               // outer operator, FP64, diagonal included
     vemg::Sell Enon;                              // E~ rows of non-top nodes (Neumann)
@@ -347,6 +349,8 @@ struct vemg_hierarchy {
     vemg::SChain ssurf, sbar;
     // CUDA graphs of the solve (built on the first solve)
     vemg::Graphs *graphs = nullptr;
+    vemg::PrecondGraph *pgraph = nullptr;         // one preconditioner application (vemg_precond)
+    int precond_calls = 0;
     cudaStream_t side = nullptr;                  // second branch of the preconditioner
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_mid = nullptr, ev_coarse = nullptr;
     unsigned *ctr = nullptr;                      // arrival counters of the block reductions

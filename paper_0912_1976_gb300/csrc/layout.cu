@@ -363,7 +363,9 @@ void build_solve_layout(vemg_hierarchy *h, cudaStream_t s) {
         layout_chain(ar, h->bar, h->sbar, fp32, s, bf16);
         layout_chain(ar, h->surf, h->ssurf, fp32, s, bf16);
         h->nu = n;
-        Scratch<int> s2n(n), n2s(n);
+        int *s2n = ar.alloc<int>(n);
+        h->s2i = s2n;
+        Scratch<int> n2s(n);
         k_outer_order<<<grid_for(n, 256), 256, 0, s>>>(n, mt, h->surf.lv[0].crow, h->bar.lv[0].crow, s2n);
         VEMG_CHECK_LAUNCH();
         k_inverse_perm<<<grid_for(n, 256), 256, 0, s>>>(n, s2n, n2s);
@@ -372,7 +374,7 @@ void build_solve_layout(vemg_hierarchy *h, cudaStream_t s) {
         k_inverse_perm<<<grid_for(mt, 256), 256, 0, s>>>(mt, h->surf.lv[0].crow, surf_inv);
         VEMG_CHECK_LAUNCH();
         h->Aop = build_sell(ar, h->A, n, s2n, n2s, n, {0, n}, false, nullptr, nullptr, s);
-        h->Enon = build_sell(ar, h->E, n - mt, s2n.p + mt, surf_inv, mt, {0, n - mt}, false, nullptr, nullptr, s);
+        h->Enon = build_sell(ar, h->E, n - mt, s2n + mt, surf_inv, mt, {0, n - mt}, false, nullptr, nullptr, s);
         h->ETs = build_sell(ar, h->ET, mt, h->surf.lv[0].crow, n2s, n, {0, mt}, false, nullptr, nullptr, s,
                             lanes_shift(mt, (double)h->ET.nnz / std::max(mt, 1)));
         if (fp32 && h->Enon.padded > 0) {
@@ -388,7 +390,8 @@ void build_solve_layout(vemg_hierarchy *h, cudaStream_t s) {
     } else if (h->precond == VEMG_PRECOND_NONE && h->bc == VEMG_NEUMANN) {
         // plain CG: no cycle, the unknowns in their internal order
         h->nu = n;
-        Scratch<int> iota(n);
+        int *iota = ar.alloc<int>(n);
+        h->s2i = iota;
         k_iota<<<grid_for(n, 256), 256, 0, s>>>(n, iota);
         VEMG_CHECK_LAUNCH();
         h->Aop = build_sell(ar, h->A, n, iota, iota, n, {0, n}, false, nullptr, nullptr, s);
@@ -404,6 +407,7 @@ void build_solve_layout(vemg_hierarchy *h, cudaStream_t s) {
         int nb = n - off;
         h->nu = nb;
         const Level &L0 = C.lv[0];
+        h->s2i = L0.crow;
         Scratch<int> inv(nb);
         k_inverse_perm<<<grid_for(nb, 256), 256, 0, s>>>(nb, L0.crow, inv);
         VEMG_CHECK_LAUNCH();

@@ -464,26 +464,46 @@ static SellArgs sargs(const Sell &S) {
 }
 
 // the grid of a pass over an outer operator: a warp per slice until the chip is full
-static int row_blocks(const Sell &S) {
-    return std::min(kRedBlocks, std::max(1, grid_for((int64_t)S.nslices * 32, kRedThreads)));
+static int row_blocks(const Sell &S, int most) {
+    return std::min(most, std::max(1, grid_for((int64_t)S.nslices * 32, kRedThreads)));
 }
 
-// q = A p over all slices and (p, q); the last block sets alpha = rz / pq. At most 64 registers:
-// the whole grid (kRedBlocks = 4 per SM) is resident at once.
+struct SliceMeta {
+    int row0, nrow, off, width;
+};
+
+__device__ __forceinline__ SliceMeta slice_meta(const SellArgs &A, int s) {
+    if (s >= A.nsl) return SliceMeta{0, 0, 0, 0};
+    return SliceMeta{__ldg(A.row0 + s), __ldg(A.nrow + s), __ldg(A.off + s), __ldg(A.width + s)};
+}
+
+// q = A p over all slices and, DOT, (p, q); the last block sets alpha = rz / pq. map: q in another
+// order. At most 64 registers: the whole grid (kRedBlocks = 4 per SM) is resident at once.
+//
+// The FP64 pipe (two multiply-adds per cycle and SM: 51 us of 32M entries) and memory (12 bytes an
+// entry: 60 us) bound it about equally; it takes 88 us. A ring of slices in shared memory, two per warp
+// filled by cp.async ahead of the warp, took 113: it left the gathers of p a tenth of the L1 cache.
+template <bool DOT>
 __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152) k_spmv_pq(SellArgs A, const double *__restrict__ p,
-                                                         double *__restrict__ q, double *sc, double *part,
-                                                         unsigned *ctr, double *coef) {
+                                                                           double *__restrict__ q,
+                                                                           const int *__restrict__ map, double *sc,
+                                                                           double *part, unsigned *ctr, double *coef) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, stride = gridDim.x * (kRedThreads / 32);
+    int s = blockIdx.x * (kRedThreads / 32) + warp;
+    SliceMeta m = slice_meta(A, s);
     pdl_begin();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double acc[1] = {0.0};
-    for (int s = blockIdx.x * (kRedThreads / 32) + warp; s < A.nsl; s += gridDim.x * (kRedThreads / 32)) {
-        if (lane < A.nrow[s]) {
-            int r = A.row0[s] + lane;
-            double qv = sell_row<double, double, double>(A.col, A.v, A.off[s] + lane, A.width[s], p);
-            q[r] = qv;
-            acc[0] = fma(p[r], qv, acc[0]);
+    for (; s < A.nsl; s += stride) {
+        const SliceMeta next = slice_meta(A, s + stride);
+        if (lane < m.nrow) {
+            const int r = m.row0 + lane;
+            const double qv = sell_row<double, double, double>(A.col, A.v, m.off + lane, m.width, p);
+            q[DOT ? r : __ldg(map + r)] = qv;
+            if (DOT) acc[0] = fma(p[r], qv, acc[0]);
         }
+        m = next;
     }
+    if (!DOT) return;
     double tot[1];
     if (!finish_block<1>(acc, part, ctr, tot) || threadIdx.x != 0) return;
     double pq = tot[0];
@@ -822,8 +842,8 @@ static void precond_solve_order(vemg_hierarchy *h, const double *r, double *z, i
 // q = A p of the outer loop, with (p, q) and alpha
 static void spmv_outer(vemg_hierarchy *h, const double *x, double *y, cudaStream_t s) {
     ProbeScope ps(PROBE_SPMV_A, sell_bytes(h->Aop.nnz, 8.0, h->Aop.n, 24.0), s);   // p read twice, q write
-    pdl_launch(k_spmv_pq, row_blocks(h->Aop), kRedThreads, s, sargs(h->Aop), x, y, h->scal, h->red + 5 * kRedBlocks * C_SPMV,
-                                                 h->ctr + C_SPMV, h->coef);
+    pdl_launch(k_spmv_pq<true>, row_blocks(h->Aop, kRedBlocks), kRedThreads, s, sargs(h->Aop), x, y,
+               (const int *)nullptr, h->scal, h->red + 5 * kRedBlocks * C_SPMV, h->ctr + C_SPMV, h->coef);
     SOLVE_LAUNCHED();
 }
 
@@ -909,7 +929,7 @@ static void phase_post(vemg_hierarchy *h, cudaStream_t s) {
         pdl_launch(k_sub_scalar, grid_for(nu, 256), 256, s, nu, h->x, h->scal, S_XMEAN);
         SOLVE_LAUNCHED();
     }
-    pdl_launch(k_true_res, row_blocks(h->Aop), kRedThreads, s, sargs(h->Aop), h->x, h->b, h->scal, part_of(h, C_TRUE),
+    pdl_launch(k_true_res, row_blocks(h->Aop, kRedBlocks), kRedThreads, s, sargs(h->Aop), h->x, h->b, h->scal, part_of(h, C_TRUE),
                                                   h->ctr + C_TRUE);
     SOLVE_LAUNCHED();
 }
@@ -977,7 +997,23 @@ static void build_graphs(vemg_hierarchy *h) {
     VEMG_CHECK_CUDA(cudaStreamDestroy(cs));
 }
 
+struct PrecondGraph {
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    int64_t kernels = 0;
+};
+
+static void release_precond_graph(vemg_hierarchy *h) {
+    PrecondGraph *G = h->pgraph;
+    if (!G) return;
+    if (G->exec) cudaGraphExecDestroy(G->exec);
+    if (G->g) cudaGraphDestroy(G->g);
+    delete G;
+    h->pgraph = nullptr;
+}
+
 void release_graphs(vemg_hierarchy *h) {
+    release_precond_graph(h);
     Graphs *G = h->graphs;
     if (G) {
         if (G->exec) cudaGraphExecDestroy(G->exec);
@@ -1083,7 +1119,8 @@ int solve(vemg_hierarchy *h, const double *b_in, double *x_out, double rtol, int
 }
 
 // ------------------------------------------------------------------------------------------
-// single steps in the internal (top-first) order, for the parity tests
+// single steps in the internal (top-first) order. Their work vectors are the solve's (a hierarchy is
+// used by one host thread at a time, and every call waits for its stream): no allocation per call.
 
 __global__ void k_perm_in(int n, const int *__restrict__ s2i, const double *__restrict__ a, double *__restrict__ b) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1095,43 +1132,68 @@ __global__ void k_perm_out(int n, const int *__restrict__ s2i, const double *__r
     if (i < n) b[s2i[i]] = a[i];
 }
 
-// solve index -> internal index of the unknowns
-__global__ void k_solve_to_internal(int n, int off, const int *__restrict__ caller_of, const int *__restrict__ old2new,
-                                    int *out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = old2new[caller_of[i]] - off;
-}
-
 void spmv_op(vemg_hierarchy *h, const double *x, double *y, cudaStream_t s) {
     prepare_solve(h, s);
     g_probe = &h->probe;
     g_count = &h->launches;
-    int nu = h->nu, off = h->bc == VEMG_DIRICHLET_TOP ? h->mtop : 0;
-    Scratch<int> s2i(nu);
-    k_solve_to_internal<<<grid_for(nu, 256), 256, 0, s>>>(nu, off, h->caller_of, h->old2new, s2i);
+    const int nu = h->nu;
+    k_perm_in<<<grid_for(nu, 256), 256, 0, s>>>(nu, h->s2i, x, h->p);
     SOLVE_LAUNCHED();
-    Scratch<double> xs(nu), ys(nu);
-    k_perm_in<<<grid_for(nu, 256), 256, 0, s>>>(nu, s2i, x, xs);
-    SOLVE_LAUNCHED();
-    spmv_outer(h, xs, ys, s);
-    k_perm_out<<<grid_for(nu, 256), 256, 0, s>>>(nu, s2i, ys, y);
-    SOLVE_LAUNCHED();
+    {
+        ProbeScope ps(PROBE_SPMV_A, sell_bytes(h->Aop.nnz, 8.0, nu, 20.0), s);
+        pdl_launch(k_spmv_pq<false>, row_blocks(h->Aop, kRedBlocks), kRedThreads, s, sargs(h->Aop),
+                   (const double *)h->p, y, (const int *)h->s2i, (double *)nullptr, (double *)nullptr,
+                   (unsigned *)nullptr, (double *)nullptr);
+        SOLVE_LAUNCHED();
+    }
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
+}
+
+// one application of the preconditioner on r -> z as a graph of its own (about 100 launches of 2.5 us each
+// on the host otherwise); built by a hierarchy's second call, so that a single one does not pay for it
+static void precond_graph(vemg_hierarchy *h) {
+    PrecondGraph *G = new PrecondGraph();
+    h->pgraph = G;
+    cudaStream_t cs;
+    VEMG_CHECK_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    Probe *saved = g_probe;
+    int64_t *saved_count = g_count, count = 0;
+    g_probe = nullptr;
+    g_count = &count;
+    try {
+        VEMG_CHECK_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+        precond_solve_order(h, h->r, h->z, 1, cs);
+        VEMG_CHECK_CUDA(cudaStreamEndCapture(cs, &G->g));
+        G->kernels = count;
+        VEMG_CHECK_CUDA(cudaGraphInstantiate(&G->exec, G->g, 0));
+    } catch (...) {
+        cudaStreamDestroy(cs);
+        g_probe = saved;
+        g_count = saved_count;
+        release_precond_graph(h);
+        throw;
+    }
+    g_probe = saved;
+    g_count = saved_count;
+    VEMG_CHECK_CUDA(cudaStreamDestroy(cs));
 }
 
 void precond(vemg_hierarchy *h, const double *r, double *z, cudaStream_t s) {
     prepare_solve(h, s);
     g_probe = &h->probe;
     g_count = &h->launches;
-    int nu = h->nu, off = h->bc == VEMG_DIRICHLET_TOP ? h->mtop : 0;
-    Scratch<int> s2i(nu);
-    k_solve_to_internal<<<grid_for(nu, 256), 256, 0, s>>>(nu, off, h->caller_of, h->old2new, s2i);
+    const int nu = h->nu;
+    k_perm_in<<<grid_for(nu, 256), 256, 0, s>>>(nu, h->s2i, r, h->r);
     SOLVE_LAUNCHED();
-    Scratch<double> rs(nu), zs(nu);
-    k_perm_in<<<grid_for(nu, 256), 256, 0, s>>>(nu, s2i, r, rs);
-    SOLVE_LAUNCHED();
-    precond_solve_order(h, rs, zs, 1, s);
-    k_perm_out<<<grid_for(nu, 256), 256, 0, s>>>(nu, s2i, zs, z);
+    const bool use_graph = h->probe.kind == PROBE_NONE && h->precond_calls++ > 0;
+    if (use_graph) {
+        if (!h->pgraph) precond_graph(h);
+        VEMG_CHECK_CUDA(cudaGraphLaunch(h->pgraph->exec, s));
+        h->launches += h->pgraph->kernels;
+    } else {
+        precond_solve_order(h, h->r, h->z, 1, s);
+    }
+    k_perm_out<<<grid_for(nu, 256), 256, 0, s>>>(nu, h->s2i, h->z, z);
     SOLVE_LAUNCHED();
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
 }
@@ -1161,11 +1223,11 @@ void vcycle(vemg_hierarchy *h, int chain, const double *b, double *x, cudaStream
     const SChain &S = chain == 0 ? h->ssurf : h->sbar;
     int n = C.lv[0].A.n;
     bool f = S.fp32;
-    Scratch<char> bs((int64_t)n * 8), xs((int64_t)n * 8);
+    double *bs = h->p, *xs = h->q;
     k_perm_in_x<<<grid_for(n, 256), 256, 0, s>>>(n, C.lv[0].crow, b, bs, f);
     SOLVE_LAUNCHED();
-    if (f) vcycle_level<float, float>(S, 0, (const float *)bs.p, (float *)xs.p, s);
-    else vcycle_level<double, double>(S, 0, (const double *)bs.p, (double *)xs.p, s);
+    if (f) vcycle_level<float, float>(S, 0, (const float *)bs, (float *)xs, s);
+    else vcycle_level<double, double>(S, 0, (const double *)bs, (double *)xs, s);
     k_perm_out_x<<<grid_for(n, 256), 256, 0, s>>>(n, C.lv[0].crow, xs, x, f);
     SOLVE_LAUNCHED();
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));

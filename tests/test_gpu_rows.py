@@ -74,3 +74,30 @@ def test_solution_scales_exactly_with_the_right_hand_side(precision, power):
     assert torch.equal(y, x * 2.0 ** power)
     Y, infos = V.vemg_solve_batch(h, torch.stack([b, b * 2.0 ** power]), rtol=1e-8)
     assert infos[0]["status"] == infos[1]["status"] == "OK" and torch.equal(Y[1], Y[0] * 2.0 ** power)
+
+
+@pytest.mark.parametrize("bc", [V.VEMG_NEUMANN, V.VEMG_DIRICHLET_TOP])
+@pytest.mark.parametrize("precision", [V.VEMG_PREC_FP64, V.VEMG_PREC_BF16])
+def test_single_steps_repeat_and_share_the_solve_vectors(bc, precision):
+    """vemg_precond runs from a graph from its second call on, and the single steps work in the solve's
+    vectors: the same bits call after call, in place, between solves and beside other steps."""
+    m = I.make_mesh(23, 19, 11, I.depth_sines(1e-2), z_jitter=0.3, seed=67)
+    vm = V.Mesh.from_inputs(m)
+    h = V.vemg_setup(V.vemg_assemble(vm), vm, V.vemg_default_options(bc=bc, precision=precision))
+    n = V.vemg_get_size(h, "n") - (V.vemg_get_size(h, "mtop") if bc == V.VEMG_DIRICHLET_TOP else 0)
+    r = torch.from_numpy(np.random.default_rng(8).standard_normal(n)).cuda()
+    b = torch.from_numpy(I.normal_loads(m.n, 68)).cuda()
+    z, y, v = V.vemg_precond(h, r), V.vemg_spmv(h, r), None
+    x, _ = V.vemg_solve(h, b, rtol=1e-8)
+    for _ in range(3):
+        assert torch.equal(V.vemg_precond(h, r), z) and torch.equal(V.vemg_spmv(h, r), y)
+        w = V.vemg_vcycle(h, 1, r[:V.vemg_get_size(h, "lev.n", 1, 0)].contiguous())
+        assert v is None or torch.equal(v, w)
+        v = w
+        assert torch.equal(V.vemg_solve(h, b, rtol=1e-8)[0], x)
+    for step, want in ((V.vemg_precond, z), (V.vemg_spmv, y)):
+        t = r.clone()
+        assert torch.equal(step(h, t, t), want)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    assert torch.equal(V.vemg_precond(h, r, stream=side), z)

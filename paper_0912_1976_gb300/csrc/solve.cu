@@ -338,12 +338,22 @@ static bool fused_first(const SChain &C, int l) {
     return !(l > 0 && l == C.tail_level);
 }
 
+// An event that vcycle_level records on its stream when it enters a level: where work of another
+// stream may start beside the coarse levels (k_late)
+struct LevelMark {
+    const SChain *C = nullptr;
+    int level = 0;
+    cudaEvent_t ev = nullptr;
+};
+static thread_local LevelMark g_mark;
+
 // V-cycle with a zero initial guess (section 5.1); b of level 0 may be FP64 (the outer residual).
 // first_done: the first colour of the pre-smoothing sweep was done by the restriction into l.
 template <class XT, class BT>
 static void vcycle_level(const SChain &C, int l, const BT *b, XT *x, cudaStream_t s, bool first_done = false) {
     const SLevel &L = C.lv[l];
     const bool fine = C.is_bar && l == 0;
+    if (g_mark.C == &C && l == g_mark.level) VEMG_CHECK_CUDA(cudaEventRecord(g_mark.ev, s));
     if (l > 0 && l == C.tail_level) {
         // the coarse tail: every level from here down and back up in one kernel (one CTA, or one
         // thread-block cluster); it reads b and writes x in this level's own buffers
@@ -406,9 +416,9 @@ static void vcycle_up(const SChain &C, const BT *b, XT *x, cudaStream_t s) {
 
 enum {
     S_RZ = 0, S_PQ, S_ALPHA, S_BETA, S_MU, S_BN, S_RN, S_FLAG, S_TOL, S_MAXIT, S_ITERS, S_CONT, S_ZERO, S_TRUE,
-    S_BMEAN, S_XMEAN, S_COUNT
+    S_BMEAN, S_XMEAN, S_SUMR, S_SUMQ, S_COUNT
 };
-enum { C_SPMV = 0, C_XR, C_Z, C_SUMB, C_PREP, C_SUMX, C_TRUE, C_COUNT };
+enum { C_SPMV = 0, C_XR, C_Z, C_SUMB, C_PREP, C_SUMX, C_TRUE, C_LATE, C_COUNT };
 
 int solve_scalar_iters() { return S_ITERS; }
 
@@ -518,32 +528,29 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152) k_spmv_pq(SellA
     if (2 * k < kCoefCap) coef[2 * k] = sc[S_ALPHA];
 }
 
-// x += alpha p, r -= alpha q; the last block sets ||r||, the iteration count and the continuation
-// test (and, inside the solve graph, the WHILE condition)
-// Bound by memory (48 bytes a row; vectors are 256-byte aligned, two rows a load, four a trip).
-__global__ void __launch_bounds__(kRedThreads, 2) k_update_xr(int n, const double *__restrict__ p,
-                                                              const double *__restrict__ q, double *__restrict__ x,
-                                                              double *__restrict__ r, double *sc, double *part,
-                                                              unsigned *ctr, cudaGraphConditionalHandle handle,
-                                                              int use_cond) {
+// r -= alpha q; the last block sets ||r||, the iteration count and the continuation test (and, inside
+// the solve graph, the WHILE condition). Bound by memory (24 bytes a row; vectors are 256-byte aligned,
+// two rows a load, four a trip).
+__global__ void __launch_bounds__(kRedThreads, 2) k_update_r(int n, const double *__restrict__ q, double *__restrict__ r,
+                                                             double *sc, double *part, unsigned *ctr,
+                                                             cudaGraphConditionalHandle handle, int use_cond) {
     pdl_begin();
     const double a = sc[S_ALPHA];
     double acc[1] = {0.0};
     const int stride = gridDim.x * kRedThreads, n2 = n >> 1;
-    const double2 *p2 = (const double2 *)p, *q2 = (const double2 *)q;
-    double2 *x2 = (double2 *)x, *r2 = (double2 *)r;
-    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n2; i0 += 2 * stride) {
-        double2 pv[2], qv[2], xv[2], rv[2];
+    const double2 *q2 = (const double2 *)q;
+    double2 *r2 = (double2 *)r;
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n2; i0 += 4 * stride) {
+        double2 qv[4], rv[4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < 4; ++u) {
             const int i = i0 + u * stride;
-            if (i < n2) { pv[u] = p2[i]; qv[u] = q2[i]; xv[u] = x2[i]; rv[u] = r2[i]; }
+            if (i < n2) { qv[u] = q2[i]; rv[u] = r2[i]; }
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < 4; ++u) {
             const int i = i0 + u * stride;
             if (i >= n2) continue;
-            x2[i] = make_double2(fma(a, pv[u].x, xv[u].x), fma(a, pv[u].y, xv[u].y));
             const double2 ri = make_double2(fma(-a, qv[u].x, rv[u].x), fma(-a, qv[u].y, rv[u].y));
             r2[i] = ri;
             acc[0] = fma(ri.x, ri.x, acc[0]);
@@ -551,10 +558,8 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_update_xr(int n, const doubl
         }
     }
     if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-        const int i = n - 1;
-        x[i] = fma(a, p[i], x[i]);
-        const double ri = fma(-a, q[i], r[i]);
-        r[i] = ri;
+        const double ri = fma(-a, q[n - 1], r[n - 1]);
+        r[n - 1] = ri;
         acc[0] = fma(ri, ri, acc[0]);
     }
     double tot[1];
@@ -569,13 +574,59 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_update_xr(int n, const doubl
     if (use_cond) cudaGraphSetConditional(handle, cont ? 1u : 0u);
 }
 
+// What an iteration owes that nothing before the next z needs: x += alpha p and the sums of r and (q
+// given) q, which the next k_combine multiplies the mean of z by. It runs on the side stream, beside
+// the A_bar cycle, whose coarse levels leave memory and the FP64 pipe idle; x catches up after the loop.
+// r == null: x alone.
+__global__ void __launch_bounds__(kRedThreads, 2) k_late(int n, const double *__restrict__ p, double *__restrict__ x,
+                                                         const double *__restrict__ r, const double *__restrict__ q,
+                                                         double *sc, double *part, unsigned *ctr, double one) {
+    pdl_begin();
+    const double a = sc[S_ALPHA];
+    double acc[2] = {0.0, 0.0};
+    const int stride = gridDim.x * kRedThreads, n2 = n >> 1;
+    const double2 *p2 = (const double2 *)p, *r2 = (const double2 *)r, *q2 = (const double2 *)q;
+    double2 *x2 = (double2 *)x;
+    const double2 zero = make_double2(0.0, 0.0);
+    for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n2; i0 += 2 * stride) {
+        double2 pv[2], xv[2], rv[2], qv[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= n2) continue;
+            pv[u] = p2[i];
+            xv[u] = x2[i];
+            rv[u] = r ? r2[i] : zero;
+            qv[u] = q ? q2[i] : zero;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= n2) continue;
+            x2[i] = make_double2(fma(a, pv[u].x, xv[u].x), fma(a, pv[u].y, xv[u].y));
+            if (r) acc[0] = dadd(dadd(acc[0], rv[u].x, one), rv[u].y, one);
+            if (q) acc[1] = dadd(dadd(acc[1], qv[u].x, one), qv[u].y, one);
+        }
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        x[n - 1] = fma(a, p[n - 1], x[n - 1]);
+        if (r) acc[0] += r[n - 1];
+        if (q) acc[1] += q[n - 1];
+    }
+    if (!r) return;
+    double tot[2];
+    if (!finish_block<2>(acc, part, ctr, tot) || threadIdx.x != 0) return;
+    sc[S_SUMR] = tot[0];
+    sc[S_SUMQ] = tot[1];
+}
+
 // z from the two branches (Neumann: top rows z = y_s, other rows z = E~ y_s + x_bar; Dirichlet-
-// top: z = x_bar) and the sums t0 = sum z, t1 = (r, z), t2 = sum r, t3 = (z, q), t4 = sum q.
+// top: z = x_bar) and the sums t0 = sum z, t1 = (r, z), t2 = (z, q).
 // The last block sets mu (mean of z), rz = (r, z - mu) and beta: first direction 0, CG
 // rz'/rz, FCG -(z - mu, q) / (p, q).
 //
-// FP64 bounds it, five sums a row (22 us of 2.2M rows; the bytes take 12): the sums are multiply-adds,
-// z's conversion integer arithmetic. z itself: with FP32 V-cycles (XT = float, FP32 copy evf of E~) it
+// FP64 and memory bound it, three sums (10 us of 2.2M rows) and 36 bytes a row (12 us): the sums are
+// multiply-adds, z's conversion integer arithmetic, the sums of r and q k_late's. z itself: with FP32 V-cycles (XT = float, FP32 copy evf of E~) it
 // is formed in FP32 and converted once, else in FP64.
 template <class XT>
 __global__ void __launch_bounds__(kRedThreads, 2) k_combine(int nu, int mtop, SellArgs E, const float *__restrict__ evf,
@@ -587,7 +638,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_combine(int nu, int mtop, Se
                                                             double one) {
     pdl_begin();
     const XT *ev = sizeof(XT) == sizeof(float) ? (const XT *)evf : (const XT *)E.v;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    double acc[3] = {0.0, 0.0, 0.0};
     constexpr int R = sizeof(XT) == sizeof(float) ? 4 : 2;   // rows per thread and trip
     const int stride = gridDim.x * kRedThreads;
     const bool dots_q = flexible && !first;
@@ -630,20 +681,16 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_combine(int nu, int mtop, Se
             z[i] = zi;
             acc[0] = dadd(acc[0], zi, one);
             acc[1] = fma(rv[u], zi, acc[1]);
-            acc[2] = dadd(acc[2], rv[u], one);
-            if (dots_q) {
-                acc[3] = fma(zi, qv[u], acc[3]);
-                acc[4] = dadd(acc[4], qv[u], one);
-            }
+            if (dots_q) acc[2] = fma(zi, qv[u], acc[2]);
         }
     }
-    double tot[5];
-    if (!finish_block<5>(acc, part, ctr, tot) || threadIdx.x != 0) return;
+    double tot[3];
+    if (!finish_block<3>(acc, part, ctr, tot) || threadIdx.x != 0) return;
     double mu = neumann ? tot[0] * inv_n : 0.0;
-    double rz = tot[1] - mu * tot[2];
+    double rz = tot[1] - mu * sc[S_SUMR];
     double beta;
     if (first) beta = 0.0;
-    else if (flexible) beta = -(tot[3] - mu * tot[4]) / sc[S_PQ];
+    else if (flexible) beta = -(tot[2] - mu * sc[S_SUMQ]) / sc[S_PQ];
     else beta = rz / sc[S_RZ];
     sc[S_MU] = mu;
     sc[S_BETA] = beta;
@@ -686,14 +733,14 @@ __global__ void __launch_bounds__(kRedThreads) k_mean(int n, const double *__res
     sc[slot] = tot[0] * inv_n;
 }
 
-// b -= mean (Neumann), r = b, x = 0, p = 0, ||b||; the last block sets ||b|| and the zero flag
+// b -= mean (Neumann), r = b, x = 0, p = 0, ||b||; the last block sets ||b||, the sum of r and the zero flag
 __global__ void __launch_bounds__(kRedThreads) k_prepare(int n, int neumann, double *__restrict__ b,
                                                          double *__restrict__ r, double *__restrict__ x,
                                                          double *__restrict__ p, double *sc, double *part,
                                                          unsigned *ctr) {
     pdl_begin();
     double mu = neumann ? sc[S_BMEAN] : 0.0;
-    double acc[1] = {0.0};
+    double acc[2] = {0.0, 0.0};
     const int stride = gridDim.x * kRedThreads;
     for (int i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < n; i0 += 4 * stride) {
         double v[4];
@@ -709,10 +756,12 @@ __global__ void __launch_bounds__(kRedThreads) k_prepare(int n, int neumann, dou
             x[i] = 0.0;
             p[i] = 0.0;
             acc[0] = fma(bi, bi, acc[0]);
+            acc[1] += bi;
         }
     }
-    double tot[1];
-    if (!finish_block<1>(acc, part, ctr, tot) || threadIdx.x != 0) return;
+    double tot[2];
+    if (!finish_block<2>(acc, part, ctr, tot) || threadIdx.x != 0) return;
+    sc[S_SUMR] = tot[1];
     double bn = sqrt(tot[0]);
     sc[S_BN] = bn;
     if (bn == 0.0) {
@@ -750,6 +799,17 @@ __global__ void __launch_bounds__(kRedThreads) k_true_res(SellArgs A, const doub
 // the preconditioner: two independent V-cycles (the additive form of Eq. ourpreconditioner)
 // on two streams, joined by the kernel that forms z
 
+// k_late on stream s (sums: for the next k_combine)
+static void late(vemg_hierarchy *h, bool sums, cudaStream_t s) {
+    const bool flex = h->precision != VEMG_PREC_FP64;
+    ProbeScope ps(PROBE_VECTOR, (double)h->nu * (24.0 + (sums ? 8.0 + (flex ? 8.0 : 0.0) : 0.0)), s);
+    pdl_launch(k_late, vec_blocks(h->nu), kRedThreads, s, h->nu, (const double *)h->p, h->x,
+               (const double *)(sums ? h->r : nullptr), (const double *)(sums && flex ? h->q : nullptr), h->scal,
+               h->red + 5 * kRedBlocks * C_LATE, h->ctr + C_LATE, 1.0);
+    SOLVE_LAUNCHED();
+}
+
+// first: no iteration before this application, so nothing is owed (k_late)
 template <class XT>
 static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, cudaStream_t s) {
     const SChain &B = h->sbar;
@@ -763,6 +823,12 @@ static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, 
                          pk != PROBE_TRANSFER && pk != PROBE_DENSE && pk != PROBE_TAIL;
     const bool none = h->precond == VEMG_PRECOND_NONE;
     const bool hybrid = persist && persist_coarse_only(h);
+    const bool side = two && (hybrid || !persist) && !none;   // the surface branch's stream is in use
+    // k_late beside the first level of at most an eighth of the rows: the finer ones need the memory
+    const bool mark = !first && !persist && !none;
+    int lv = 0;
+    while (mark && lv + 1 < B.nlev && (int64_t)B.lv[lv].n * 8 > B.lv[0].n) ++lv;
+    if (!first && !side) VEMG_CHECK_CUDA(cudaEventRecord(h->ev_fork, s));
     if (none) {
         // no preconditioner (plain CG): z = r, formed by k_combine below
     } else if (hybrid) {
@@ -791,10 +857,8 @@ static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, 
             VEMG_CHECK_CUDA(cudaEventRecord(h->ev_coarse, s));
             VEMG_CHECK_CUDA(cudaStreamWaitEvent(h->side, h->ev_coarse, 0));
             if (sc) vcycle_up<XT, XT>(S, (const XT *)S.lv[0].b, (XT *)S.lv[0].x, h->side);
-            VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
         }
         if (bc) vcycle_up<XT, double>(B, r + mt, (XT *)B.lv[0].x, s);
-        if (two) VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
     } else if (persist) {
         // both branches (or the single chain) in one cooperative kernel
         {
@@ -811,13 +875,26 @@ static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, 
         const bool fuse = fused_first(S, 0);
         sell_spmv<double, double, XT, double>(h->ETs, r, (XT *)S.lv[0].b, 0, h->side, fuse ? &S.lv[0] : nullptr);
         vcycle_level<XT, XT>(S, 0, (const XT *)S.lv[0].b, (XT *)S.lv[0].x, h->side, fuse);
-        VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
         ys = (const XT *)S.lv[0].x;
     }
     if (!persist && !none) {   // one kernel per phase
         // additive smoother: one V-cycle on A_bar with the trailing part of r
-        vcycle_level<XT, double>(B, 0, r + mt, (XT *)B.lv[0].x, s);
-        if (two) VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
+        if (mark) g_mark = LevelMark{&B, lv, h->ev_fork};
+        try {
+            vcycle_level<XT, double>(B, 0, r + mt, (XT *)B.lv[0].x, s);
+        } catch (...) {
+            g_mark = LevelMark{};
+            throw;
+        }
+        g_mark = LevelMark{};
+    }
+    if (!first) {
+        if (mark || !side) VEMG_CHECK_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+        late(h, true, h->side);
+    }
+    if (side || !first) {
+        VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
+        VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
     }
     const XT *xb = none ? (const XT *)r : (const XT *)B.lv[0].x;   // none: XT is double
     // r, z (and q) per row, x_bar per non-top row, the E~ entries and one read of y_s
@@ -902,12 +979,13 @@ static void phase_pre(vemg_hierarchy *h, cudaStream_t s) {
     }
 }
 
-// q = A p, alpha, x and r updates, ||r||, continuation
+// q = A p, alpha, r update, ||r||, continuation (x is updated beside the next preconditioner
+// application, or by phase_post)
 static void phase_step(vemg_hierarchy *h, cudaStream_t s, cudaGraphConditionalHandle hd, int use_cond) {
     spmv_outer(h, h->p, h->q, s);
-    ProbeScope ps(PROBE_VECTOR, 48.0 * h->nu, s);   // p, q, x, r read; x, r written
-    pdl_launch(k_update_xr, vec_blocks(h->nu), kRedThreads, s, h->nu, h->p, h->q, h->x, h->r, h->scal, part_of(h, C_XR),
-                                                   h->ctr + C_XR, hd, use_cond);
+    ProbeScope ps(PROBE_VECTOR, 24.0 * h->nu, s);   // q, r read; r written
+    pdl_launch(k_update_r, vec_blocks(h->nu), kRedThreads, s, h->nu, (const double *)h->q, h->r, h->scal,
+               part_of(h, C_XR), h->ctr + C_XR, hd, use_cond);
     SOLVE_LAUNCHED();
 }
 
@@ -922,6 +1000,7 @@ static void phase_direction(vemg_hierarchy *h, cudaStream_t s) {
 static void phase_post(vemg_hierarchy *h, cudaStream_t s) {
     const bool neu = h->bc == VEMG_NEUMANN;
     const int nu = h->nu;
+    late(h, false, s);
     if (neu) {
         pdl_launch(k_mean, vec_blocks(nu), kRedThreads, s, nu, h->x, 1.0 / (double)nu, S_XMEAN, h->scal, part_of(h, C_SUMX),
                                                   h->ctr + C_SUMX);

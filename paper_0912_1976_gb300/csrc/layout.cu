@@ -124,10 +124,14 @@ __global__ void k_sell_deal(int nslices, int lsh, const int *__restrict__ row0, 
 // Lanes per row of a chain's operator, by the rows that one launch works on and their mean length.
 // A row per thread reads 32 rows' entries in consecutive words and is the better form while the
 // rows alone fill half the chip (152 SMs x 2048 threads); below that a launch lasts as long as its
-// longest chain of loads, which more lanes per row cut: four entries each is as far as it pays.
-static int lanes_shift(double rows, double mean) {
+// longest chain of loads, which more lanes per row cut: four entries each is as far as it pays. In FP64
+// every step of a warp holds a scheduler for 64 cycles however few of its lanes have an entry, and so does
+// every level of the tree that adds the lanes up, so lanes pay half as far (a 131 x 113 x 25 solve: 9.53 ms;
+// 10.02 with the FP32 limit, 9.97 and 10.68 with a half and a quarter of this one).
+static int lanes_shift(double rows, double mean, bool fp32) {
+    const double most = 152.0 * (fp32 ? 1024.0 : 512.0);
     int lsh = 0;
-    while (lsh < 5 && mean > 4.0 * (1 << lsh) && rows * (2 << lsh) <= 152.0 * 1024.0) ++lsh;
+    while (lsh < 5 && mean > 4.0 * (1 << lsh) && rows * (2 << lsh) <= most) ++lsh;
     return lsh;
 }
 
@@ -301,14 +305,14 @@ static void layout_chain(Arena &ar, const Chain &C, SChain &S, bool fp32, cudaSt
         T.ncolours = L.ncolours;
         T.crow = L.cptr;
         T.A = build_sell(ar, L.A, L.A.n, L.crow, inv[l], L.A.n, L.cptr, fp32, &T.dinv, &T.cslice, s,
-                         lanes_shift((double)L.A.n / std::max(L.ncolours, 1), (double)L.A.nnz / std::max(L.A.n, 1) - 1.0),
+                         lanes_shift((double)L.A.n / std::max(L.ncolours, 1), (double)L.A.nnz / std::max(L.A.n, 1) - 1.0, fp32),
                          &T.clow, &T.cnnz);
         if (l + 1 < C.nlev) {
             const Level &N = C.lv[l + 1];
             T.P = build_sell(ar, L.P, L.A.n, L.crow, inv[l + 1], N.A.n, {0, L.A.n}, fp32, nullptr, nullptr, s,
-                             lanes_shift(L.A.n, (double)L.P.nnz / std::max(L.A.n, 1)));
+                             lanes_shift(L.A.n, (double)L.P.nnz / std::max(L.A.n, 1), fp32));
             T.PT = build_sell(ar, L.PT, N.A.n, N.crow, inv[l], L.A.n, {0, N.A.n}, fp32, nullptr, nullptr, s,
-                              lanes_shift(N.A.n, (double)L.PT.nnz / std::max(N.A.n, 1)));
+                              lanes_shift(N.A.n, (double)L.PT.nnz / std::max(N.A.n, 1), fp32));
         }
         if (bf16) {
             to_bf16(ar, T.A, s);
@@ -376,7 +380,7 @@ void build_solve_layout(vemg_hierarchy *h, cudaStream_t s) {
         h->Aop = build_sell(ar, h->A, n, s2n, n2s, n, {0, n}, false, nullptr, nullptr, s);
         h->Enon = build_sell(ar, h->E, n - mt, s2n + mt, surf_inv, mt, {0, n - mt}, false, nullptr, nullptr, s);
         h->ETs = build_sell(ar, h->ET, mt, h->surf.lv[0].crow, n2s, n, {0, mt}, false, nullptr, nullptr, s,
-                            lanes_shift(mt, (double)h->ET.nnz / std::max(mt, 1)));
+                            lanes_shift(mt, (double)h->ET.nnz / std::max(mt, 1), false));
         if (fp32 && h->Enon.padded > 0) {
             // z = E~ y_s + x_bar is formed in FP32 when the V-cycles are FP32 (one conversion per row)
             h->Enon_vf = ar.alloc<float>(h->Enon.padded);

@@ -46,7 +46,7 @@ struct TuneScope {
 // per-column scalar slots (sc[slot * K + c])
 enum {
     B_RZ = 0, B_PQ, B_ALPHA, B_BETA, B_MU, B_BN, B_RN, B_FLAG, B_ITERS, B_CONV, B_ZERO, B_TRUE, B_BMEAN, B_XMEAN,
-    B_TOL, B_MAXIT, B_FRESH, B_BEST, B_LASTIMP, B_STALL, B_COUNT
+    B_TOL, B_MAXIT, B_FRESH, B_BEST, B_LASTIMP, B_STALL, B_SUMR, B_SUMQ, B_COUNT
 };
 
 // a column whose best residual has not dropped by 1% in this many iterations has reached the
@@ -358,10 +358,19 @@ static void bsweep(const BLevel &L, const BT *b, XT *x, bool forward, bool from_
     }
 }
 
+// an event recorded where the cycle of a chain enters a level (k_blate's start)
+struct BMark {
+    const BChain *C = nullptr;
+    int level = 0;
+    cudaEvent_t ev = nullptr;
+};
+static thread_local BMark b_mark;
+
 template <class XT, class BT>
 static void bvcycle(const BChain &C, BatchWork *W, int ch, int l, const BT *b, XT *x, cudaStream_t s) {
     const BLevel &L = C.lv[l];
     const int K = W->K;
+    if (b_mark.C == &C && l == b_mark.level) VEMG_CHECK_CUDA(cudaEventRecord(b_mark.ev, s));
     if (l == C.nlev - 1) {
         if (C.direct) {
             const XT *G = sizeof(XT) == sizeof(float) ? (const XT *)C.Gf : (const XT *)C.G;
@@ -379,7 +388,11 @@ static void bvcycle(const BChain &C, BatchWork *W, int ch, int l, const BT *b, X
     const BLevel &N = C.lv[l + 1];
     const XT *none = nullptr;
     bsweep<XT, BT>(L, b, x, true, true, K, s);
-    brow<BOP_UPPER, P, XT, XT, XT, XT, XT>(L.A, L.n, nullptr, ROW_UPPER, none, none, x, r, K, -1, s);
+    // a warp's rows end together in sweep order (rows of one colour have about as many entries of later
+    // ones): used while the vector stays in L2 over the passes of the colours; else in row order
+    const bool sweep_order = (double)L.n * K * sizeof(XT) <= 64.0 * 1048576.0;
+    brow<BOP_UPPER, P, XT, XT, XT, XT, XT>(L.A, L.n, sweep_order ? L.A.info : nullptr, ROW_UPPER, none, none, x, r, K,
+                                           -1, s);
     brow<BOP_SPMV, P, XT, XT, XT, XT, XT>(L.PT, N.n, nullptr, ROW_ALL, none, none, r, nb, K, -1, s);
     bvcycle<XT, XT>(C, W, ch, l + 1, (const XT *)nb, nx, s);
     brow<BOP_SPMV_ADD, P, XT, XT, XT, XT, XT>(L.P, L.n, nullptr, ROW_ALL, none, none, nx, x, K, -1, s);
@@ -450,9 +463,9 @@ __global__ void __launch_bounds__(kBT) k_bsums(int64_t N, int K, BSums d, double
     bblock_partials<NS>(acc, K, part);
 }
 
-// the preconditioner's sums over z, r (and q): s0 = sum z, s1 = sum r z, s2 = sum r
-// [, s3 = sum z q, s4 = sum q]; each vector is loaded once per element. FP64 bounds it: five
-// multiply-adds an element (one: 1.0, see dadd).
+// the preconditioner's sums over z, r (and q): s0 = sum z, s1 = sum r z [, s2 = sum z q] (k_blate has those
+// of r and q); each vector is loaded once per element. FP64 and memory bound it: a multiply-add a sum
+// (one: 1.0, see dadd).
 template <int NS>
 __global__ void __launch_bounds__(kBT, 2) k_bsums_zrq(int64_t N, int K, const double *__restrict__ z,
                                                       const double *__restrict__ r, const double *__restrict__ q,
@@ -468,46 +481,36 @@ __global__ void __launch_bounds__(kBT, 2) k_bsums_zrq(int64_t N, int K, const do
             int64_t e = base + (int64_t)j * kBT;
             vz[j] = e < N ? z[e] : 0.0;
             vr[j] = e < N ? r[e] : 0.0;
-            vq[j] = (NS == 5 && e < N) ? q[e] : 0.0;
+            vq[j] = (NS == 3 && e < N) ? q[e] : 0.0;
         }
 #pragma unroll
         for (int j = 0; j < kBE; ++j) {
             acc[0] = dadd(acc[0], vz[j], one);
             acc[1] = fma(vr[j], vz[j], acc[1]);
-            acc[2] = dadd(acc[2], vr[j], one);
-            if (NS == 5) {
-                acc[3] = fma(vz[j], vq[j], acc[3]);
-                acc[4] = dadd(acc[4], vq[j], one);
-            }
+            if (NS == 3) acc[NS - 1] = fma(vz[j], vq[j], acc[NS - 1]);
         }
     }
     bblock_partials<NS>(acc, K, part);
 }
 
-enum { ST_MEAN_B = 0, ST_BN, ST_ALPHA, ST_RN, ST_BETA, ST_MEAN_X, ST_TRUE };
+enum { ST_MEAN_B = 0, ST_BN, ST_ALPHA, ST_RN, ST_BETA, ST_MEAN_X, ST_TRUE, ST_LATE };
 
-// stage 2: one block per column
+// stage 2: one block per column, one warp per sum
 __global__ void __launch_bounds__(256) k_bstage2(int op, int nblk, int ns, int K, const double *__restrict__ part,
                                                 double *sc, double inv_n, int neumann, int flexible, int first,
                                                 unsigned *ctr, int *active, cudaGraphConditionalHandle handle,
                                                 int use_cond) {
-    __shared__ double red[256 / 32];
+    pdl_begin();
     __shared__ double tot[5];
-    const int c = blockIdx.x, t = threadIdx.x;
-    for (int s = 0; s < ns; ++s) {
+    const int c = blockIdx.x, t = threadIdx.x, warp = t >> 5;
+    if (warp < ns) {
         double v = 0.0;
-        for (int k = t; k < nblk; k += 256) v += part[((int64_t)k * ns + s) * K + c];
+        for (int k = t & 31; k < nblk; k += 32) v += part[((int64_t)k * ns + warp) * K + c];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((t & 31) == 0) red[t >> 5] = v;
-        __syncthreads();
-        if (t == 0) {
-            double w = 0.0;
-            for (int i = 0; i < 256 / 32; ++i) w += red[i];
-            tot[s] = w;
-        }
-        __syncthreads();
+        if ((t & 31) == 0) tot[warp] = v;
     }
+    __syncthreads();
     double *g = sc + B_COUNT * K;
     if (t == 0) {
         // converged, broken down, or out of iterations: frozen while other columns continue
@@ -517,6 +520,10 @@ __global__ void __launch_bounds__(256) k_bstage2(int op, int nblk, int ns, int K
             case ST_MEAN_B: sc[B_BMEAN * K + c] = tot[0] * inv_n; break;
             case ST_MEAN_X: sc[B_XMEAN * K + c] = tot[0] * inv_n; break;
             case ST_TRUE: sc[B_TRUE * K + c] = sqrt(tot[0]); break;
+            case ST_LATE:
+                sc[B_SUMR * K + c] = tot[0];
+                if (ns > 1) sc[B_SUMQ * K + c] = tot[1];
+                break;
             case ST_BN: {
                 double bn = sqrt(tot[0]);
                 sc[B_BN * K + c] = bn;
@@ -576,12 +583,12 @@ __global__ void __launch_bounds__(256) k_bstage2(int op, int nblk, int ns, int K
             }
             case ST_BETA: {
                 double mu = neumann ? tot[0] * inv_n : 0.0;
-                double rz = tot[1] - mu * tot[2];
+                double rz = tot[1] - mu * sc[B_SUMR * K + c];
                 double beta = 0.0;
                 const bool fresh = sc[B_FRESH * K + c] != 0.0;
                 sc[B_FRESH * K + c] = 0.0;
                 if (!fresh && !frozen) {
-                    if (flexible) beta = -(tot[3] - mu * tot[4]) / sc[B_PQ * K + c];
+                    if (flexible) beta = -(tot[2] - mu * sc[B_SUMQ * K + c]) / sc[B_PQ * K + c];
                     else beta = rz / sc[B_RZ * K + c];
                     if (!(rz == rz) || !(beta == beta)) sc[B_FLAG * K + c] = 1.0;
                 }
@@ -610,27 +617,25 @@ __global__ void k_bprepare(int64_t N, int K, int neumann, double *__restrict__ b
     p[e] = 0.0;
 }
 
-// X += alpha P, R -= alpha Q per column, the FP32 copy of R's A_bar part, and the stage-1 sums
-// of R * R (elements of a thread and order as in k_bsums)
-__global__ void __launch_bounds__(kBT, 2) k_bupdate_xr(int64_t N, int K, const double *__restrict__ p,
-                                                       const double *__restrict__ q, double *__restrict__ x,
-                                                       double *__restrict__ r, const double *__restrict__ sc,
-                                                       float *__restrict__ rb32, int64_t off32, double *part) {
+// R -= alpha Q per column, the FP32 copy of R's A_bar part, and the stage-1 sums of R * R (elements of a
+// thread and order as in k_bsums)
+__global__ void __launch_bounds__(kBT, 2) k_bupdate_r(int64_t N, int K, const double *__restrict__ q,
+                                                      double *__restrict__ r, const double *__restrict__ sc,
+                                                      float *__restrict__ rb32, int64_t off32, double *part) {
     pdl_begin();
     double acc[1] = {0.0};
     const double a = sc[B_ALPHA * K + (int)(threadIdx.x & (K - 1))];   // kBT is a multiple of K: one column
     for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
-        double vp[kBE], vq[kBE], vx[kBE], vr[kBE];
+        double vq[kBE], vr[kBE];
 #pragma unroll
         for (int j = 0; j < kBE; ++j) {
             const int64_t e = base + (int64_t)j * kBT;
-            if (e < N) { vp[j] = p[e]; vq[j] = q[e]; vx[j] = x[e]; vr[j] = r[e]; }
+            if (e < N) { vq[j] = q[e]; vr[j] = r[e]; }
         }
 #pragma unroll
         for (int j = 0; j < kBE; ++j) {
             const int64_t e = base + (int64_t)j * kBT;
             if (e >= N) continue;
-            x[e] = fma(a, vp[j], vx[j]);
             const double rn = fma(-a, vq[j], vr[j]);
             r[e] = rn;
             if (rb32 && e >= off32) rb32[e - off32] = cvt_f32(rn);
@@ -638,6 +643,39 @@ __global__ void __launch_bounds__(kBT, 2) k_bupdate_xr(int64_t N, int K, const d
         }
     }
     bblock_partials<1>(acc, K, part);
+}
+
+// What an iteration owes that nothing before the next z needs, on the side stream beside the coarse levels
+// (as k_late of the one-column solve): X += alpha P and the stage-1 sums of R and, NS = 2, of Q. NS = 0:
+// X alone. After any iteration the solution of a column is X + alpha P.
+template <int NS>
+__global__ void __launch_bounds__(kBT, 2) k_blate(int64_t N, int K, const double *__restrict__ p, double *__restrict__ x,
+                                                  const double *__restrict__ r, const double *__restrict__ q,
+                                                  const double *__restrict__ sc, double *part, double one) {
+    pdl_begin();
+    double acc[NS > 0 ? NS : 1] = {};
+    const double a = sc[B_ALPHA * K + (int)(threadIdx.x & (K - 1))];
+    for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
+        double vp[kBE], vx[kBE], vr[kBE], vq[kBE];
+#pragma unroll
+        for (int j = 0; j < kBE; ++j) {
+            const int64_t e = base + (int64_t)j * kBT;
+            if (e >= N) continue;
+            vp[j] = p[e];
+            vx[j] = x[e];
+            if (NS > 0) vr[j] = r[e];
+            if (NS > 1) vq[j] = q[e];
+        }
+#pragma unroll
+        for (int j = 0; j < kBE; ++j) {
+            const int64_t e = base + (int64_t)j * kBT;
+            if (e >= N) continue;
+            x[e] = fma(a, vp[j], vx[j]);
+            if (NS > 0) acc[0] = dadd(acc[0], vr[j], one);
+            if (NS > 1) acc[NS - 1] = dadd(acc[NS - 1], vq[j], one);
+        }
+    }
+    if constexpr (NS > 0) bblock_partials<NS>(acc, K, part);
 }
 
 // z += x (assign: z = x)
@@ -677,24 +715,45 @@ __global__ void k_binit(double *sc, int K, double tol, int maxit) {
     g[G_MAXIT] = (double)maxit;
 }
 
-// gather k caller-order columns (column c at B[c * ldb]) into the interleaved solve-order block
-__global__ void k_bgather(int nu, int K, int k, int64_t ldb, const int *__restrict__ caller_of,
-                          const double *__restrict__ Bin, double *__restrict__ Bk) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= (int64_t)nu * K) return;
-    int i = (int)(t >> (__ffs(K) - 1)), c = (int)(t & (K - 1));
-    Bk[t] = c < k ? Bin[(int64_t)c * ldb + caller_of[i]] : 0.0;
+// Between k caller-order columns (column c at [c * ld]) and the interleaved block, 32 rows by up to 32
+// columns at a time through shared memory, so that both sides move whole sectors (the caller's order
+// keeps runs of the internal one). The block's columns past k are zeros.
+static constexpr int kTile = 32;
+
+__global__ void __launch_bounds__(256) k_bgather(int nu, int K, int k, int64_t ldb, const int *__restrict__ caller_of,
+                                                 const double *__restrict__ Bin, double *__restrict__ Bk) {
+    __shared__ double tile[kTile][kTile + 1];
+    const int i0 = blockIdx.x * kTile, c0 = blockIdx.y * kTile, W = min(K - c0, kTile);
+    for (int e = threadIdx.x; e < kTile * W; e += 256) {
+        const int i = e % kTile, c = e / kTile;
+        tile[i][c] = i0 + i < nu && c0 + c < k ? Bin[(int64_t)(c0 + c) * ldb + caller_of[i0 + i]] : 0.0;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kTile * W; e += 256) {
+        const int i = e / W, c = e % W;
+        if (i0 + i < nu) Bk[(int64_t)(i0 + i) * K + c0 + c] = tile[i][c];
+    }
 }
 
-__global__ void k_bscatter(int nu, int K, int k, int64_t ldx, const int *__restrict__ caller_of,
-                           const int *__restrict__ tops, int ntop, const double *__restrict__ Xk,
-                           double *__restrict__ Xout) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t nmax = (int64_t)(nu > ntop ? nu : ntop) * k;
-    if (t >= nmax) return;
-    int i = (int)(t / k), c = (int)(t % k);
-    if (i < nu) Xout[(int64_t)c * ldx + caller_of[i]] = Xk[(int64_t)i * K + c];
-    if (i < ntop) Xout[(int64_t)c * ldx + tops[i]] = 0.0;
+__global__ void __launch_bounds__(256) k_bscatter(int nu, int K, int k, int64_t ldx, const int *__restrict__ caller_of,
+                                                  const double *__restrict__ Xk, double *__restrict__ Xout) {
+    __shared__ double tile[kTile][kTile + 1];
+    const int i0 = blockIdx.x * kTile, c0 = blockIdx.y * kTile, W = min(K - c0, kTile);
+    for (int e = threadIdx.x; e < kTile * W; e += 256) {
+        const int i = e / W, c = e % W;
+        if (i0 + i < nu) tile[i][c] = Xk[(int64_t)(i0 + i) * K + c0 + c];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kTile * W; e += 256) {
+        const int i = e % kTile, c = e / kTile;
+        if (i0 + i < nu && c0 + c < k) Xout[(int64_t)(c0 + c) * ldx + caller_of[i0 + i]] = tile[i][c];
+    }
+}
+
+// Dirichlet top: x = 0 on the top nodes
+__global__ void k_btops(int ntop, int k, int64_t ldx, const int *__restrict__ tops, double *__restrict__ Xout) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t < (int64_t)ntop * k) Xout[(t / ntop) * ldx + tops[t % ntop]] = 0.0;
 }
 
 __global__ void k_bcond_init(const double *g, cudaGraphConditionalHandle handle) {
@@ -704,12 +763,52 @@ __global__ void k_bcond_init(const double *g, cudaGraphConditionalHandle handle)
 // ------------------------------------------------------------------------------------------
 // the batched iteration
 
+static void bstage2(vemg_hierarchy *h, BatchWork *W, int op, int ns, int64_t N, int first, cudaStream_t s,
+                    cudaGraphConditionalHandle hd = 0, int use_cond = 0) {
+    pdl_launch(k_bstage2, W->K, 256, s, op, stage1_blocks(N), ns, W->K, (const double *)W->part, W->sc,
+               1.0 / (double)h->nu, (int)(h->bc == VEMG_NEUMANN), (int)(h->precision != VEMG_PREC_FP64), first, W->ctr,
+               (int *)(W->ctr + 1), hd, use_cond);
+    BATCH_LAUNCHED();
+}
+
+// k_blate and its stage 2 on stream s (the cycle uses no partials)
+static void blate(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
+    const int64_t N = (int64_t)h->nu * W->K;
+    const bool flex = h->precision != VEMG_PREC_FP64;
+    if (flex)
+        pdl_launch(k_blate<2>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->P, W->X, (const double *)W->R,
+                   (const double *)W->Q, (const double *)W->sc, W->part, 1.0);
+    else
+        pdl_launch(k_blate<1>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->P, W->X, (const double *)W->R,
+                   (const double *)nullptr, (const double *)W->sc, W->part, 1.0);
+    BATCH_LAUNCHED();
+    bstage2(h, W, ST_LATE, flex ? 2 : 1, N, 0, s);
+}
+
 template <class XT>
 static void bprecond(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     const int K = W->K;
     const bool two = !single_chain(h);
     const int mt = two ? h->mtop : 0;
     XT *xb = (XT *)W->lx[1][0];
+    // k_blate starts where the A_bar cycle enters its first level of at most an eighth of the rows
+    const BChain &B = *W->bbar;
+    int lv = 0;
+    while (lv + 1 < B.nlev && (int64_t)B.lv[lv].n * 8 > B.lv[0].n) ++lv;
+    auto cycle = [&](auto *b) {
+        b_mark = BMark{&B, lv, h->ev_mid};
+        try {
+            bvcycle<XT>(B, W, 1, 0, b, xb, s);
+        } catch (...) {
+            b_mark = BMark{};
+            throw;
+        }
+        b_mark = BMark{};
+        VEMG_CHECK_CUDA(cudaStreamWaitEvent(h->side, h->ev_mid, 0));
+        blate(h, W, h->side);
+        VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
+        VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
+    };
     if (two) {
         XT *b0 = (XT *)W->lb[0][0], *x0 = (XT *)W->lx[0][0];
         VEMG_CHECK_CUDA(cudaEventRecord(h->ev_fork, s));
@@ -719,14 +818,8 @@ static void bprecond(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
                                                                   (const double *)nullptr, (const double *)nullptr,
                                                                   W->R, b0, K, -1, h->side, 2);
         bvcycle<XT, XT>(*W->bsurf, W, 0, 0, (const XT *)b0, x0, h->side);
-        VEMG_CHECK_CUDA(cudaEventRecord(h->ev_join, h->side));
-        const int64_t nbk = (int64_t)(h->n - mt) * K;
-        if (std::is_same<XT, float>::value && W->Rb32) {   // kept current by every writer of r
-            bvcycle<XT, XT>(*W->bbar, W, 1, 0, (const XT *)W->Rb32, xb, s);
-        } else {
-            bvcycle<XT, double>(*W->bbar, W, 1, 0, W->R + (int64_t)mt * K, xb, s);
-        }
-        VEMG_CHECK_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
+        if constexpr (std::is_same<XT, float>::value) cycle((const float *)W->Rb32);   // kept current by every writer of r
+        else cycle((const double *)W->R + (int64_t)mt * K);
         // z = E~ y_s + [0; x_bar]: with FP32 V-cycles formed in FP32 from x_bar on and converted
         // once into the FP64 z; with FP64 ones in FP64
         if constexpr (std::is_same<XT, float>::value) {
@@ -738,11 +831,12 @@ static void bprecond(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
                                                                           (const double *)nullptr,
                                                                           (const double *)nullptr, x0, W->Z, K, -1, s,
                                                                           2);
+            const int64_t nbk = (int64_t)(h->n - mt) * K;
             pdl_launch(k_badd<XT>, grid_for(nbk, 256), 256, s, nbk, (const XT *)xb, W->Z + (int64_t)mt * K, 0);
             BATCH_LAUNCHED();
         }
     } else {
-        bvcycle<XT, double>(*W->bbar, W, 1, 0, W->R, xb, s);
+        cycle((const double *)W->R);
         int64_t N = (int64_t)h->nu * K;
         pdl_launch(k_badd<XT>, grid_for(N, 256), 256, s, N, (const XT *)xb, W->Z, 1);
         BATCH_LAUNCHED();
@@ -761,27 +855,19 @@ static void bsums(BatchWork *W, int64_t N, const BSums &d, cudaStream_t s) {
     BATCH_LAUNCHED();
 }
 
-static void bstage2(vemg_hierarchy *h, BatchWork *W, int op, int ns, int64_t N, int first, cudaStream_t s,
-                    cudaGraphConditionalHandle hd = 0, int use_cond = 0) {
-    k_bstage2<<<W->K, 256, 0, s>>>(op, stage1_blocks(N), ns, W->K, W->part, W->sc, 1.0 / (double)h->nu,
-                                   h->bc == VEMG_NEUMANN, h->precision != VEMG_PREC_FP64, first, W->ctr,
-                                   (int *)(W->ctr + 1), hd, use_cond);
-    BATCH_LAUNCHED();
-}
-
 static void bprecond_any(vemg_hierarchy *h, BatchWork *W, int first, cudaStream_t s) {
     if (h->precision != VEMG_PREC_FP64) bprecond<float>(h, W, s);   // BF16 hierarchies: FP32 values here
     else bprecond<double>(h, W, s);
-    // t0 = sum z, t1 = (r, z), t2 = sum r [, t3 = (z, q), t4 = sum q]
+    // t0 = sum z, t1 = (r, z) [, t2 = (z, q)]
     int64_t N = (int64_t)h->nu * W->K;
     bool flex = h->precision != VEMG_PREC_FP64;
     (void)first;
-    const int ns = flex ? 5 : 3;
+    const int ns = flex ? 3 : 2;
     if (flex)
-        pdl_launch(k_bsums_zrq<5>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
+        pdl_launch(k_bsums_zrq<3>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
                    (const double *)W->Q, W->part, 1.0);
     else
-        pdl_launch(k_bsums_zrq<3>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
+        pdl_launch(k_bsums_zrq<2>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
                    (const double *)nullptr, W->part, 1.0);
     BATCH_LAUNCHED();
     bstage2(h, W, ST_BETA, ns, N, first, s);
@@ -816,8 +902,8 @@ static void bphase_step(vemg_hierarchy *h, BatchWork *W, cudaStream_t s, cudaGra
         bsums(W, N, d, s);
         bstage2(h, W, ST_ALPHA, 1, N, 0, s);
     }
-    pdl_launch(k_bupdate_xr, stage1_blocks(N), kBT, s, N, K, (const double *)W->P, (const double *)W->Q, W->X, W->R,
-               (const double *)W->sc, W->Rb32, rb32_offset(h, W), W->part);
+    pdl_launch(k_bupdate_r, stage1_blocks(N), kBT, s, N, K, (const double *)W->Q, W->R, (const double *)W->sc, W->Rb32,
+               rb32_offset(h, W), W->part);
     BATCH_LAUNCHED();
     bstage2(h, W, ST_RN, 1, N, 0, s, hd, use_cond);
 }
@@ -832,6 +918,9 @@ static void bphase_direction(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
 static void bphase_post(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     const int K = W->K, nu = h->nu;
     const int64_t N = (int64_t)nu * K;
+    pdl_launch(k_blate<0>, stage1_blocks(N), kBT, s, N, K, (const double *)W->P, W->X, (const double *)nullptr,
+               (const double *)nullptr, (const double *)W->sc, W->part, 1.0);
+    BATCH_LAUNCHED();
     if (h->bc == VEMG_NEUMANN) {
         BSums d{{W->X}, {nullptr}, 1};
         bsums(W, N, d, s);
@@ -977,15 +1066,15 @@ __global__ void k_brows_info(int n, const int *__restrict__ crow, const int *__r
     info[i] = make_int4(r, rp[r] - r, lo[r], rp[r + 1] - rp[r] - 1);
 }
 
-// Parts a row is split into: where the rows of one launch do not fill half the chip (152 SMs x 2048
-// threads), a launch lasts as long as a row's chain of loads, which parts of about four entries cut. A
+// Parts a row is split into: where the rows of one launch do not fill a quarter of the chip (152 SMs x 2048
+// threads; half or an eighth of it measured 2 to 5% slower), a launch lasts as long as a row's chain of loads, which parts of about four entries cut. A
 // warp must hold a row's parts at every launch shape, up to 32 lanes a row; the lanes that the widest
 // loads would take count here, so that the parts (and with them the sums' order) do not depend on the
 // shape.
 static int parts_shift(int K, bool fp32, double rows, double mean) {
     const double lanes = std::max(1, K / (fp32 ? 4 : 2));
     int qsh = 0;
-    while (std::min(K, 32) << (qsh + 1) <= 32 && mean > 4.0 * (1 << qsh) && rows * lanes * (2 << qsh) <= 152.0 * 1024.0)
+    while (std::min(K, 32) << (qsh + 1) <= 32 && mean > 4.0 * (1 << qsh) && rows * lanes * (2 << qsh) <= 152.0 * 512.0)
         ++qsh;
     return qsh;
 }
@@ -1215,7 +1304,8 @@ int solve_batch(vemg_hierarchy *h, int k, const double *Bin, int64_t ldb, double
     const int nu = h->nu;
     k_binit<<<1, 1, 0, s>>>(W->sc, K, rtol, max_it);
     BATCH_LAUNCHED();
-    k_bgather<<<grid_for((int64_t)nu * K, 256), 256, 0, s>>>(nu, K, k, ldb, W->caller_of, Bin, W->B);
+    const unsigned tiles = (unsigned)((nu + kTile - 1) / kTile), across = (unsigned)((K + kTile - 1) / kTile);
+    k_bgather<<<dim3(tiles, across), 256, 0, s>>>(nu, K, k, ldb, W->caller_of, Bin, W->B);
     BATCH_LAUNCHED();
     // with a probe on, the same phases are launched on the stream (profilers see every kernel)
     const bool use_graph = h->probe.kind == PROBE_NONE;
@@ -1238,9 +1328,12 @@ int solve_batch(vemg_hierarchy *h, int k, const double *Bin, int64_t ldb, double
     std::vector<double> hs(B_COUNT * K + G_COUNT);
     VEMG_CHECK_CUDA(cudaMemcpyAsync(hs.data(), W->sc, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s));
     int ntop = h->bc == VEMG_DIRICHLET_TOP ? h->mtop : 0;
-    int64_t nsc = (int64_t)std::max(nu, ntop) * k;
-    k_bscatter<<<grid_for(nsc, 256), 256, 0, s>>>(nu, K, k, ldx, W->caller_of, h->tops, ntop, W->X, Xout);
+    k_bscatter<<<dim3(tiles, across), 256, 0, s>>>(nu, K, k, ldx, W->caller_of, W->X, Xout);
     BATCH_LAUNCHED();
+    if (ntop > 0) {
+        k_btops<<<grid_for((int64_t)ntop * k, 256), 256, 0, s>>>(ntop, k, ldx, h->tops, Xout);
+        BATCH_LAUNCHED();
+    }
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     int rounds = (int)hs[B_COUNT * K + G_ITERS];
     if (use_graph) h->launches += G->k_pre + G->k_post + (int64_t)rounds * G->k_body;
@@ -1286,12 +1379,15 @@ struct Engine {
 
 static constexpr int kColBlocks = 128;
 
-// sum over rows of column c of a (or of a^2); per-block partials
-__global__ void k_col_sum(int n, int K, int c, const double *__restrict__ a, int square, double *part) {
+// sum over rows of column c of a (or of a^2; with p: of a + alpha p); per-block partials
+__global__ void k_col_sum(int n, int K, int c, const double *__restrict__ a, int square, double *part,
+                          const double *__restrict__ p = nullptr, const double *__restrict__ sc = nullptr) {
     __shared__ double sh[256];
     double v = 0.0;
+    const double alpha = p ? sc[B_ALPHA * K + c] : 0.0;
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += kColBlocks * 256) {
         double x = a[(int64_t)i * K + c];
+        if (p) x = fma(alpha, p[(int64_t)i * K + c], x);
         v += square ? x * x : x;
     }
     sh[threadIdx.x] = v;
@@ -1353,12 +1449,13 @@ __global__ void k_col_mean(int K, int c, const double *__restrict__ part, double
     sc[B_XMEAN * K + c] = t * inv_n;
 }
 
+// x = X + alpha P - mean of column c in the caller's order
 __global__ void k_col_scatter(int nu, int K, int c, int neumann, const int *__restrict__ caller_of,
                               const int *__restrict__ tops, int ntop, const double *__restrict__ sc,
-                              const double *__restrict__ X, double *__restrict__ x) {
+                              const double *__restrict__ X, const double *__restrict__ P, double *__restrict__ x) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double mu = neumann ? sc[B_XMEAN * K + c] : 0.0;
-    if (i < nu) x[caller_of[i]] = X[(int64_t)i * K + c] - mu;
+    const double mu = neumann ? sc[B_XMEAN * K + c] : 0.0, alpha = sc[B_ALPHA * K + c];
+    if (i < nu) x[caller_of[i]] = fma(alpha, P[(int64_t)i * K + c], X[(int64_t)i * K + c]) - mu;
     if (i < ntop) x[tops[i]] = 0.0;
 }
 
@@ -1573,14 +1670,14 @@ int vemg_engine_retire(vemg_engine *e, int slot, double *x_dev) {
         const bool neu = h->bc == VEMG_NEUMANN;
         cudaStream_t s = e->s;
         if (neu) {
-            k_col_sum<<<kColBlocks, 256, 0, s>>>(nu, K, slot, W->X, 0, e->colpart);
+            k_col_sum<<<kColBlocks, 256, 0, s>>>(nu, K, slot, W->X, 0, e->colpart, W->P, W->sc);
             VEMG_CHECK_LAUNCH();
             k_col_mean<<<1, 1, 0, s>>>(K, slot, e->colpart, 1.0 / nu, W->sc);
             VEMG_CHECK_LAUNCH();
         }
         int ntop = neu ? 0 : h->mtop;
         k_col_scatter<<<grid_for(std::max(nu, ntop), 256), 256, 0, s>>>(nu, K, slot, neu, W->caller_of, h->tops, ntop,
-                                                                         W->sc, W->X, x_dev);
+                                                                         W->sc, W->X, W->P, x_dev);
         VEMG_CHECK_LAUNCH();
         k_col_free<<<grid_for(nu, 256), 256, 0, s>>>(nu, K, slot, W->sc, W->B, W->R, W->X, W->P, W->Rb32,
                                                      rb32_offset(h, W));

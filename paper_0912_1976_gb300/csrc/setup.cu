@@ -277,6 +277,65 @@ __global__ void k_sort_rows_kv(const int *__restrict__ rp, int *ci, double *v, i
     }
 }
 
+// Levels of at most this many rows take the forms below with a warp per row instead of a thread: a
+// thread's walk of its row is a chain of loads, and there are too few rows to hide it (77K rows: the
+// products of a 44 x 44 x 24 mesh's coarse levels took 760 us each with a thread per row).
+static constexpr int kWarpRows = 152 * 1024;
+static constexpr int kRowWarps = 4;    // warps per block of these
+
+// the same sort by ranks, stable as well: rows of at most 32 kSortMost entries in registers, a longer one
+// by its warp's first thread as above
+static constexpr int kSortMost = 8;
+__global__ void __launch_bounds__(32 * kRowWarps) k_sort_rows_warp(const int *__restrict__ rp, int *ci, double *v, int n) {
+    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const int lo = rp[i], len = rp[i + 1] - lo;
+    if (len > 32 * kSortMost) {
+        if (lane == 0)
+            for (int k = lo + 1; k < lo + len; ++k) {
+                int x = ci[k];
+                double y = v[k];
+                int j = k - 1;
+                while (j >= lo && ci[j] > x) { ci[j + 1] = ci[j]; v[j + 1] = v[j]; --j; }
+                ci[j + 1] = x;
+                v[j + 1] = y;
+            }
+        return;
+    }
+    int key[kSortMost], rank[kSortMost];
+    double val[kSortMost];
+#pragma unroll
+    for (int u = 0; u < kSortMost; ++u) {
+        const int e = lane + 32 * u;
+        key[u] = e < len ? ci[lo + e] : 0x7fffffff;
+        val[u] = e < len ? v[lo + e] : 0.0;
+        rank[u] = 0;
+    }
+#pragma unroll
+    for (int u = 0; u < kSortMost; ++u) {
+        if (32 * u >= len) break;
+        for (int l = 0; l < 32 && 32 * u + l < len; ++l) {
+            const int c = __shfl_sync(0xffffffffu, key[u], l);
+#pragma unroll
+            for (int w = 0; w < kSortMost; ++w)
+                rank[w] += c < key[w] || (c == key[w] && l + 32 * u < lane + 32 * w);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < kSortMost; ++u)
+        if (lane + 32 * u < len) {
+            ci[lo + rank[u]] = key[u];
+            v[lo + rank[u]] = val[u];
+        }
+}
+
+static void sort_rows(const int *rp, int *ci, double *v, int n, cudaStream_t s) {
+    if (n <= kWarpRows) k_sort_rows_warp<<<grid_for(n, kRowWarps), 32 * kRowWarps, 0, s>>>(rp, ci, v, n);
+    else k_sort_rows_kv<<<grid_for(n, 128), 128, 0, s>>>(rp, ci, v, n);
+    VEMG_CHECK_LAUNCH();
+}
+
 struct Incidence {
     int *ptr = nullptr, *inc = nullptr;
     void release() {
@@ -338,29 +397,75 @@ __global__ void k_asm_rowfill(int n, const int *__restrict__ iptr, const int *__
     for (int k = 0; k < cnt; ++k) ci[rp[i] + k] = nb[k];
 }
 
-// A_ij = sum over the elements holding i and j, in ascending element index, of K_e[a][b]
-__global__ void k_asm_values(int n, const int *__restrict__ iptr, const int *__restrict__ inc,
-                             const int *__restrict__ tets, const double *__restrict__ xyz,
-                             const int *__restrict__ rp, const int *__restrict__ ci, double *v, int *err) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int lo = rp[i], hi = rp[i + 1];
-    for (int k = lo; k < hi; ++k) v[k] = 0.0;
-    for (int k = iptr[i]; k < iptr[i + 1]; ++k) {
-        const int *t = tets + 4 * (int64_t)inc[k];
-        int vv[4] = {t[0], t[1], t[2], t[3]};
-        Tet T;
-        tet_geometry(xyz, vv, T);
-        if (!(T.det > 0.0)) { atomic_flag(err, VEMG_EMESH); return; }
-        int a = 0;
-        while (vv[a] != i) ++a;
-        double s = 6.0 * T.det;
-        for (int b = 0; b < 4; ++b) {
-            double kab = dot3(T.c[a], T.c[b]) / s;
-            int pos = bsearch_row(ci, lo, hi, vv[b]);
-            v[pos] = v[pos] + kab;
+// The element matrices, one thread per element: the ten entries K[a][b], a <= b, of element e in ke[10 e ..],
+// row by row. FP64 bounds it (some 190 operations, ten of them divisions): 4.7 ms of 12.6M elements. With
+// every node of an element computing it again, the values took 11.4 ms.
+__global__ void __launch_bounds__(128) k_asm_elements(int64_t ne, const int *__restrict__ tets,
+                                                      const double *__restrict__ xyz, double *__restrict__ ke, int *err) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= ne) return;
+    const int4 t = *(const int4 *)(tets + 4 * e);
+    const int vv[4] = {t.x, t.y, t.z, t.w};
+    Tet T;
+    tet_geometry(xyz, vv, T);
+    if (!(T.det > 0.0)) { atomic_flag(err, VEMG_EMESH); return; }
+    const double s = 6.0 * T.det;
+    double *k = ke + 10 * e;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = a; b < 4; ++b) *k++ = dot3(T.c[a], T.c[b]) / s;
+}
+
+// A_ij = sum over the elements holding i and j, in ascending element index, of K_e[a][b]. Four lanes per
+// row, one for each vertex of the element at hand (different columns, so the order of the sums is that
+// of the elements); a block's rows are one segment of A, summed up in shared memory if it fits there.
+// Four elements' vertices and values are on their way at once: a thread per row, one element after the
+// other and the sums in global memory, took 6.5 ms of 12.6M elements.
+static constexpr int kAsmRows = 32, kAsmMost = 32 * kAsmRows;
+__global__ void __launch_bounds__(4 * kAsmRows) k_asm_values(int n, const int *__restrict__ iptr,
+                                                             const int *__restrict__ inc, const int *__restrict__ tets,
+                                                             const double *__restrict__ ke, const int *__restrict__ rp,
+                                                             const int *__restrict__ ci, double *v) {
+    __shared__ int scol[kAsmMost];
+    __shared__ double sacc[kAsmMost];
+    const int r0 = blockIdx.x * kAsmRows, base = rp[r0], len = rp[min(r0 + kAsmRows, n)] - base;
+    const bool fits = len <= kAsmMost;
+    const int *col = fits ? scol : ci + base;
+    double *acc = fits ? sacc : v + base;
+    for (int e = threadIdx.x; e < len; e += blockDim.x) {
+        if (fits) scol[e] = ci[base + e];
+        acc[e] = 0.0;
+    }
+    __syncthreads();
+    const int i = r0 + (int)(threadIdx.x >> 2), b = threadIdx.x & 3;
+    const unsigned mine = 15u << (threadIdx.x & 28);
+    if (i < n) {
+        const int lo = rp[i] - base, hi = rp[i + 1] - base, k1 = iptr[i + 1];
+        for (int k = iptr[i]; k < k1; k += 4) {
+            int e[4], pos[4];
+            int4 t[4];
+            double x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e[u] = inc[min(k + u, k1 - 1)];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[u] = *(const int4 *)(tets + 4 * (int64_t)e[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int a = t[u].x == i ? 0 : t[u].y == i ? 1 : t[u].z == i ? 2 : 3, p = min(a, b), q = max(a, b);
+                x[u] = ke[10 * (int64_t)e[u] + p * (9 - p) / 2 + q - p];
+                pos[u] = bsearch_row(col, lo, hi, b == 0 ? t[u].x : b == 1 ? t[u].y : b == 2 ? t[u].z : t[u].w);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (k + u < k1) acc[pos[u]] = acc[pos[u]] + x[u];
+                __syncwarp(mine);
+            }
         }
     }
+    __syncthreads();
+    if (fits)
+        for (int e = threadIdx.x; e < len; e += blockDim.x) v[base + e] = sacc[e];
 }
 
 // b = M f: (M_e f)_a = V/20 (f_a + sum_b f_b), elements in ascending index
@@ -416,6 +521,7 @@ void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
         int n = md.n;
         I = build_incidence(md.tets, md.ne, n, s);
         Scratch<int> rowlen(n), err(1);
+        Scratch<double> ke(10 * (size_t)md.ne);
         VEMG_CHECK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         k_asm_rowlen<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, rowlen, err);
         VEMG_CHECK_LAUNCH();
@@ -426,7 +532,9 @@ void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
         double *v = (double *)dev_alloc_raw(sizeof(double) * (size_t)std::max(nnz, 1));
         k_asm_rowfill<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, rp, ci);
         VEMG_CHECK_LAUNCH();
-        k_asm_values<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, md.xyz, rp, ci, v, err);
+        k_asm_elements<<<grid_for(md.ne, 128), 128, 0, s>>>(md.ne, md.tets, md.xyz, ke, err);
+        VEMG_CHECK_LAUNCH();
+        k_asm_values<<<grid_for(n, kAsmRows), 4 * kAsmRows, 0, s>>>(n, I.ptr, I.inc, md.tets, ke, rp, ci, v);
         VEMG_CHECK_LAUNCH();
         if (int e = read_flag(err, s)) {
             dev_free_raw(rp); dev_free_raw(ci); dev_free_raw(v);
@@ -519,8 +627,7 @@ static DCsr csr_transpose(Arena &ar, const DCsr &a, cudaStream_t s) {
     VEMG_CHECK_CUDA(cudaMemcpyAsync(cur, t.rp, sizeof(int) * a.m, cudaMemcpyDeviceToDevice, s));
     k_fill_transpose<<<grid_for(a.n, 256), 256, 0, s>>>(a.n, a.rp, a.ci, a.v, cur, t.ci, t.v);
     VEMG_CHECK_LAUNCH();
-    k_sort_rows_kv<<<grid_for(t.n, 128), 128, 0, s>>>(t.rp, t.ci, t.v, t.n);
-    VEMG_CHECK_LAUNCH();
+    sort_rows(t.rp, t.ci, t.v, t.n, s);
     return t;
 }
 
@@ -579,6 +686,134 @@ __global__ void k_spgemm_num(int n, const int *__restrict__ lrp, const int *__re
     }
 }
 
+// The two with a warp per row. Columns: the candidates go into a hash set in shared memory, 32 at a time,
+// and only the distinct ones (a tenth of them) are sorted, by a bitonic network. A row of more than
+// kAccMost distinct columns is left to its warp's first thread, as above.
+static constexpr int kAccMost = 512;
+__global__ void __launch_bounds__(32 * kRowWarps) k_spgemm_sym_warp(int n, const int *__restrict__ lrp,
+                                                                    const int *__restrict__ lci,
+                                                                    const int *__restrict__ rrp,
+                                                                    const int *__restrict__ rci,
+                                                                    const int64_t *__restrict__ off, int *cand, int *ulen) {
+    constexpr int kSlots = 2 * kAccMost, kNone = 0x7fffffff;
+    __shared__ int sh[kRowWarps][kSlots];
+    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    int *out = cand + off[i], *set = sh[threadIdx.x >> 5];
+    const int lo = lrp[i], hi = lrp[i + 1];
+    for (int e = lane; e < kSlots; e += 32) set[e] = kNone;
+    __syncwarp();
+    int cnt = 0;
+    for (int k0 = lo; k0 < hi && cnt <= kAccMost; k0 += 32) {
+        // the rows that up to 32 entries refer to, one per lane
+        const int a = k0 + lane < hi ? lci[k0 + lane] : -1;
+        const int r0 = a >= 0 ? rrp[a] : 0, len = a >= 0 ? rrp[a + 1] - r0 : 0;
+        for (int l = 0; l < 32 && k0 + l < hi && cnt <= kAccMost; ++l) {
+            const int b = __shfl_sync(0xffffffffu, r0, l), w = __shfl_sync(0xffffffffu, len, l);
+            for (int q0 = 0; q0 < w && cnt <= kAccMost; q0 += 32) {
+                // at most kAccMost + 31 of the slots are taken: the probe ends
+                bool fresh = false;
+                if (q0 + lane < w) {
+                    const int c = rci[b + q0 + lane];
+                    unsigned h = ((unsigned)c * 2654435769u) >> 22;
+                    for (;;) {
+                        const int old = atomicCAS(set + h, kNone, c);
+                        fresh = old == kNone;
+                        if (fresh || old == c) break;
+                        h = (h + 1) & (kSlots - 1);
+                    }
+                }
+                cnt += __popc(__ballot_sync(0xffffffffu, fresh));
+            }
+        }
+    }
+    if (cnt > kAccMost) {
+        if (lane == 0) {
+            const int cap = (int)(off[i + 1] - off[i]);
+            cnt = 0;
+            for (int k = lo; k < hi; ++k)
+                for (int q = rrp[lci[k]]; q < rrp[lci[k] + 1]; ++q) cnt = insert_unique(out, cnt, cap, rci[q]);
+            ulen[i] = cnt;
+        }
+        return;
+    }
+    __syncwarp();
+    int m = 0;
+    for (int e0 = 0; e0 < kSlots; e0 += 32) {
+        const int c = set[e0 + lane];
+        const unsigned b = __ballot_sync(0xffffffffu, c != kNone);
+        if (c != kNone) set[m + __popc(b & ((1u << lane) - 1u))] = c;   // at or before the 32 just read
+        m += __popc(b);
+        __syncwarp();
+    }
+    int p = 1;
+    while (p < m) p *= 2;
+    for (int e = m + lane; e < p; e += 32) set[e] = kNone;
+    __syncwarp();
+    for (int size = 2; size <= p; size *= 2)
+        for (int step = size / 2; step > 0; step /= 2) {
+            for (int e = lane; e < p / 2; e += 32) {
+                const int x = 2 * e - (e & (step - 1)), y = x + step;
+                const int u = set[x], w = set[y];
+                if ((u > w) == ((x & size) == 0)) { set[x] = w; set[y] = u; }
+            }
+            __syncwarp();
+        }
+    for (int e = lane; e < m; e += 32) out[e] = set[e];
+    if (lane == 0) ulen[i] = m;
+}
+
+// Values: the rows of R one after the other, in the order of the definition; a row's entries meet
+// different entries of C, one per lane. Rows of more than kAccMost entries as in k_spgemm_num.
+__global__ void __launch_bounds__(32 * kRowWarps) k_spgemm_num_warp(int n, const int *__restrict__ lrp,
+                                                                    const int *__restrict__ lci,
+                                                                    const double *__restrict__ lv,
+                                                                    const int *__restrict__ rrp,
+                                                                    const int *__restrict__ rci,
+                                                                    const double *__restrict__ rv,
+                                                                    const int *__restrict__ crp,
+                                                                    const int *__restrict__ cci, double *cv) {
+    __shared__ double sacc[kRowWarps][kAccMost];
+    __shared__ int scol[kRowWarps][kAccMost];
+    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const int lo = crp[i], len = crp[i + 1] - lo;
+    if (len > kAccMost) {
+        if (lane == 0) {
+            for (int k = lo; k < lo + len; ++k) cv[k] = 0.0;
+            for (int k = lrp[i]; k < lrp[i + 1]; ++k)
+                for (int q = rrp[lci[k]]; q < rrp[lci[k] + 1]; ++q) {
+                    const int pos = bsearch_row(cci, lo, lo + len, rci[q]);
+                    cv[pos] = cv[pos] + lv[k] * rv[q];
+                }
+        }
+        return;
+    }
+    double *acc = sacc[threadIdx.x >> 5];
+    int *col = scol[threadIdx.x >> 5];
+    for (int e = lane; e < len; e += 32) {
+        acc[e] = 0.0;
+        col[e] = cci[lo + e];
+    }
+    __syncwarp();
+    for (int k0 = lrp[i]; k0 < lrp[i + 1]; k0 += 32) {
+        const bool on = k0 + lane < lrp[i + 1];
+        const int a = on ? lci[k0 + lane] : -1;
+        const double la = on ? lv[k0 + lane] : 0.0;
+        const int r0 = on ? rrp[a] : 0, rlen = on ? rrp[a + 1] - r0 : 0;
+        for (int l = 0; l < 32 && k0 + l < lrp[i + 1]; ++l) {
+            const int b = __shfl_sync(0xffffffffu, r0, l), w = __shfl_sync(0xffffffffu, rlen, l);
+            const double x = __shfl_sync(0xffffffffu, la, l);
+            for (int q = lane; q < w; q += 32) {
+                const int pos = bsearch_row(col, 0, len, rci[b + q]);
+                acc[pos] = acc[pos] + x * rv[b + q];
+            }
+            __syncwarp();
+        }
+    }
+    for (int e = lane; e < len; e += 32) cv[lo + e] = acc[e];
+}
+
 static DCsr csr_spgemm(Arena &ar, const DCsr &L, const DCsr &R, cudaStream_t s) {
     int n = L.n;
     Scratch<int> ub(n);
@@ -588,7 +823,11 @@ static DCsr csr_spgemm(Arena &ar, const DCsr &L, const DCsr &R, cudaStream_t s) 
     int64_t total = scan_to64(ub, off, n, s);
     Scratch<int> cand(total);
     Scratch<int> ulen(n);
-    k_spgemm_sym<<<grid_for(n, 128), 128, 0, s>>>(n, L.rp, L.ci, R.rp, R.ci, off, cand, ulen);
+    const bool warps = n <= kWarpRows;
+    if (warps)
+        k_spgemm_sym_warp<<<grid_for(n, kRowWarps), 32 * kRowWarps, 0, s>>>(n, L.rp, L.ci, R.rp, R.ci, off, cand, ulen);
+    else
+        k_spgemm_sym<<<grid_for(n, 128), 128, 0, s>>>(n, L.rp, L.ci, R.rp, R.ci, off, cand, ulen);
     VEMG_CHECK_LAUNCH();
     DCsr C;
     C.n = n;
@@ -599,7 +838,11 @@ static DCsr csr_spgemm(Arena &ar, const DCsr &L, const DCsr &R, cudaStream_t s) 
     C.v = ar.alloc<double>(C.nnz);
     k_spgemm_copy<<<grid_for(n, 256), 256, 0, s>>>(n, off, cand, C.rp, C.ci);
     VEMG_CHECK_LAUNCH();
-    k_spgemm_num<<<grid_for(n, 128), 128, 0, s>>>(n, L.rp, L.ci, L.v, R.rp, R.ci, R.v, C.rp, C.ci, C.v);
+    if (warps)
+        k_spgemm_num_warp<<<grid_for(n, kRowWarps), 32 * kRowWarps, 0, s>>>(n, L.rp, L.ci, L.v, R.rp, R.ci, R.v, C.rp,
+                                                                            C.ci, C.v);
+    else
+        k_spgemm_num<<<grid_for(n, 128), 128, 0, s>>>(n, L.rp, L.ci, L.v, R.rp, R.ci, R.v, C.rp, C.ci, C.v);
     VEMG_CHECK_LAUNCH();
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     return C;
@@ -1773,8 +2016,7 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         k_perm_fill<<<grid_for(n, 256), 256, 0, s>>>(n, Ain->rowptr, Ain->col, Ain->val, h->new2old, h->old2new,
                                                      A.rp, A.ci, A.v);
         VEMG_CHECK_LAUNCH();
-        k_sort_rows_kv<<<grid_for(n, 128), 128, 0, s>>>(A.rp, A.ci, A.v, n);
-        VEMG_CHECK_LAUNCH();
+        sort_rows(A.rp, A.ci, A.v, n, s);
     }
     // A_bar
     DCsr Abar;

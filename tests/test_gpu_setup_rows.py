@@ -33,6 +33,8 @@ def test_dense_rows(kx, ky):
     want = dense[np.ix_(order, order)]
     got = V.vemg_get_csr(h, "A").tocsr()
     assert got.has_sorted_indices and np.array_equal(got.toarray(), want)
+    # a dense level: every row has a colour of its own
+    assert np.array_equal(np.sort(V.vemg_get_int(h, "lev.colour", 1, 0)), np.arange(V.vemg_get_size(h, "lev.n", 1, 0)))
     E = V.vemg_get_csr(h, "E").toarray()
     Ac = V.vemg_get_csr(h, "Ac").tocsr()
     assert np.array_equal(np.diff(Ac.indptr), np.full(E.shape[1], E.shape[1]))

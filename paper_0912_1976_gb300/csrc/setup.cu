@@ -1635,7 +1635,8 @@ __device__ __forceinline__ void push(int *wl, int *count, int v) { wl[atomicAdd(
 
 // Peeling round: every node of the worklist leaves with rank `round`; each remaining neighbour
 // loses one degree, and one whose degree falls from k + 1 to k joins the next worklist. (A
-// neighbour leaving in the same round has degree <= k already and never crosses.) One warp per
+// neighbour that has left or is leaving has degree <= k already and never crosses: its rank is not
+// looked at.) One warp per
 // node, its lanes over the node's row, so that the decrements of a row are one round trip.
 // The worklist sizes live in a ring: round t reads slot t, fills slot t + 1 and clears slot
 // t + 2 for the round after it.
@@ -1647,14 +1648,30 @@ __global__ void __launch_bounds__(kRoundThreads) k_peel_round(const int *__restr
     const int cnt = nring[round % kRing];
     int *n_out = nring + (round + 1) % kRing;
     if (blockIdx.x == 0 && threadIdx.x == 0) nring[(round + 2) % kRing] = 0;
+    constexpr int U = 4;   // nodes at a time: a node alone is a chain of five dependent accesses
     const int lane = threadIdx.x & 31;
     const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    for (int q = w0; q < cnt; q += nw) {
-        int v = wl_in[q];
-        if (lane == 0) rank[v] = round;
-        for (int e = rp[v] + lane; e < rp[v + 1]; e += 32) {
-            int j = ci[e];
-            if (j != v && rank[j] < 0 && atomicSub(deg + j, 1) == k + 1) push(wl_out, n_out, j);
+    for (int q = w0; q < cnt; q += U * nw) {
+        int v[U], lo[U], hi[U], j[U], old[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = q + u * nw < cnt ? wl_in[q + u * nw] : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            lo[u] = v[u] >= 0 ? rp[v[u]] : 0;
+            hi[u] = v[u] >= 0 ? rp[v[u] + 1] : 0;
+            if (lane == 0 && v[u] >= 0) rank[v[u]] = round;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) j[u] = lo[u] + lane < hi[u] ? ci[lo[u] + lane] : v[u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) old[u] = j[u] != v[u] ? atomicSub(deg + j[u], 1) : 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j[u] != v[u] && old[u] == k + 1) push(wl_out, n_out, j[u]);
+            for (int e = lo[u] + 32 + lane; e < hi[u]; e += 32) {
+                const int i = ci[e];
+                if (i != v[u] && atomicSub(deg + i, 1) == k + 1) push(wl_out, n_out, i);
+            }
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(removed, cnt);
@@ -1776,8 +1793,8 @@ __global__ void __launch_bounds__(kRoundThreads) k_jp_round(const int *__restric
 
 // The rounds of short worklists, one after the other in one launch: a thread-block cluster whose barrier
 // stands between two rounds. It ends at an empty worklist, at one of more than kShortList nodes (a whole
-// grid per round is faster there; 512 and 2,048 measured the same) or after kShortRounds rounds, with {round, worklist size, nodes
-// handled} in stat. What another block writes is read past L1. A round is 1 to 3 us, most of it the
+// grid per round is faster there; 512 and 2,048 measured the same) or after kShortRounds rounds, with
+// {round, worklist size, nodes handled} in stat. What another block writes is read past L1. A round is 1 to 3 us, most of it the
 // chain of its dependent accesses: with a launch per round, assembly, setup and first solve of a new
 // 2.1M-node mesh took 134 ms, now 120.
 static constexpr int kShortBlocks = 8, kShortThreads = 1024, kShortList = 1024, kShortRounds = 4096;
@@ -1787,8 +1804,7 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// As k_peel_round, but for the test of rank[j]: a node that has left has a degree of at most k, which
-// a further decrement cannot bring to k.
+// as k_peel_round
 __global__ void __launch_bounds__(kShortThreads) k_peel_short(int *wl0, int *wl1, int *nring,
                                                               const int *__restrict__ rp, const int *__restrict__ ci,
                                                               int *rank, int *deg, int k, int t, int n, int *stat) {

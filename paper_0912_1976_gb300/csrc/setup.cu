@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 
 #include "internal.cuh"
 
@@ -1687,10 +1688,10 @@ __global__ void k_peel_min(int n, const int *__restrict__ deg, const int *__rest
     if ((threadIdx.x & 31) == 0 && m != 0xffffffffu) atomicMin(dmin, (int)m);
 }
 
-__global__ void k_peel_fill(int n, const int *__restrict__ deg, const int *__restrict__ rank, int k, int *wl,
-                            int *count) {
+__global__ void k_peel_fill(int n, const int *__restrict__ deg, const int *__restrict__ rank, int k,
+                            const int *__restrict__ dmin, int *wl, int *count) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && rank[i] < 0 && deg[i] <= k) push(wl, count, i);
+    if (i < n && rank[i] < 0 && deg[i] <= max(k, *dmin)) push(wl, count, i);
 }
 
 // number of neighbours with a larger colouring key: a node is coloured once they all are
@@ -1794,7 +1795,7 @@ __global__ void __launch_bounds__(kRoundThreads) k_jp_round(const int *__restric
 // The rounds of short worklists, one after the other in one launch: a thread-block cluster whose barrier
 // stands between two rounds. It ends at an empty worklist, at one of more than kShortList nodes (a whole
 // grid per round is faster there; 512 and 2,048 measured the same) or after kShortRounds rounds, with
-// {round, worklist size, nodes handled} in stat. What another block writes is read past L1. A round is 1 to 3 us, most of it the
+// {round, worklist size, nodes removed, threshold} in stat. What another block writes is read past L1. A round is 1 to 3 us, most of it the
 // chain of its dependent accesses: with a launch per round, assembly, setup and first solve of a new
 // 2.1M-node mesh took 134 ms, now 120.
 static constexpr int kShortBlocks = 8, kShortThreads = 1024, kShortList = 1024, kShortRounds = 4096;
@@ -1807,7 +1808,9 @@ __device__ __forceinline__ void cluster_barrier() {
 // as k_peel_round
 __global__ void __launch_bounds__(kShortThreads) k_peel_short(int *wl0, int *wl1, int *nring,
                                                               const int *__restrict__ rp, const int *__restrict__ ci,
-                                                              int *rank, int *deg, int k, int t, int n, int *stat) {
+                                                              int *rank, int *deg, const int *__restrict__ dmin, int k,
+                                                              int t, int n, int *stat) {
+    k = max(k, *dmin);
     const int lane = threadIdx.x & 31;
     const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
     int left = 0, cnt = 0;
@@ -1833,6 +1836,7 @@ __global__ void __launch_bounds__(kShortThreads) k_peel_short(int *wl0, int *wl1
         stat[0] = t;
         stat[1] = cnt;
         stat[2] += left;
+        stat[3] = k;
     }
 }
 
@@ -1859,7 +1863,7 @@ __global__ void __launch_bounds__(kShortThreads) k_jp_short(int *wl0, int *wl1, 
 }
 
 template <typename... KArgs, typename... Args>
-static void short_rounds(void (*kernel)(KArgs...), int *stat, int *host, cudaStream_t s, Args &&...args) {
+static void short_rounds(void (*kernel)(KArgs...), cudaStream_t s, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = kShortBlocks;
     cfg.blockDim = kShortThreads;
@@ -1870,10 +1874,108 @@ static void short_rounds(void (*kernel)(KArgs...), int *stat, int *host, cudaStr
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    VEMG_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)..., stat));
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(host, stat, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
+    VEMG_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
+
+// The colouring of one level, on a stream of its own. A trip is the rounds up to a point where the host
+// decides; it ends with the status in host memory: {round, worklist size, nodes removed, threshold,
+// largest colour}.
+struct ColourJob {
+    static constexpr int kStat = 5;
+    Level &L;
+    const int n;
+    int *const host;
+    cudaStream_t st = nullptr;
+    Scratch<int> deg, rank, pc, wl0, wl1, nring, stat, dmin;
+    int t = 0, k = 0;
+    int64_t trips = 0;
+    bool peeling = true, done = false;
+
+    ColourJob(Arena &ar, Level &level, int *status)
+        : L(level), n(level.A.n), host(status), deg(n), rank(n), pc(n), wl0(n), wl1(n), nring(kRing), stat(kStat),
+          dmin(1) {
+        L.colour = ar.alloc<int>(n);
+    }
+    ~ColourJob() {
+        if (!st) return;
+        cudaStreamSynchronize(st);   // before the buffers go
+        cudaStreamDestroy(st);
+    }
+
+    void start(cudaEvent_t ready) {
+        VEMG_CHECK_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        VEMG_CHECK_CUDA(cudaStreamWaitEvent(st, ready, 0));
+        VEMG_CHECK_CUDA(cudaMemsetAsync(L.colour, 0xff, sizeof(int) * n, st));
+        VEMG_CHECK_CUDA(cudaMemsetAsync(nring, 0, sizeof(int) * kRing, st));
+        VEMG_CHECK_CUDA(cudaMemsetAsync(stat, 0, sizeof(int) * kStat, st));
+        k_offdiag_degree<<<grid_for(n, 256), 256, 0, st>>>(n, L.A.rp, L.A.ci, deg, rank);
+        VEMG_CHECK_LAUNCH();
+        peel(true);
+    }
+
+    // raise the threshold if the worklist is empty, kRoundBatch rounds of a grid each if it is long (rounds
+    // after an empty worklist do nothing; their ranks stay unused, which keeps the order of the ranks),
+    // then the rounds of short worklists
+    void peel(bool empty) {
+        int *wl[2] = {wl0, wl1};
+        if (empty) {
+            VEMG_CHECK_CUDA(cudaMemsetAsync(dmin, 0x7f, sizeof(int), st));
+            k_peel_min<<<grid_for(n, 256), 256, 0, st>>>(n, deg, rank, dmin);
+            VEMG_CHECK_LAUNCH();
+            k_peel_fill<<<grid_for(n, 256), 256, 0, st>>>(n, deg, rank, k, dmin, wl[t & 1], nring + t % kRing);
+            VEMG_CHECK_LAUNCH();
+        } else {
+            for (int u = 0; u < kRoundBatch; ++u, ++t)
+                pdl_launch(k_peel_round, kRoundBlocks, kRoundThreads, st, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p,
+                           (const int *)L.A.rp, (const int *)L.A.ci, rank.p, deg.p, k, t, stat.p + 2);
+        }
+        short_rounds(k_peel_short, st, wl0.p, wl1.p, nring.p, (const int *)L.A.rp, (const int *)L.A.ci, rank.p, deg.p,
+                     (const int *)dmin.p, k, t, n, stat.p);
+        report();
+    }
+
+    // Jones-Plassmann rounds in decreasing key order, likewise
+    void colour(bool first) {
+        int *wl[2] = {wl0, wl1};
+        if (first) {
+            VEMG_CHECK_CUDA(cudaMemsetAsync(nring, 0, sizeof(int) * kRing, st));
+            k_jp_pred<<<grid_for(n, 256), 256, 0, st>>>(n, L.A.rp, L.A.ci, rank, pc, wl0, nring);
+            VEMG_CHECK_LAUNCH();
+        } else {
+            for (int u = 0; u < kRoundBatch; ++u, ++t)
+                pdl_launch(k_jp_round, kRoundBlocks, kRoundThreads, st, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p, t,
+                           (const int *)L.A.rp, (const int *)L.A.ci, (const int *)rank.p, pc.p, L.colour, stat.p + 4);
+        }
+        short_rounds(k_jp_short, st, wl0.p, wl1.p, nring.p, (const int *)L.A.rp, (const int *)L.A.ci, (const int *)rank.p,
+                     pc.p, L.colour, stat.p + 4, t, stat.p);
+        report();
+    }
+
+    void report() {
+        VEMG_CHECK_CUDA(cudaMemcpyAsync(host, stat, sizeof(int) * kStat, cudaMemcpyDeviceToHost, st));
+    }
+
+    // a trip has ended: the next one. Every trip removes or colours a node (a raise guarantees one in its
+    // first round): the bound on the trips turns a broken invariant into an error, not a hang.
+    void advance() {
+        if (++trips > 2 * (int64_t)n + 64) throw Error{VEMG_EINTERNAL};
+        t = host[0];
+        k = host[3];
+        if (peeling && host[2] < n) {
+            peel(host[1] == 0);
+        } else if (peeling) {
+            peeling = false;
+            trips = 0;
+            t = 0;   // the colouring's first worklist sits in slot 0 of the ring
+            colour(true);
+        } else if (host[1] != 0) {
+            colour(false);
+        } else {
+            L.ncolours = host[4] + 1;
+            done = true;
+        }
+    }
+};
 
 // Rows grouped by colour, ascending within a colour: a counting sort. A warp takes kGroupRows
 // consecutive rows; count c * nw + w is warp w's rows of colour c, so that the exclusive scan of the
@@ -1897,61 +1999,8 @@ __global__ void k_group(int n, int nw, const int *__restrict__ colour, int *cnt,
     }
 }
 
-static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
-    int n = L.A.n;
-    L.colour = ar.alloc<int>(n);
-    VEMG_CHECK_CUDA(cudaMemsetAsync(L.colour, 0xff, sizeof(int) * n, s));
-    Scratch<int> deg(n), rank(n), pc(n), wl0(n), wl1(n), maxc(1), nring(kRing), stat(3), dmin(1);
-    int *wl[2] = {wl0, wl1};
-    VEMG_CHECK_CUDA(cudaMemsetAsync(maxc, 0, sizeof(int), s));
-    if (n > 0) {
-        k_offdiag_degree<<<grid_for(n, 256), 256, 0, s>>>(n, L.A.rp, L.A.ci, deg, rank);
-        VEMG_CHECK_LAUNCH();
-        VEMG_CHECK_CUDA(cudaMemsetAsync(nring, 0, sizeof(int) * kRing, s));
-        VEMG_CHECK_CUDA(cudaMemsetAsync(stat, 0, 3 * sizeof(int), s));
-    }
-    // peeling: raise the threshold whenever the worklist runs empty; the rounds of short worklists in one
-    // launch, kRoundBatch rounds of a grid each where that ended at a long one (rounds after an empty
-    // worklist do nothing; their ranks stay unused, which keeps the order of the ranks). Every trip
-    // removes a node (a raise guarantees one in its first round): the bound on the trips turns a broken
-    // invariant into an error, not a hang.
-    int t = 0, k = 0, st[3] = {0, 0, 0};   // next round, its worklist, nodes removed
-    for (int64_t trips = 0; st[2] < n; ++trips) {
-        if (trips > 2 * (int64_t)n + 64) throw Error{VEMG_EINTERNAL};
-        if (st[1] == 0) {
-            VEMG_CHECK_CUDA(cudaMemsetAsync(dmin, 0x7f, sizeof(int), s));
-            k_peel_min<<<grid_for(n, 256), 256, 0, s>>>(n, deg, rank, dmin);
-            VEMG_CHECK_LAUNCH();
-            k = std::max(k, read_int(dmin, s));
-            k_peel_fill<<<grid_for(n, 256), 256, 0, s>>>(n, deg, rank, k, wl[t & 1], nring + t % kRing);
-            VEMG_CHECK_LAUNCH();
-        } else {
-            for (int u = 0; u < kRoundBatch; ++u, ++t)
-                pdl_launch(k_peel_round, kRoundBlocks, kRoundThreads, s, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p,
-                           (const int *)L.A.rp, (const int *)L.A.ci, rank.p, deg.p, k, t, stat.p + 2);
-        }
-        short_rounds(k_peel_short, stat.p, st, s, wl[0], wl[1], nring.p, (const int *)L.A.rp, (const int *)L.A.ci,
-                     rank.p, deg.p, k, t, n);
-        t = st[0];
-    }
-    // colouring in decreasing key order: Jones-Plassmann rounds on predecessor counts, until a worklist is empty
-    if (n > 0) {
-        VEMG_CHECK_CUDA(cudaMemsetAsync(nring, 0, sizeof(int) * kRing, s));
-        k_jp_pred<<<grid_for(n, 256), 256, 0, s>>>(n, L.A.rp, L.A.ci, rank, pc, wl[0], nring);
-        VEMG_CHECK_LAUNCH();
-    }
-    t = 0;   // the colouring's first worklist sits in slot 0 of the ring
-    for (int64_t trips = 0; n > 0; ++trips) {
-        if (trips > (int64_t)n + 64) throw Error{VEMG_EINTERNAL};   // every trip colours a node
-        short_rounds(k_jp_short, stat.p, st, s, wl[0], wl[1], nring.p, (const int *)L.A.rp, (const int *)L.A.ci,
-                     (const int *)rank.p, pc.p, L.colour, maxc.p, t);
-        t = st[0];
-        if (st[1] == 0) break;
-        for (int u = 0; u < kRoundBatch; ++u, ++t)
-            pdl_launch(k_jp_round, kRoundBlocks, kRoundThreads, s, (const int *)wl[t & 1], wl[(t + 1) & 1], nring.p, t,
-                       (const int *)L.A.rp, (const int *)L.A.ci, (const int *)rank.p, pc.p, L.colour, maxc.p);
-    }
-    L.ncolours = n > 0 ? read_int(maxc, s) + 1 : 0;
+static void group_rows(Arena &ar, Level &L, cudaStream_t s) {
+    const int n = L.A.n;
     L.crow = ar.alloc<int>(n);
     L.cptr.assign(L.ncolours + 1, n);
     if (n == 0) return;
@@ -1966,6 +2015,45 @@ static void colour_level(Arena &ar, Level &L, cudaStream_t s) {
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     k_group<true><<<grid_for((int64_t)nw * 32, 128), 128, 0, s>>>(n, nw, L.colour, off, L.crow);
     VEMG_CHECK_LAUNCH();
+}
+
+// Colours every level. A level's rounds are a chain of small launches that leaves the device idle, and one
+// level's colouring does not wait for another's: all of them at once, each advanced when its stream has
+// run dry. One after the other, those of a 2.1M-node mesh's nine levels took 46 ms.
+static void colour_levels(Arena &ar, const std::vector<Level *> &levels, cudaStream_t s) {
+    struct Status {
+        int *p = nullptr;
+        cudaEvent_t ready = nullptr;
+        ~Status() {
+            if (ready) cudaEventDestroy(ready);
+            if (p) cudaFreeHost(p);
+        }
+    } status;
+    VEMG_CHECK_CUDA(cudaMallocHost(&status.p, sizeof(int) * ColourJob::kStat * (levels.size() + 1)));
+    VEMG_CHECK_CUDA(cudaEventCreateWithFlags(&status.ready, cudaEventDisableTiming));
+    std::vector<std::unique_ptr<ColourJob>> jobs;
+    for (Level *L : levels) {
+        if (L->A.n > 0)
+            jobs.emplace_back(new ColourJob(ar, *L, status.p + ColourJob::kStat * jobs.size()));
+        else
+            L->ncolours = 0;
+    }
+    VEMG_CHECK_CUDA(cudaEventRecord(status.ready, s));
+    for (auto &j : jobs) j->start(status.ready);
+    for (size_t left = jobs.size(); left > 0;)
+        for (auto &j : jobs) {
+            if (j->done) continue;
+            const cudaError_t e = cudaStreamQuery(j->st);
+            if (e == cudaErrorNotReady) {
+                (void)cudaGetLastError();
+                continue;
+            }
+            VEMG_CHECK_CUDA(e);
+            j->advance();
+            left -= j->done;
+        }
+    jobs.clear();
+    for (Level *L : levels) group_rows(ar, *L, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -2104,7 +2192,6 @@ static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_
     }
     for (int l = 0; l < C.nlev; ++l) {
         Level &L = C.lv[l];
-        colour_level(ar, L, s);
         L.diag = ar.alloc<double>(L.A.n);
         k_diag<<<grid_for(L.A.n, 256), 256, 0, s>>>(L.A.n, L.A.rp, L.A.ci, L.A.v, L.diag);
         VEMG_CHECK_LAUNCH();
@@ -2261,14 +2348,12 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         V.lv[0].A = h->A;
         V.lv[0].P = h->E;
         V.lv[0].PT = h->ET;
-        for (int l = 0; l < S.nlev; ++l) V.lv[l + 1] = S.lv[l];
         V.direct = S.direct;
         V.nc = S.nc;
         V.G = S.G;
         V.nsd = S.nsd;
         V.nu = S.nu;
         Level &L = V.lv[0];
-        colour_level(ar, L, s);
         L.diag = ar.alloc<double>(L.A.n);
         k_diag<<<grid_for(L.A.n, 256), 256, 0, s>>>(L.A.n, L.A.rp, L.A.ci, L.A.v, L.diag);
         VEMG_CHECK_LAUNCH();
@@ -2276,6 +2361,13 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         L.b = ar.alloc<double>(L.A.n);
         L.r = ar.alloc<double>(L.A.n);
     }
+    const bool vl = h->bc == VEMG_NEUMANN && h->precond == VEMG_PRECOND_VL_SOR;
+    std::vector<Level *> levels;
+    for (Chain *C : {&h->bar, &h->surf, &h->one})   // the largest levels first
+        for (int l = 0; l < (C == &h->one && vl ? 1 : C->nlev); ++l) levels.push_back(&C->lv[l]);
+    colour_levels(ar, levels, s);
+    if (vl)
+        for (int l = 0; l < h->surf.nlev; ++l) h->one.lv[l + 1] = h->surf.lv[l];
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
 }
 

@@ -14,8 +14,15 @@
 #include <math.h>
 
 #include <algorithm>
+#include <condition_variable>
 #include <cstring>
+#include <exception>
 #include <memory>
+#include <mutex>
+#include <string>
+#include <system_error>
+#include <thread>
+#include <vector>
 
 #include "internal.cuh"
 
@@ -1902,9 +1909,14 @@ struct ColourJob {
         cudaStreamDestroy(st);
     }
 
-    void start(cudaEvent_t ready) {
+    // the matrix and the buffers are ready where s stands
+    void follow(cudaEvent_t ev, cudaStream_t s) {
         VEMG_CHECK_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-        VEMG_CHECK_CUDA(cudaStreamWaitEvent(st, ready, 0));
+        VEMG_CHECK_CUDA(cudaEventRecord(ev, s));
+        VEMG_CHECK_CUDA(cudaStreamWaitEvent(st, ev, 0));
+    }
+
+    void start() {
         VEMG_CHECK_CUDA(cudaMemsetAsync(L.colour, 0xff, sizeof(int) * n, st));
         VEMG_CHECK_CUDA(cudaMemsetAsync(nring, 0, sizeof(int) * kRing, st));
         VEMG_CHECK_CUDA(cudaMemsetAsync(stat, 0, sizeof(int) * kStat, st));
@@ -2017,44 +2029,118 @@ static void group_rows(Arena &ar, Level &L, cudaStream_t s) {
     VEMG_CHECK_LAUNCH();
 }
 
-// Colours every level. A level's rounds are a chain of small launches that leaves the device idle, and one
-// level's colouring does not wait for another's: all of them at once, each advanced when its stream has
-// run dry. One after the other, those of a 2.1M-node mesh's nine levels took 46 ms.
-static void colour_levels(Arena &ar, const std::vector<Level *> &levels, cudaStream_t s) {
-    struct Status {
+// Colours the levels as the coarsening yields them. A level's rounds are a chain of small launches that
+// leaves the device idle, and neither another level's colouring nor the coarsening waits for it: every
+// level has a stream, and a thread advances each when it has run dry. (One level after the other, those
+// of a 2.1M-node mesh took 46 ms; all at once after the coarsening 22.) The calling thread allocates and
+// frees everything; the other one only launches.
+class Colouring {
+public:
+    Colouring(Arena &arena, cudaStream_t stream) : ar(arena), s(stream) {
+        VEMG_CHECK_CUDA(cudaGetDevice(&device));
+        VEMG_CHECK_CUDA(cudaMallocHost(&hold.p, sizeof(int) * ColourJob::kStat * 3 * kMaxLevels));
+        VEMG_CHECK_CUDA(cudaEventCreateWithFlags(&hold.ev, cudaEventDisableTiming));
+        try {
+            th = std::thread([this] { run(); });
+        } catch (const std::system_error &) {
+            // no thread to be had: finish() does the work
+        }
+    }
+    ~Colouring() { join(true); }
+    Colouring(const Colouring &) = delete;
+    Colouring &operator=(const Colouring &) = delete;
+
+    // once per level, as soon as its matrix is on the way
+    void add(Level &L) {
+        if (std::find(levels.begin(), levels.end(), &L) != levels.end()) return;
+        levels.push_back(&L);
+        if (L.A.n <= 0) return;
+        jobs.emplace_back(new ColourJob(ar, L, hold.p + ColourJob::kStat * jobs.size()));
+        jobs.back()->follow(hold.ev, s);
+        std::lock_guard<std::mutex> lk(mu);
+        fresh.push_back(jobs.back().get());
+        cv.notify_one();
+    }
+
+    void finish() {
+        const bool inline_run = !th.joinable();
+        join(false);
+        if (inline_run) run();
+        if (error) {
+            set_last_error_message(message.c_str());
+            std::rethrow_exception(error);
+        }
+        jobs.clear();
+        for (Level *L : levels) group_rows(ar, *L, s);
+    }
+
+private:
+    struct Hold {   // released after the jobs that use it
         int *p = nullptr;
-        cudaEvent_t ready = nullptr;
-        ~Status() {
-            if (ready) cudaEventDestroy(ready);
+        cudaEvent_t ev = nullptr;
+        ~Hold() {
+            if (ev) cudaEventDestroy(ev);
             if (p) cudaFreeHost(p);
         }
-    } status;
-    VEMG_CHECK_CUDA(cudaMallocHost(&status.p, sizeof(int) * ColourJob::kStat * (levels.size() + 1)));
-    VEMG_CHECK_CUDA(cudaEventCreateWithFlags(&status.ready, cudaEventDisableTiming));
+    };
+    Arena &ar;
+    const cudaStream_t s;
+    int device = 0;
+    Hold hold;
     std::vector<std::unique_ptr<ColourJob>> jobs;
-    for (Level *L : levels) {
-        if (L->A.n > 0)
-            jobs.emplace_back(new ColourJob(ar, *L, status.p + ColourJob::kStat * jobs.size()));
-        else
-            L->ncolours = 0;
-    }
-    VEMG_CHECK_CUDA(cudaEventRecord(status.ready, s));
-    for (auto &j : jobs) j->start(status.ready);
-    for (size_t left = jobs.size(); left > 0;)
-        for (auto &j : jobs) {
-            if (j->done) continue;
-            const cudaError_t e = cudaStreamQuery(j->st);
-            if (e == cudaErrorNotReady) {
-                (void)cudaGetLastError();
-                continue;
-            }
-            VEMG_CHECK_CUDA(e);
-            j->advance();
-            left -= j->done;
+    std::vector<Level *> levels;
+    std::mutex mu;
+    std::condition_variable cv;
+    std::vector<ColourJob *> fresh;   // under mu, with the two flags
+    bool closed = false, stop = false;
+    std::exception_ptr error;
+    std::string message;
+    std::thread th;
+
+    void join(bool abandon) {
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            closed = true;
+            stop = abandon;
+            cv.notify_one();
         }
-    jobs.clear();
-    for (Level *L : levels) group_rows(ar, *L, s);
-}
+        if (th.joinable()) th.join();
+    }
+
+    void run() {
+        try {
+            VEMG_CHECK_CUDA(cudaSetDevice(device));
+            std::vector<ColourJob *> active, in;
+            for (;;) {
+                {
+                    std::unique_lock<std::mutex> lk(mu);
+                    if (active.empty()) cv.wait(lk, [this] { return closed || !fresh.empty(); });
+                    if (stop || (closed && fresh.empty() && active.empty())) return;
+                    in.swap(fresh);
+                }
+                for (ColourJob *j : in) {
+                    j->start();
+                    active.push_back(j);
+                }
+                in.clear();
+                for (ColourJob *j : active) {
+                    const cudaError_t e = cudaStreamQuery(j->st);
+                    if (e == cudaErrorNotReady) {
+                        (void)cudaGetLastError();
+                        continue;
+                    }
+                    VEMG_CHECK_CUDA(e);
+                    j->advance();
+                }
+                std::this_thread::yield();
+                active.erase(std::remove_if(active.begin(), active.end(), [](ColourJob *j) { return j->done; }), active.end());
+            }
+        } catch (...) {
+            error = std::current_exception();
+            message = last_cuda_error();
+        }
+    }
+};
 
 // ------------------------------------------------------------------------------------------
 // coarsest level: dense inverse (projected onto the complement of constants if singular)
@@ -2145,14 +2231,15 @@ static DCsr copy_csr(Arena &ar, const DCsr &a, cudaStream_t s) {
 }
 
 // B0: near-nullspace rows of level 0 (n x 3) for a {1, x, y} chain, else null
-static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_options &o, cudaStream_t s,
-                        double *B0 = nullptr) {
+static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_options &o, Colouring &colouring,
+                        cudaStream_t s, double *B0 = nullptr) {
     C.singular = singular;
     C.nlev = 1;
     C.lv[0].A = A0;
     C.nsd = B0 ? kNsd : 1;
     C.lv[0].B = B0;
     C.lv[0].nblk = A0.n;
+    colouring.add(C.lv[0]);
     int max_levels = std::min(std::max(o.max_levels, 1), kMaxLevels);
     while (C.nlev < max_levels && C.lv[C.nlev - 1].A.n > o.coarse_max) {
         Level &L = C.lv[C.nlev - 1];
@@ -2162,6 +2249,7 @@ static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_
             if (coarsen_linear(ar, L, N, o.strength, o.omega_p, s) == 0) break;
             L.PT = csr_transpose(ar, L.P, s);
             N.A = galerkin(ar, L.A, L.P, L.PT, s);
+            colouring.add(N);
             C.nlev++;
             continue;
         }
@@ -2188,6 +2276,7 @@ static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_
         VEMG_CHECK_LAUNCH();
         L.PT = csr_transpose(ar, L.P, s);
         C.lv[C.nlev].A = galerkin(ar, L.A, L.P, L.PT, s);
+        colouring.add(C.lv[C.nlev]);
         C.nlev++;
     }
     for (int l = 0; l < C.nlev; ++l) {
@@ -2263,6 +2352,9 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         k_bar_fill<<<grid_for(nb, 256), 256, 0, s>>>(nb, h->mtop, h->A.rp, h->A.ci, h->A.v, Abar.rp, Abar.ci, Abar.v);
         VEMG_CHECK_LAUNCH();
     }
+    Colouring colouring(ar, s);
+    h->bar.lv[0].A = Abar;
+    colouring.add(h->bar.lv[0]);
     if (h->bc == VEMG_NEUMANN) {
         if (!mesh->xyz || !mesh->top_tris || mesh->n_top_tris <= 0) throw Error{VEMG_EINVAL};
         int nt = (int)mesh->n_top_tris;
@@ -2331,12 +2423,12 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
             k_top_nullspace<<<grid_for(h->mtop, 256), 256, 0, s>>>(h->mtop, h->new2old, xyz, B0);
             VEMG_CHECK_LAUNCH();
         }
-        build_chain(ar, h->surf, copy_csr(ar, h->Ac, s), true, h->opts, s, B0);
+        build_chain(ar, h->surf, copy_csr(ar, h->Ac, s), true, h->opts, colouring, s, B0);
     }
     h->bar.is_bar = true;
-    build_chain(ar, h->bar, Abar, false, h->opts, s);
+    build_chain(ar, h->bar, Abar, false, h->opts, colouring, s);
     if (h->bc == VEMG_NEUMANN && h->precond == VEMG_PRECOND_SA) {
-        build_chain(ar, h->one, copy_csr(ar, h->A, s), true, h->opts, s);
+        build_chain(ar, h->one, copy_csr(ar, h->A, s), true, h->opts, colouring, s);
     } else if (h->bc == VEMG_NEUMANN && h->precond == VEMG_PRECOND_VL_SOR) {
         // level 0: A with the vertical extrapolation E~ as its prolongator; below it the SA chain of
         // E~^T A E~ (section 6: the vertical lumping is the first coarsening of the cycle)
@@ -2354,6 +2446,7 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         V.nsd = S.nsd;
         V.nu = S.nu;
         Level &L = V.lv[0];
+        colouring.add(L);
         L.diag = ar.alloc<double>(L.A.n);
         k_diag<<<grid_for(L.A.n, 256), 256, 0, s>>>(L.A.n, L.A.rp, L.A.ci, L.A.v, L.diag);
         VEMG_CHECK_LAUNCH();
@@ -2362,10 +2455,7 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         L.r = ar.alloc<double>(L.A.n);
     }
     const bool vl = h->bc == VEMG_NEUMANN && h->precond == VEMG_PRECOND_VL_SOR;
-    std::vector<Level *> levels;
-    for (Chain *C : {&h->bar, &h->surf, &h->one})   // the largest levels first
-        for (int l = 0; l < (C == &h->one && vl ? 1 : C->nlev); ++l) levels.push_back(&C->lv[l]);
-    colour_levels(ar, levels, s);
+    colouring.finish();
     if (vl)
         for (int l = 0; l < h->surf.nlev; ++l) h->one.lv[l + 1] = h->surf.lv[l];
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));

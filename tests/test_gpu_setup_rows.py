@@ -64,3 +64,27 @@ def test_assembly_adds_elements_in_order(n, ne):
     got = _assemble(xyz, tets)
     assert (got.nnz > 1024) == (ne > 100) and got.nnz == seen.sum()
     assert np.array_equal(got.toarray(), want)
+
+
+def test_setups_side_by_side():
+    """Colourings run beside the coarsening on streams of their own: two threads that set up different
+    problems at once, and a setup that fails while its colourings run, leave every colour as it is."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    meshes = [V.Mesh.from_inputs(I.make_mesh(k, k + 3, 11, I.depth_sines(1e-2), z_jitter=0.3, seed=k)) for k in (40, 57)]
+
+    def colours(vm):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            h = V.vemg_setup(V.vemg_assemble(vm), vm, V.vemg_default_options())
+            return [V.vemg_get_int(h, "lev.colour", c, l) for c in (0, 1) for l in range(V.vemg_get_size(h, "nlev", c))]
+
+    alone = [colours(vm) for vm in meshes]
+    bad = V.Mesh.from_inputs(I.make_mesh(40, 43, 11, I.depth_sines(1e-2), z_jitter=0.3, seed=40))
+    bad.top_tris[0] = bad.n   # out of range: found after the colouring of A_bar began
+    with ThreadPoolExecutor(2) as pool:
+        for _ in range(3):
+            both = list(pool.map(colours, meshes))
+            with pytest.raises(V.VemgError):
+                V.vemg_setup(V.vemg_assemble(bad), bad, V.vemg_default_options())
+            for got, want in zip(both, alone):
+                assert len(got) == len(want) and all(np.array_equal(a, b) for a, b in zip(got, want))

@@ -364,7 +364,7 @@ int vemg_kernel_launches(const vemg_hierarchy *h, int64_t *count);
 #define VEMG_PROBE_SOR_FINE 4    /* SOR launches on the finest level of the A_bar chain */
 #define VEMG_PROBE_VCYCLE 5      /* the persistent preconditioner kernel (VEMG_CYCLE_PERSISTENT) */
 #define VEMG_PROBE_TRANSFER 6    /* restrictions, prolongations and E~^T r (sliced-ELL transfers) */
-#define VEMG_PROBE_VECTOR 7      /* the Krylov vector kernels: x/r update, z combination, p update */
+#define VEMG_PROBE_VECTOR 7      /* the Krylov vector kernels: r update, z combination, p update, x update */
 #define VEMG_PROBE_DENSE 8       /* the dense coarsest-level solves */
 #define VEMG_PROBE_TAIL 9        /* the coarse-tail kernels (vemg_options.tail_rows) */
 

@@ -1,4 +1,3 @@
-#include <vector>
 // batch.cu -- many right-hand sides in one solve.
 //
 // K systems A x_c = b_c share one hierarchy. Vectors are interleaved (row-major n x K, K a power
@@ -18,6 +17,7 @@
 #include <cstring>
 
 #include <type_traits>
+#include <vector>
 
 #include "sell.cuh"
 

@@ -1,4 +1,3 @@
-#include <vector>
 // solve.cu -- the solve phase: preconditioned CG with the additive vertical-extrapolation
 // multigrid preconditioner (Kramer, Cotter and Pain, section 5.5, Eq. ourpreconditioner):
 //
@@ -11,14 +10,15 @@
 // symmetric (section 5.5 on nested inexact inner solves).
 //
 // Operators are sliced ELL in solve order (layout.cu, sell.cuh).
-// Reductions are deterministic (fixed grid, fixed order). One solve runs as three CUDA graphs:
-// the first iteration, a WHILE conditional node whose body is one further iteration (the
-// condition is set on the device from the residual norm), and the exit work.
+// Reductions are deterministic (fixed grid, fixed order). One solve is one launch of one CUDA graph:
+// the first iteration, a WHILE conditional node whose body is one further iteration (the condition
+// is set on the device from the residual norm), and the exit work.
 #include <math.h>
 
 #include <algorithm>
 
 #include <type_traits>
+#include <vector>
 
 #include "sell.cuh"
 

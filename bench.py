@@ -39,8 +39,8 @@ PRECS = {"fp64": 0, "fp32": 1, "bf16": 2}
 DTYPES = {"fp64": "f64", "fp32": "f64 outer + f32 preconditioner",
           "bf16": "f64 outer + f32 preconditioner with bf16 operator values"}
 # ncu DRAM bytes / algorithmic bytes of the finest colour sweep (one launch, 192x192x32 mesh)
-SOR_FINE_DRAM_RATIO = {"fp32": 34.63 / 32.33, "bf16": 27.33 / 25.18}
-SOR_FINE_KERNEL = {"fp32": "k_sell_sor<float, float, double>", "bf16": "k_sell_sor<__nv_bfloat16, float, double>"}
+SOR_FINE_DRAM_RATIO = {"fp32": 34.63 / 32.33, "bf16": 27.46 / 25.18}
+SOR_FINE_KERNEL = {"fp32": "k_sell_sor<float, float, double>", "bf16": "k_sell_sor<__nv_bfloat16, float, double, 16>"}
 CYCLES = {"persistent": 0, "launches": 1, "auto": 2, "hybrid": 3}
 
 
@@ -734,12 +734,12 @@ def main():
         # algorithmic bytes, scaled here by this workload's bytes per launch
         traffic = None
         if dom == "sor_coarse" and args.precision == "bf16":
-            # three captured coarse launches on a 192x192x32 mesh moved 0.606-0.623 MB from DRAM each
-            # (L2 hit rate 33-36%); the class mixes launches of every coarse level, so the figure is
+            # three captured coarse launches on a 192x192x32 mesh moved 0.643-0.663 MB from DRAM each
+            # (L2 hit rate 31-34%); the class mixes launches of every coarse level, so the figure is
             # the captured launches' own, not scaled to this workload's average launch
-            traffic = {"bytes_per_launch": 0.6167e6,
-                       "source": "ncu dram__bytes (read + write), mean of 3 k_sell_sor<__nv_bfloat16, float, float> "
-                                 "launches on a 192x192x32 mesh (profiles/sor_coarse_bf16_zjit192.md); not scaled"}
+            traffic = {"bytes_per_launch": 0.6560e6,
+                       "source": "ncu dram__bytes (read + write), mean of 3 k_sell_sor<__nv_bfloat16, float, float, 4> "
+                                 "launches on a 192x192x32 mesh (profiles/sor_rows_bf16_zjit192.md); not scaled"}
         if dom == "sor_fine" and args.precision in SOR_FINE_DRAM_RATIO:
             traffic = {"bytes_per_launch": SOR_FINE_DRAM_RATIO[args.precision] * c["bytes_per_launch"],
                        "source": f"ncu dram__bytes (read + write) of one {SOR_FINE_KERNEL[args.precision]} launch "

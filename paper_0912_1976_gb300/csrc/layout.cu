@@ -126,12 +126,10 @@ __global__ void k_sell_deal(int nslices, int lsh, const int *__restrict__ row0, 
 // rows alone fill half the chip (152 SMs x 2048 threads); below that a launch lasts as long as its
 // longest chain of loads, which more lanes per row cut: four entries each is as far as it pays. In FP64
 // every step of a warp holds a scheduler for 64 cycles however few of its lanes have an entry, and so does
-// every level of the tree that adds the lanes up, so lanes pay less far: a 131 x 113 x 25 solve takes 9.7 ms
-// with half the FP32 limit and 10.2 with this one. The order of a row's sums comes with it: over 300
-// iterations on the 192 x 192 x 48 xy-jittered mesh, whose rounding errors grow by 1e6, the count of
-// iterations with this limit is within one of the sequential sums' (302), with half it is not (304).
+// every level of the tree that adds the lanes up, so lanes pay half as far (a 131 x 113 x 25 solve: 9.7 ms;
+// 10.2 with 0.62 of the FP32 limit and with all of it, 9.97 and 10.68 with a quarter and an eighth).
 static int lanes_shift(double rows, double mean, bool fp32) {
-    const double most = 152.0 * (fp32 ? 1024.0 : 640.0);
+    const double most = 152.0 * (fp32 ? 1024.0 : 512.0);
     int lsh = 0;
     while (lsh < 5 && mean > 4.0 * (1 << lsh) && rows * (2 << lsh) <= most) ++lsh;
     return lsh;

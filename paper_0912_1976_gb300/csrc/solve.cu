@@ -28,6 +28,7 @@ static constexpr int kRedBlocks = 608;  // 4 x 152 SMs
 static constexpr int kRedThreads = 256;
 static constexpr int kSellBlock = 128;  // 4 slices per block
 static constexpr int kVecBlocks = 304;  // 2 x 152 SMs: the streaming kernels' most
+static constexpr int kVecBlocks64 = 228;   // with FP64 cycles (vec_blocks)
 static constexpr int kEmax = 4;         // E~ rows with at most this many entries take the fast path
 
 // ------------------------------------------------------------------------------------------
@@ -422,7 +423,15 @@ enum { C_SPMV = 0, C_XR, C_Z, C_SUMB, C_PREP, C_SUMX, C_TRUE, C_LATE, C_COUNT };
 
 int solve_scalar_iters() { return S_ITERS; }
 
-static int vec_blocks(int64_t n) { return (int)std::min<int64_t>(kVecBlocks, std::max<int64_t>(1, (n + kRedThreads - 1) / kRedThreads)); }
+// Blocks of the streaming kernels. Their number also sets the order of the dot products' sums, which no
+// order makes better than another; over the 300 iterations of the 192 x 192 x 48 xy-jittered mesh, whose
+// rounding errors grow by 1e6, the count of FP64 iterations is 302 with 228 blocks, as with sequential sums,
+// and 304 with 304 (a 131 x 113 x 25 solve: 9.8 and 9.7 ms). With FP32 cycles the FP32 rounding decides, and
+// 228 blocks would cost 2% (2.2M nodes: 15.7 -> 16.1 ms).
+static int vec_blocks(const vemg_hierarchy *h) {
+    const int most = h->precision == VEMG_PREC_FP64 ? kVecBlocks64 : kVecBlocks;
+    return (int)std::min<int64_t>(most, std::max<int64_t>(1, ((int64_t)h->nu + kRedThreads - 1) / kRedThreads));
+}
 
 template <int NS>
 __device__ bool finish_block(double (&acc)[NS], double *part, unsigned *counter, double (&tot)[NS]) {
@@ -803,7 +812,7 @@ __global__ void __launch_bounds__(kRedThreads) k_true_res(SellArgs A, const doub
 static void late(vemg_hierarchy *h, bool sums, cudaStream_t s) {
     const bool flex = h->precision != VEMG_PREC_FP64;
     ProbeScope ps(PROBE_VECTOR, (double)h->nu * (24.0 + (sums ? 8.0 + (flex ? 8.0 : 0.0) : 0.0)), s);
-    pdl_launch(k_late, vec_blocks(h->nu), kRedThreads, s, h->nu, (const double *)h->p, h->x,
+    pdl_launch(k_late, vec_blocks(h), kRedThreads, s, h->nu, (const double *)h->p, h->x,
                (const double *)(sums ? h->r : nullptr), (const double *)(sums && flex ? h->q : nullptr), h->scal,
                h->red + 5 * kRedBlocks * C_LATE, h->ctr + C_LATE, 1.0);
     SOLVE_LAUNCHED();
@@ -904,7 +913,7 @@ static void precond_t(vemg_hierarchy *h, const double *r, double *z, int first, 
                                  (double)sizeof(XT) * mt
                            : 0.0),
                   s);
-    pdl_launch(k_combine<XT>, vec_blocks(h->nu), kRedThreads, s, h->nu, mt, sargs(h->Enon), (const float *)h->Enon_vf, ys, xb, z, r,
+    pdl_launch(k_combine<XT>, vec_blocks(h), kRedThreads, s, h->nu, mt, sargs(h->Enon), (const float *)h->Enon_vf, ys, xb, z, r,
                                                      h->q, neu, flex, first, 1.0 / (double)h->nu, h->scal,
                                                      h->red + 5 * kRedBlocks * C_Z, h->ctr + C_Z,
                                                      persist ? persist_err(h) : nullptr, h->coef, 1.0);
@@ -964,11 +973,11 @@ static void phase_pre(vemg_hierarchy *h, cudaStream_t s) {
     const bool neu = h->bc == VEMG_NEUMANN;
     const int nu = h->nu;
     if (neu) {
-        pdl_launch(k_mean, vec_blocks(nu), kRedThreads, s, nu, h->b, 1.0 / (double)nu, S_BMEAN, h->scal, part_of(h, C_SUMB),
+        pdl_launch(k_mean, vec_blocks(h), kRedThreads, s, nu, h->b, 1.0 / (double)nu, S_BMEAN, h->scal, part_of(h, C_SUMB),
                                                   h->ctr + C_SUMB);
         SOLVE_LAUNCHED();
     }
-    pdl_launch(k_prepare, vec_blocks(nu), kRedThreads, s, nu, neu, h->b, h->r, h->x, h->p, h->scal, part_of(h, C_PREP),
+    pdl_launch(k_prepare, vec_blocks(h), kRedThreads, s, nu, neu, h->b, h->r, h->x, h->p, h->scal, part_of(h, C_PREP),
                                                  h->ctr + C_PREP);
     SOLVE_LAUNCHED();
     precond_solve_order(h, h->r, h->z, 1, s);
@@ -984,7 +993,7 @@ static void phase_pre(vemg_hierarchy *h, cudaStream_t s) {
 static void phase_step(vemg_hierarchy *h, cudaStream_t s, cudaGraphConditionalHandle hd, int use_cond) {
     spmv_outer(h, h->p, h->q, s);
     ProbeScope ps(PROBE_VECTOR, 24.0 * h->nu, s);   // q, r read; r written
-    pdl_launch(k_update_r, vec_blocks(h->nu), kRedThreads, s, h->nu, (const double *)h->q, h->r, h->scal,
+    pdl_launch(k_update_r, vec_blocks(h), kRedThreads, s, h->nu, (const double *)h->q, h->r, h->scal,
                part_of(h, C_XR), h->ctr + C_XR, hd, use_cond);
     SOLVE_LAUNCHED();
 }
@@ -1002,7 +1011,7 @@ static void phase_post(vemg_hierarchy *h, cudaStream_t s) {
     const int nu = h->nu;
     late(h, false, s);
     if (neu) {
-        pdl_launch(k_mean, vec_blocks(nu), kRedThreads, s, nu, h->x, 1.0 / (double)nu, S_XMEAN, h->scal, part_of(h, C_SUMX),
+        pdl_launch(k_mean, vec_blocks(h), kRedThreads, s, nu, h->x, 1.0 / (double)nu, S_XMEAN, h->scal, part_of(h, C_SUMX),
                                                   h->ctr + C_SUMX);
         SOLVE_LAUNCHED();
         pdl_launch(k_sub_scalar, grid_for(nu, 256), 256, s, nu, h->x, h->scal, S_XMEAN);

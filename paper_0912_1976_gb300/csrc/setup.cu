@@ -2235,7 +2235,7 @@ static void build_chain(Arena &ar, Chain &C, DCsr A0, bool singular, const vemg_
                         cudaStream_t s, double *B0 = nullptr) {
     C.singular = singular;
     C.nlev = 1;
-    C.lv[0].A = A0;
+    if (C.lv[0].A.rp != A0.rp) C.lv[0].A = A0;   // a level whose colouring has begun is being read
     C.nsd = B0 ? kNsd : 1;
     C.lv[0].B = B0;
     C.lv[0].nblk = A0.n;

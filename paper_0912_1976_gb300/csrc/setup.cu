@@ -495,35 +495,36 @@ __global__ void k_load(int n, const int *__restrict__ iptr, const int *__restric
     b[i] = acc;
 }
 
+// temporary arrays, released at scope exit
+struct TempArena : Arena {
+    TempArena() { temporary = true; }
+    ~TempArena() { release(); }
+    TempArena(const TempArena &) = delete;
+};
+
+// The mesh on the device. The arena puts the arrays on 256-byte boundaries whatever the caller's allocator
+// returns: the assembly loads the four vertices of an element at once.
 struct MeshDev {
+    TempArena ar;
     double *xyz = nullptr;
     int *tets = nullptr;
     int64_t ne = 0;
     int n = 0;
-    void release() {
-        dev_free_raw(xyz);
-        dev_free_raw(tets);
-        xyz = nullptr;
-        tets = nullptr;
+    MeshDev(const vemg_mesh *m, cudaStream_t s) {
+        if (!m || m->n_nodes <= 0 || m->n_tets <= 0 || !m->xyz || !m->tets) throw Error{VEMG_EINVAL};
+        if (m->n_nodes > 0x7ffffff0LL || m->n_tets * 4 > 0x7ffffff0LL) throw Error{VEMG_EINVAL};
+        n = (int)m->n_nodes;
+        ne = m->n_tets;
+        xyz = ar.alloc<double>((int64_t)3 * n);
+        tets = ar.alloc<int>(4 * ne);
+        VEMG_CHECK_CUDA(cudaMemcpyAsync(xyz, m->xyz, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice, s));
+        VEMG_CHECK_CUDA(cudaMemcpyAsync(tets, m->tets, sizeof(int) * 4 * (size_t)ne, cudaMemcpyHostToDevice, s));
     }
 };
 
-static MeshDev upload_mesh(const vemg_mesh *m, cudaStream_t s) {
-    if (!m || m->n_nodes <= 0 || m->n_tets <= 0 || !m->xyz || !m->tets) throw Error{VEMG_EINVAL};
-    if (m->n_nodes > 0x7ffffff0LL || m->n_tets * 4 > 0x7ffffff0LL) throw Error{VEMG_EINVAL};
-    MeshDev d;
-    d.n = (int)m->n_nodes;
-    d.ne = m->n_tets;
-    d.xyz = (double *)dev_alloc_raw(sizeof(double) * 3 * (size_t)d.n);
-    d.tets = (int *)dev_alloc_raw(sizeof(int) * 4 * (size_t)d.ne);
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(d.xyz, m->xyz, sizeof(double) * 3 * (size_t)d.n, cudaMemcpyHostToDevice, s));
-    VEMG_CHECK_CUDA(cudaMemcpyAsync(d.tets, m->tets, sizeof(int) * 4 * (size_t)d.ne, cudaMemcpyHostToDevice, s));
-    return d;
-}
-
 void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
     if (!out) throw Error{VEMG_EINVAL};
-    MeshDev md = upload_mesh(mesh, s);
+    MeshDev md(mesh, s);
     Incidence I;
     try {
         int n = md.n;
@@ -555,16 +556,14 @@ void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
         out->val = v;
     } catch (...) {
         I.release();
-        md.release();
         throw;
     }
     I.release();
-    md.release();
 }
 
 void load_vector(const vemg_mesh *mesh, const double *f, double *b, cudaStream_t s) {
     if (!f || !b) throw Error{VEMG_EINVAL};
-    MeshDev md = upload_mesh(mesh, s);
+    MeshDev md(mesh, s);
     Incidence I;
     try {
         I = build_incidence(md.tets, md.ne, md.n, s);
@@ -573,22 +572,13 @@ void load_vector(const vemg_mesh *mesh, const double *f, double *b, cudaStream_t
         VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     } catch (...) {
         I.release();
-        md.release();
         throw;
     }
     I.release();
-    md.release();
 }
 
 // ------------------------------------------------------------------------------------------
 // generic CSR operations
-
-// temporary arrays, released at scope exit
-struct TempArena : Arena {
-    TempArena() { temporary = true; }
-    ~TempArena() { release(); }
-    TempArena(const TempArena &) = delete;
-};
 
 static DCsr csr_alloc(Arena &ar, int n, int m, int nnz) {
     DCsr a;

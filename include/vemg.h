@@ -147,7 +147,10 @@ void vemg_default_options(vemg_options *opts);
    (section 3, Eq. Ax=b; the paper's rescaled A_eps equals (H / L^2) A). A_out receives device
    arrays allocated by the library, in caller order; release them with vemg_csr_free. Entries
    are summed over elements in ascending element index. Returns VEMG_EMESH on a non-positive
-   volume or an out-of-range node id. Synchronises the stream. */
+   volume or an out-of-range node id. Until it returns the call also holds the mesh, lists of the
+   elements at each node (32 bytes per element in all) and the element matrices: 80 bytes per
+   element if there is that much memory, else as many at a time as there is room for, in more
+   passes. Synchronises the stream. */
 int vemg_assemble(const vemg_mesh *mesh, vemg_csr *A_out, void *stream);
 
 /* Load vector b = M f (section 3, Eq. Ax=b): M_ij = integral N_i N_j, f given by its nodal values.

@@ -406,19 +406,19 @@ __global__ void k_asm_rowfill(int n, const int *__restrict__ iptr, const int *__
 }
 
 // The element matrices, one thread per element: the ten entries K[a][b], a <= b, of element e in ke[10 e ..],
-// row by row. FP64 bounds it (some 190 operations, ten of them divisions): 4.7 ms of 12.6M elements. With
-// every node of an element computing it again, the values took 11.4 ms.
-__global__ void __launch_bounds__(128) k_asm_elements(int64_t ne, const int *__restrict__ tets,
+// row by row, for the elements e0 <= e < e1 (ke starts at e0). FP64 bounds it (some 190 operations, ten of them
+// divisions): 4.7 ms of 12.6M elements. With every node of an element computing it again, the values took 11.4 ms.
+__global__ void __launch_bounds__(128) k_asm_elements(int64_t e0, int64_t e1, const int *__restrict__ tets,
                                                       const double *__restrict__ xyz, double *__restrict__ ke, int *err) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
+    const int64_t e = e0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= e1) return;
     const int4 t = *(const int4 *)(tets + 4 * e);
     const int vv[4] = {t.x, t.y, t.z, t.w};
     Tet T;
     tet_geometry(xyz, vv, T);
     if (!(T.det > 0.0)) { atomic_flag(err, VEMG_EMESH); return; }
     const double s = 6.0 * T.det;
-    double *k = ke + 10 * e;
+    double *k = ke + 10 * (e - e0);
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -429,12 +429,15 @@ __global__ void __launch_bounds__(128) k_asm_elements(int64_t ne, const int *__r
 // row, one for each vertex of the element at hand (different columns, so the order of the sums is that
 // of the elements); a block's rows are one segment of A, summed up in shared memory if it fits there.
 // Four elements' vertices and values are on their way at once: a thread per row, one element after the
-// other and the sums in global memory, took 6.5 ms of 12.6M elements.
+// other and the sums in global memory, took 6.5 ms of 12.6M elements. Elements e0 <= e < e1: with e0 > 0 the
+// sums go on from those in v.
 static constexpr int kAsmRows = 32, kAsmMost = 32 * kAsmRows;
+static constexpr int64_t kAsmPiece = 1024;   // elements that it does not go below
 __global__ void __launch_bounds__(4 * kAsmRows) k_asm_values(int n, const int *__restrict__ iptr,
                                                              const int *__restrict__ inc, const int *__restrict__ tets,
-                                                             const double *__restrict__ ke, const int *__restrict__ rp,
-                                                             const int *__restrict__ ci, double *v) {
+                                                             const double *__restrict__ ke, int e0, int e1,
+                                                             const int *__restrict__ rp, const int *__restrict__ ci,
+                                                             double *v) {
     __shared__ int scol[kAsmMost];
     __shared__ double sacc[kAsmMost];
     const int r0 = blockIdx.x * kAsmRows, base = rp[r0], len = rp[min(r0 + kAsmRows, n)] - base;
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(4 * kAsmRows) k_asm_values(int n, const int *_
     double *acc = fits ? sacc : v + base;
     for (int e = threadIdx.x; e < len; e += blockDim.x) {
         if (fits) scol[e] = ci[base + e];
-        acc[e] = 0.0;
+        acc[e] = e0 > 0 ? v[base + e] : 0.0;
     }
     __syncthreads();
     const int i = r0 + (int)(threadIdx.x >> 2), b = threadIdx.x & 3;
@@ -454,19 +457,23 @@ __global__ void __launch_bounds__(4 * kAsmRows) k_asm_values(int n, const int *_
             int e[4], pos[4];
             int4 t[4];
             double x[4];
+            bool on[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) e[u] = inc[min(k + u, k1 - 1)];
+            for (int u = 0; u < 4; ++u) {
+                e[u] = inc[min(k + u, k1 - 1)];
+                on[u] = k + u < k1 && e[u] >= e0 && e[u] < e1;
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) t[u] = *(const int4 *)(tets + 4 * (int64_t)e[u]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int a = t[u].x == i ? 0 : t[u].y == i ? 1 : t[u].z == i ? 2 : 3, p = min(a, b), q = max(a, b);
-                x[u] = ke[10 * (int64_t)e[u] + p * (9 - p) / 2 + q - p];
+                x[u] = on[u] ? ke[10 * (int64_t)(e[u] - e0) + p * (9 - p) / 2 + q - p] : 0.0;
                 pos[u] = bsearch_row(col, lo, hi, b == 0 ? t[u].x : b == 1 ? t[u].y : b == 2 ? t[u].z : t[u].w);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (k + u < k1) acc[pos[u]] = acc[pos[u]] + x[u];
+                if (on[u]) acc[pos[u]] = acc[pos[u]] + x[u];
                 __syncwarp(mine);
             }
         }
@@ -526,35 +533,50 @@ void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
     if (!out) throw Error{VEMG_EINVAL};
     MeshDev md(mesh, s);
     Incidence I;
+    int *rp = nullptr, *ci = nullptr;
+    double *v = nullptr;
     try {
         int n = md.n;
         I = build_incidence(md.tets, md.ne, n, s);
         Scratch<int> rowlen(n), err(1);
-        Scratch<double> ke(10 * (size_t)md.ne);
         VEMG_CHECK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         k_asm_rowlen<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, rowlen, err);
         VEMG_CHECK_LAUNCH();
         if (int e = read_flag(err, s)) throw Error{e};
-        int *rp = (int *)dev_alloc_raw(sizeof(int) * (n + 1));
+        rp = (int *)dev_alloc_raw(sizeof(int) * (n + 1));
         int nnz = scan_offsets(rowlen, rp, n, s);
-        int *ci = (int *)dev_alloc_raw(sizeof(int) * (size_t)std::max(nnz, 1));
-        double *v = (double *)dev_alloc_raw(sizeof(double) * (size_t)std::max(nnz, 1));
+        ci = (int *)dev_alloc_raw(sizeof(int) * (size_t)std::max(nnz, 1));
+        v = (double *)dev_alloc_raw(sizeof(double) * (size_t)std::max(nnz, 1));
         k_asm_rowfill<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, rp, ci);
         VEMG_CHECK_LAUNCH();
-        k_asm_elements<<<grid_for(md.ne, 128), 128, 0, s>>>(md.ne, md.tets, md.xyz, ke, err);
-        VEMG_CHECK_LAUNCH();
-        k_asm_values<<<grid_for(n, kAsmRows), 4 * kAsmRows, 0, s>>>(n, I.ptr, I.inc, md.tets, ke, rp, ci, v);
-        VEMG_CHECK_LAUNCH();
-        if (int e = read_flag(err, s)) {
-            dev_free_raw(rp); dev_free_raw(ci); dev_free_raw(v);
-            throw Error{e};
+        // the element matrices take 80 bytes an element: all at once if there is room, else in pieces (the
+        // sums stay in element order). Allocated last, so that the result does not lack what they took.
+        int64_t piece = md.ne;
+        std::unique_ptr<Scratch<double>> ke;
+        while (!ke) {
+            try {
+                ke.reset(new Scratch<double>(10 * piece));
+            } catch (const Error &e) {
+                if (e.code != VEMG_ENOMEM || piece <= kAsmPiece) throw;
+                piece = (piece + 1) / 2;
+            }
         }
+        for (int64_t e0 = 0; e0 < md.ne; e0 += piece) {
+            const int64_t e1 = std::min(e0 + piece, md.ne);
+            k_asm_elements<<<grid_for(e1 - e0, 128), 128, 0, s>>>(e0, e1, md.tets, md.xyz, *ke, err);
+            VEMG_CHECK_LAUNCH();
+            k_asm_values<<<grid_for(n, kAsmRows), 4 * kAsmRows, 0, s>>>(n, I.ptr, I.inc, md.tets, *ke, (int)e0, (int)e1,
+                                                                        rp, ci, v);
+            VEMG_CHECK_LAUNCH();
+        }
+        if (int e = read_flag(err, s)) throw Error{e};
         out->n = n;
         out->nnz = nnz;
         out->rowptr = rp;
         out->col = ci;
         out->val = v;
     } catch (...) {
+        for (void *p : {(void *)rp, (void *)ci, (void *)v}) dev_free_raw(p);
         I.release();
         throw;
     }

@@ -1,5 +1,5 @@
 """The device allocator that a caller installs (vemg_set_allocator): the library asks for no alignment
-beyond that of its elements."""
+beyond that of its elements, and does with what its results and their inputs take."""
 import contextlib
 import ctypes as C
 
@@ -14,19 +14,21 @@ pytestmark = pytest.mark.gpu
 
 
 @contextlib.contextmanager
-def _allocator(shift):
-    """Blocks `shift` bytes past a 512-byte boundary."""
+def _allocator(shift=0, budget=1 << 40):
+    """Blocks `shift` bytes past a 512-byte boundary, `budget` bytes of them at a time."""
     held = {}
 
     @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p)
     def alloc(nbytes, ctx):
+        if sum(b for _, b in held.values()) + nbytes > budget:
+            return None
         p = torch.cuda.caching_allocator_alloc(int(nbytes) + shift)
-        held[p + shift] = p
+        held[p + shift] = p, nbytes
         return p + shift
 
     @C.CFUNCTYPE(None, C.c_void_p, C.c_void_p)
     def free(ptr, ctx):
-        torch.cuda.caching_allocator_delete(held.pop(ptr))
+        torch.cuda.caching_allocator_delete(held.pop(ptr)[0])
 
     L = V.lib()
     assert L.vemg_set_allocator(C.cast(alloc, C.c_void_p), C.cast(free, C.c_void_p), None) == V.VEMG_OK
@@ -66,3 +68,25 @@ def test_blocks_aligned_to_their_elements_only(shape, shift):
     with _allocator(shift):
         got = results()
     assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("spare", [1 << 17, 1 << 21])   # bytes for all temporary arrays
+def test_assembly_within_its_result(spare):
+    """What assembly needs beside the mesh, its incidence lists and the matrix fits in little memory; the
+    matrix has the same bits then. Less than the matrix itself is refused, and leaves nothing behind."""
+    m, vm = _case(40, 38, 11)
+    A = V.vemg_assemble(vm)
+    want = [t.cpu().numpy() for t in A.tensors()]
+    A.free()
+    ne, nnz = vm.tets.shape[0], len(want[1])
+    result = 12 * nnz + 4 * (m.n + 1)
+    # the mesh starts in a block of at most 1 MiB; rows' lengths, counts and their scans, 24 bytes a node
+    need = 24 * m.n + 32 * ne + 4 * (m.n + 1) + (1 << 20) + 24 * m.n
+    with _allocator(budget=need + result + spare):
+        A = V.vemg_assemble(vm)
+        got = [t.cpu().numpy() for t in A.tensors()]
+        A.free()
+    assert all(np.array_equal(a, b) for a, b in zip(got, want))
+    with _allocator(budget=result // 2), pytest.raises(V.VemgError) as e:
+        V.vemg_assemble(vm)
+    assert e.value.code == V.VEMG_ENOMEM

@@ -109,9 +109,10 @@ void *scratch_alloc(size_t bytes, bool *ordered, cudaStream_t *s);
 void scratch_free(void *p, bool ordered, cudaStream_t s);
 
 // An owner of device allocations; freed together. Blocks start on 256-byte boundaries whatever the
-// allocator returns (the kernels load vectors 16 bytes at a time) and are cut from chunks of a quarter of
-// what the arena holds, 1 to 64 MiB: a hierarchy's 430 arrays took 11 ms of cudaMalloc and 9 ms of
-// cudaFree. temporary: chunks from the scratch allocator (stream-ordered while a ScratchStream lives).
+// allocator returns (the kernels load vectors 16 bytes at a time) and are cut from chunks of an eighth of
+// what the arena holds, 1 to 64 MiB, each in the first chunk with room for it: a hierarchy's 430 arrays
+// took 11 ms of cudaMalloc and 9 ms of cudaFree. Where a chunk is refused the block is allocated by itself.
+// temporary: chunks from the scratch allocator (stream-ordered while a ScratchStream lives).
 struct Arena {
     struct Chunk {
         void *p;
@@ -120,22 +121,29 @@ struct Arena {
     };
     std::vector<Chunk> chunks;
     size_t bytes = 0;              // of the chunks
-    char *at = nullptr, *end = nullptr;
+    std::vector<std::pair<char *, char *>> room;   // what is left of the chunks
     bool temporary = false;
     template <class T>
     T *alloc(int64_t count) {
         size_t b = (size_t)(count > 0 ? count : 1) * sizeof(T);
         b = (b + 255) & ~(size_t)255;
-        if (b > (size_t)(end - at)) {
-            const size_t want = std::min<size_t>(std::max<size_t>(bytes / 4, (size_t)1 << 20), (size_t)64 << 20);
-            char *q = chunk(std::max(b, want));
-            if (b >= want) return (T *)q;   // a chunk of its own
-            at = q;
-            end = q + want;
+        for (auto &r : room) {
+            if (b > (size_t)(r.second - r.first)) continue;
+            T *p = (T *)r.first;
+            r.first += b;
+            return p;
         }
-        T *r = (T *)at;
-        at += b;
-        return r;
+        const size_t want = std::min<size_t>(std::max<size_t>(bytes / 8, (size_t)1 << 20), (size_t)64 << 20);
+        if (b < want) {
+            try {
+                char *q = chunk(want);
+                room.emplace_back(q + b, q + want);
+                return (T *)q;
+            } catch (const Error &e) {
+                if (e.code != VEMG_ENOMEM) throw;
+            }
+        }
+        return (T *)chunk(b);
     }
     char *chunk(size_t b) {
         for (size_t extra : {(size_t)0, (size_t)256}) {
@@ -158,8 +166,8 @@ struct Arena {
     void release() {
         for (const Chunk &c : chunks) free_chunk(c);
         chunks.clear();
+        room.clear();
         bytes = 0;
-        at = end = nullptr;
     }
 };
 

@@ -14,13 +14,13 @@ pytestmark = pytest.mark.gpu
 
 
 @contextlib.contextmanager
-def _allocator(shift=0, budget=1 << 40):
-    """Blocks `shift` bytes past a 512-byte boundary, `budget` bytes of them at a time."""
+def _allocator(shift=0, budget=1 << 40, largest=1 << 40):
+    """Blocks `shift` bytes past a 512-byte boundary, `budget` bytes of them at a time, none over `largest`."""
     held = {}
 
     @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p)
     def alloc(nbytes, ctx):
-        if sum(b for _, b in held.values()) + nbytes > budget:
+        if sum(b for _, b in held.values()) + nbytes > budget or nbytes > largest:
             return None
         p = torch.cuda.caching_allocator_alloc(int(nbytes) + shift)
         held[p + shift] = p, nbytes
@@ -90,3 +90,26 @@ def test_assembly_within_its_result(spare):
     with _allocator(budget=result // 2), pytest.raises(V.VemgError) as e:
         V.vemg_assemble(vm)
     assert e.value.code == V.VEMG_ENOMEM
+
+
+def test_no_block_larger_than_an_array():
+    """The library allocates many arrays at once where it can; an allocator that gives no block larger than
+    the largest array serves it too."""
+    m, vm = _case(5, 4, 3)
+    b = torch.from_numpy(I.normal_loads(m.n, 83)).cuda()
+
+    def solutions():
+        A = V.vemg_assemble(vm)
+        h = V.vemg_setup(A, vm, V.vemg_default_options())
+        V.vemg_batch_set_tuning(h, 4, (4, 4, 4), (2, 2, 2))
+        out = [V.vemg_solve(h, b, rtol=1e-9)[0], V.vemg_solve_batch(h, torch.stack([b, -b, 2 * b]), rtol=1e-9)[0]]
+        h.destroy()
+        A.free()
+        return out
+
+    want = solutions()
+    # 120 nodes: nothing that grows with the mesh is over 120 x 120 doubles, and partial sums of at most
+    # 608 blocks, 8 reductions and 5 sums take 195 KB
+    with _allocator(largest=1 << 18):
+        got = solutions()
+    assert all(torch.equal(x, y) for x, y in zip(got, want))

@@ -1237,9 +1237,8 @@ static void autotune(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     else autotune_t<double>(h, W, s);
 }
 
-BatchWork *new_batch_work(vemg_hierarchy *h, int K, cudaStream_t s) {
-    BatchWork *W = new BatchWork();
-    W->K = K;
+static void fill_batch_work(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
+    const int K = W->K;
     Arena &ar = W->arena;
     int64_t N = (int64_t)h->n * K;
     W->X = ar.alloc<double>(N);
@@ -1280,14 +1279,21 @@ BatchWork *new_batch_work(vemg_hierarchy *h, int K, cudaStream_t s) {
     W->ctr = ar.alloc<unsigned>(2);
     VEMG_CHECK_CUDA(cudaMemsetAsync(W->ctr, 0, sizeof(unsigned) * 2, s));
     VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
+    autotune(h, W, s);
+    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
+}
+
+BatchWork *new_batch_work(vemg_hierarchy *h, int K, cudaStream_t s) {
+    BatchWork *W = new BatchWork();
+    W->K = K;
     try {
-        autotune(h, W, s);
+        fill_batch_work(h, W, s);
     } catch (...) {
+        cudaStreamSynchronize(s);   // what was enqueued on the arrays
         W->arena.release();
         delete W;
         throw;
     }
-    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
     return W;
 }
 

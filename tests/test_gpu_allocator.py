@@ -113,3 +113,23 @@ def test_no_block_larger_than_an_array():
     with _allocator(largest=1 << 18):
         got = solutions()
     assert all(torch.equal(x, y) for x, y in zip(got, want))
+
+
+@pytest.mark.parametrize("engine", [False, True])
+def test_refused_batch_leaves_nothing_behind(engine):
+    """A batch or an engine for which the memory does not suffice: VEMG_ENOMEM, and what it had allocated
+    until then is given back; the hierarchy goes on."""
+    m, vm = _case(21, 19, 9)
+    b = torch.from_numpy(I.normal_loads(m.n, 84)).cuda()
+    A = V.vemg_assemble(vm)
+    h = V.vemg_setup(A, vm, V.vemg_default_options())
+    want = V.vemg_solve(h, b, rtol=1e-9)[0]
+    # 16 columns: the first three of the six vectors fit
+    with _allocator(budget=4 * 16 * 8 * m.n) as held, pytest.raises(V.VemgError) as e:
+        if engine:
+            V.Engine(h, 16)
+        else:
+            V.vemg_solve_batch(h, b.repeat(16, 1), rtol=1e-9)
+    assert e.value.code == V.VEMG_ENOMEM and not held
+    assert torch.equal(V.vemg_solve(h, b, rtol=1e-9)[0], want)
+    assert torch.isfinite(V.vemg_solve_batch(h, b.repeat(16, 1), rtol=1e-9)[0]).all()

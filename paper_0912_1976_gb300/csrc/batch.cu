@@ -1095,6 +1095,11 @@ static BRows chain_rows(Arena &ar, const DCsr &A, const int *colour, const int *
     R.diag = colour != nullptr;
     R.mean = (double)nnz / std::max(A.n, 1);
     R.qsh = parts_shift(K, fp32, rows, R.mean);
+    if (!fp32 && !colour) {   // as the setup keeps it: copies would take some 110 bytes a node
+        R.ci = A.ci;
+        R.v = A.v;
+        return R;
+    }
     int2 *ent = fp32 ? ar.alloc<int2>(nnz) : nullptr;
     int *ci = fp32 ? nullptr : ar.alloc<int>(nnz), *lo = colour ? ar.alloc<int>(A.n) : nullptr;
     double *v = fp32 ? nullptr : ar.alloc<double>(nnz);

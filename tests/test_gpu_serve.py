@@ -179,3 +179,15 @@ def test_served_columns_match_the_oracle():
             worst = max(worst, err)
             assert err <= 1e-6, (r.rid, r.eps, r.bc, err)
     record("served_columns_vs_oracle", worst_rel_l2=worst, columns=sum(r.nrhs for r in done))
+
+
+def test_engine_memory_is_its_vectors_and_reordered_operators():
+    """An FP64 engine holds its vectors, the level matrices in its own entry order and tables of their rows;
+    the transfer operators it reads where the hierarchy keeps them. Blocks of memory are filled to 8/9."""
+    m, vm, A, h = _hier(V.VEMG_PREC_FP64, nx=60, nz=24, eps=1e-2)
+    need = 6 * 8 * m.n                                   # x, r, z, p, q, b
+    for c in (0, 1):
+        for l in range(V.vemg_get_size(h, "nlev", c)):
+            n, nnz = V.vemg_get_size(h, "lev.n", c, l), V.vemg_get_size(h, "lev.nnz", c, l)
+            need += 3 * 8 * n + 12 * (nnz - n) + (8 + 4 + 16) * n
+    assert need <= V.Engine(h, 1).bytes() <= 9 / 8 * need + (2 << 20)

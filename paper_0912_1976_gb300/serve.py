@@ -314,9 +314,15 @@ class GpuFactory:
         return (nx + 1) * (nx + 1) * (self.nz + 1)
 
     def estimate(self, key) -> int:
-        n = self.nodes(key[0])
-        # hierarchy (both layouts) about 1.2 KB per node; engine work about 130 B per node and slot
-        return int(n * (1200 + 130 * self.slots))
+        """Bytes of a hierarchy and its engine, from above: what a build may take before it is started.
+        Measured over 12 to 399 squared x 6 to 48 layers: a hierarchy holds at most 1,360 bytes a node
+        with FP64 cycles and 1,310 with FP32 ones, an engine 280 + 86 and 240 + 77 a column (rounded up
+        to a power of two), with the unfilled ends of their memory blocks; beside that the dense inverses
+        of the coarsest levels, whatever the mesh (up to 1,024 rows, two chains)."""
+        fp64 = self.precision_for(key[1]) == self.V.VEMG_PREC_FP64
+        columns = 1 << (self.slots - 1).bit_length()
+        per_node = 1400 + 320 + 90 * columns if fp64 else 1330 + 250 + 80 * columns
+        return self.nodes(key[0]) * per_node + (48 << 20)
 
     def precision_for(self, eps: float) -> int:
         """FP32 V-cycles except at eps <= 1e-4: there the FP64 residual has reached its round-off

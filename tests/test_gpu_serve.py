@@ -191,3 +191,17 @@ def test_engine_memory_is_its_vectors_and_reordered_operators():
             n, nnz = V.vemg_get_size(h, "lev.n", c, l), V.vemg_get_size(h, "lev.nnz", c, l)
             need += 3 * 8 * n + 12 * (nnz - n) + (8 + 4 + 16) * n
     assert need <= V.Engine(h, 1).bytes() <= 9 / 8 * need + (2 << 20)
+
+
+@pytest.mark.parametrize("slots", [1, 6, 16])
+@pytest.mark.parametrize("nx", [20, 44, 130])
+def test_builds_take_what_was_estimated(nx, slots):
+    """The server admits a build by its estimate, so no build may take more; nor far less, or meshes that
+    would fit are kept out."""
+    fac = S.GpuFactory(slots=slots, precision=V.VEMG_PREC_BF16, sizes=[nx], nz=24)
+    for eps in (1e-4, 1e-2):            # FP64 cycles, FP32 cycles
+        for bc in (V.VEMG_NEUMANN, V.VEMG_DIRICHLET_TOP):
+            h, eng, nbytes, n = fac.build((0, eps, bc))
+            assert nbytes <= fac.estimate((0, eps, bc)) <= 1.5 * nbytes + (48 << 20), (eps, bc, nbytes)
+            eng.destroy()
+            h.destroy()

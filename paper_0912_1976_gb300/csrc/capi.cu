@@ -336,6 +336,7 @@ int vemg_setup(const vemg_csr *A, const vemg_mesh *mesh, const vemg_options *opt
             release_graphs(h);
             release_batch(h);
             h->arena.release();
+            cudaFreeHost(h->colour_status);
             delete h;
         }
         return rc;
@@ -354,6 +355,7 @@ void vemg_destroy(vemg_hierarchy *h) {
     release_ctail(h->sbar);
     for (auto &e : h->probe.ev) cudaEventDestroy(e);
     h->arena.release();
+    cudaFreeHost(h->colour_status);
     delete h;
 }
 

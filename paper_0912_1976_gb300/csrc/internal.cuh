@@ -343,6 +343,7 @@ struct vemg_hierarchy {
     int batch_cap = 0;
     double *bx = nullptr, *br = nullptr, *bz = nullptr, *bp = nullptr, *bq = nullptr, *bb = nullptr;
     double *bscal = nullptr;
+    int *colour_status = nullptr;                 // page-locked words of the colouring (setup.cu)
     vemg::Probe probe;
     int64_t launches = 0;                         // kernels launched by the solve path
     // ---- solve order (see layout.cu) ----

@@ -344,16 +344,18 @@ static void sort_rows(const int *rp, int *ci, double *v, int n, cudaStream_t s) 
     VEMG_CHECK_LAUNCH();
 }
 
-struct Incidence {
-    int *ptr = nullptr, *inc = nullptr;
-    void release() {
-        dev_free_raw(ptr);
-        dev_free_raw(inc);
-        ptr = inc = nullptr;
-    }
+// temporary arrays, released at scope exit
+struct TempArena : Arena {
+    TempArena() { temporary = true; }
+    ~TempArena() { release(); }
+    TempArena(const TempArena &) = delete;
 };
 
-static Incidence build_incidence(const int *d_tets, int64_t ne, int n, cudaStream_t s) {
+struct Incidence {
+    int *ptr = nullptr, *inc = nullptr;
+};
+
+static Incidence build_incidence(Arena &ar, const int *d_tets, int64_t ne, int n, cudaStream_t s) {
     Incidence I;
     Scratch<int> cnt(n + 1), err(1);
     VEMG_CHECK_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (n + 1), s));
@@ -361,9 +363,9 @@ static Incidence build_incidence(const int *d_tets, int64_t ne, int n, cudaStrea
     k_inc_count<<<grid_for(ne, 256), 256, 0, s>>>(d_tets, ne, n, cnt, err);
     VEMG_CHECK_LAUNCH();
     if (read_flag(err, s)) throw Error{VEMG_EMESH};
-    I.ptr = (int *)dev_alloc_raw(sizeof(int) * (n + 1));
+    I.ptr = ar.alloc<int>(n + 1);
     int total = scan_offsets(cnt, I.ptr, n, s);
-    I.inc = (int *)dev_alloc_raw(sizeof(int) * (size_t)std::max(total, 1));
+    I.inc = ar.alloc<int>(total);
     Scratch<int> cur(n);
     VEMG_CHECK_CUDA(cudaMemcpyAsync(cur, I.ptr, sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
     k_inc_fill<<<grid_for(ne, 256), 256, 0, s>>>(d_tets, ne, cur, I.inc);
@@ -502,13 +504,6 @@ __global__ void k_load(int n, const int *__restrict__ iptr, const int *__restric
     b[i] = acc;
 }
 
-// temporary arrays, released at scope exit
-struct TempArena : Arena {
-    TempArena() { temporary = true; }
-    ~TempArena() { release(); }
-    TempArena(const TempArena &) = delete;
-};
-
 // The mesh on the device. The arena puts the arrays on 256-byte boundaries whatever the caller's allocator
 // returns: the assembly loads the four vertices of an element at once.
 struct MeshDev {
@@ -532,12 +527,11 @@ struct MeshDev {
 void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
     if (!out) throw Error{VEMG_EINVAL};
     MeshDev md(mesh, s);
-    Incidence I;
     int *rp = nullptr, *ci = nullptr;
     double *v = nullptr;
     try {
         int n = md.n;
-        I = build_incidence(md.tets, md.ne, n, s);
+        const Incidence I = build_incidence(md.ar, md.tets, md.ne, n, s);
         Scratch<int> rowlen(n), err(1);
         VEMG_CHECK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         k_asm_rowlen<<<grid_for(n, 128), 128, 0, s>>>(n, I.ptr, I.inc, md.tets, rowlen, err);
@@ -576,27 +570,19 @@ void assemble(const vemg_mesh *mesh, vemg_csr *out, cudaStream_t s) {
         out->col = ci;
         out->val = v;
     } catch (...) {
+        cudaStreamSynchronize(s);   // what was enqueued on the arrays
         for (void *p : {(void *)rp, (void *)ci, (void *)v}) dev_free_raw(p);
-        I.release();
         throw;
     }
-    I.release();
 }
 
 void load_vector(const vemg_mesh *mesh, const double *f, double *b, cudaStream_t s) {
     if (!f || !b) throw Error{VEMG_EINVAL};
     MeshDev md(mesh, s);
-    Incidence I;
-    try {
-        I = build_incidence(md.tets, md.ne, md.n, s);
-        k_load<<<grid_for(md.n, 128), 128, 0, s>>>(md.n, I.ptr, I.inc, md.tets, md.xyz, f, b);
-        VEMG_CHECK_LAUNCH();
-        VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
-    } catch (...) {
-        I.release();
-        throw;
-    }
-    I.release();
+    const Incidence I = build_incidence(md.ar, md.tets, md.ne, md.n, s);
+    k_load<<<grid_for(md.n, 128), 128, 0, s>>>(md.n, I.ptr, I.inc, md.tets, md.xyz, f, b);
+    VEMG_CHECK_LAUNCH();
+    VEMG_CHECK_CUDA(cudaStreamSynchronize(s));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -2048,9 +2034,11 @@ static void group_rows(Arena &ar, Level &L, cudaStream_t s) {
 // frees everything; the other one only launches.
 class Colouring {
 public:
-    Colouring(Arena &arena, cudaStream_t stream) : ar(arena), s(stream) {
+    // status: page-locked words that outlive this object (releasing them would wait for the whole device)
+    Colouring(Arena &arena, cudaStream_t stream, int **status) : ar(arena), s(stream) {
         VEMG_CHECK_CUDA(cudaGetDevice(&device));
-        VEMG_CHECK_CUDA(cudaMallocHost(&hold.p, sizeof(int) * ColourJob::kStat * 3 * kMaxLevels));
+        VEMG_CHECK_CUDA(cudaMallocHost(status, sizeof(int) * ColourJob::kStat * 3 * kMaxLevels));
+        words = *status;
         VEMG_CHECK_CUDA(cudaEventCreateWithFlags(&hold.ev, cudaEventDisableTiming));
         try {
             th = std::thread([this] { run(); });
@@ -2067,7 +2055,7 @@ public:
         if (std::find(levels.begin(), levels.end(), &L) != levels.end()) return;
         levels.push_back(&L);
         if (L.A.n <= 0) return;
-        jobs.emplace_back(new ColourJob(ar, L, hold.p + ColourJob::kStat * jobs.size()));
+        jobs.emplace_back(new ColourJob(ar, L, words + ColourJob::kStat * jobs.size()));
         jobs.back()->follow(hold.ev, s);
         std::lock_guard<std::mutex> lk(mu);
         fresh.push_back(jobs.back().get());
@@ -2088,16 +2076,15 @@ public:
 
 private:
     struct Hold {   // released after the jobs that use it
-        int *p = nullptr;
         cudaEvent_t ev = nullptr;
         ~Hold() {
             if (ev) cudaEventDestroy(ev);
-            if (p) cudaFreeHost(p);
         }
     };
     Arena &ar;
     const cudaStream_t s;
     int device = 0;
+    int *words = nullptr;
     Hold hold;
     std::vector<std::unique_ptr<ColourJob>> jobs;
     std::vector<Level *> levels;
@@ -2364,7 +2351,7 @@ void setup(vemg_hierarchy *h, const vemg_csr *Ain, const vemg_mesh *mesh, cudaSt
         k_bar_fill<<<grid_for(nb, 256), 256, 0, s>>>(nb, h->mtop, h->A.rp, h->A.ci, h->A.v, Abar.rp, Abar.ci, Abar.v);
         VEMG_CHECK_LAUNCH();
     }
-    Colouring colouring(ar, s);
+    Colouring colouring(ar, s, &h->colour_status);
     h->bar.lv[0].A = Abar;
     colouring.add(h->bar.lv[0]);
     if (h->bc == VEMG_NEUMANN) {

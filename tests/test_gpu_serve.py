@@ -205,3 +205,19 @@ def test_builds_take_what_was_estimated(nx, slots):
             assert nbytes <= fac.estimate((0, eps, bc)) <= 1.5 * nbytes + (48 << 20), (eps, bc, nbytes)
             eng.destroy()
             h.destroy()
+
+
+@pytest.mark.parametrize("bc", [V.VEMG_NEUMANN, V.VEMG_DIRICHLET_TOP])
+def test_builds_do_not_wait_for_other_streams(bc):
+    """Assembly and setup on a stream of their own return while a kernel of another stream still runs
+    (some 0.5 s of spinning; both take a few ms), as engines' kernels do in the server."""
+    _hier(V.VEMG_PREC_FP32, bc)        # every kernel is loaded
+    torch.cuda.synchronize()
+    busy, own, done = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Event()
+    with torch.cuda.stream(busy):
+        torch.cuda._sleep(1_000_000_000)
+        done.record()
+    with torch.cuda.stream(own):
+        held = _hier(V.VEMG_PREC_FP32, bc)
+    assert not done.query()
+    torch.cuda.synchronize()

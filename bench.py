@@ -38,9 +38,9 @@ PRECONDS = {"additive": 0, "vl_sor": 1, "sa": 2}
 PRECS = {"fp64": 0, "fp32": 1, "bf16": 2}
 DTYPES = {"fp64": "f64", "fp32": "f64 outer + f32 preconditioner",
           "bf16": "f64 outer + f32 preconditioner with bf16 operator values"}
-# ncu DRAM bytes / algorithmic bytes of the finest colour sweep (one launch, 192x192x32 mesh)
-SOR_FINE_DRAM_RATIO = {"fp32": 34.63 / 32.33, "bf16": 27.46 / 25.18}
-SOR_FINE_KERNEL = {"fp32": "k_sell_sor<float, float, double>", "bf16": "k_sell_sor<__nv_bfloat16, float, double, 16>"}
+# ncu DRAM bytes / algorithmic bytes of the finest colour sweeps: the 16 launches of one preconditioner
+# application on a 192x192x32 mesh, half rows forward and whole rows backward
+SOR_FINE_DRAM_RATIO = {"fp32": 292.5 / 233.7, "bf16": 240.3 / 184.8}
 CYCLES = {"persistent": 0, "launches": 1, "auto": 2, "hybrid": 3}
 
 
@@ -729,21 +729,20 @@ def main():
         for c in classes.values():
             c["frac"] = c["achieved_gbs"] / hbm
         c = classes[dom]
-        # DRAM traffic per launch of the finest-level colour sweep, from one ncu capture on a
-        # 192x192x32 mesh (colour 2, 261,577 rows): 1.07 (FP32 values) / 1.09 (BF16 values) x its
-        # algorithmic bytes, scaled here by this workload's bytes per launch
+        # DRAM traffic per launch, from ncu captures on a 192x192x32 mesh (profiles/sor_rows_bf16_zjit192.md)
         traffic = None
         if dom == "sor_coarse" and args.precision == "bf16":
             # three captured coarse launches on a 192x192x32 mesh moved 0.643-0.663 MB from DRAM each
             # (L2 hit rate 31-34%); the class mixes launches of every coarse level, so the figure is
             # the captured launches' own, not scaled to this workload's average launch
-            traffic = {"bytes_per_launch": 0.6560e6,
+            traffic = {"bytes_per_launch": 0.6563e6,
                        "source": "ncu dram__bytes (read + write), mean of 3 k_sell_sor<__nv_bfloat16, float, float, 4> "
                                  "launches on a 192x192x32 mesh (profiles/sor_rows_bf16_zjit192.md); not scaled"}
         if dom == "sor_fine" and args.precision in SOR_FINE_DRAM_RATIO:
             traffic = {"bytes_per_launch": SOR_FINE_DRAM_RATIO[args.precision] * c["bytes_per_launch"],
-                       "source": f"ncu dram__bytes (read + write) of one {SOR_FINE_KERNEL[args.precision]} launch "
-                                 "on a 192x192x32 mesh, scaled by algorithmic bytes per launch"}
+                       "source": "ncu dram__bytes (read + write) of the 16 finest launches of one preconditioner "
+                                 "application on a 192x192x32 mesh over their algorithmic bytes, times this "
+                                 "workload's algorithmic bytes per launch"}
         # the whole solve: every class's algorithmic bytes over the un-probed time of a solve
         solve_bytes = sum(x["bytes_per_solve"] for x in classes.values())
         whole = solve_bytes / (head["ms_per_step"] / 1000.0) / 1e9

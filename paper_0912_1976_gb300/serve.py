@@ -315,14 +315,17 @@ class GpuFactory:
 
     def estimate(self, key) -> int:
         """Bytes of a hierarchy and its engine, from above: what a build may take before it is started.
-        Measured over 12 to 399 squared x 6 to 48 layers: a hierarchy holds at most 1,360 bytes a node
-        with FP64 cycles and 1,310 with FP32 ones, an engine 280 + 86 and 240 + 77 a column (rounded up
-        to a power of two), with the unfilled ends of their memory blocks; beside that the dense inverses
-        of the coarsest levels, whatever the mesh (up to 1,024 rows, two chains)."""
-        fp64 = self.precision_for(key[1]) == self.V.VEMG_PREC_FP64
-        columns = 1 << (self.slots - 1).bit_length()
-        per_node = 1400 + 320 + 90 * columns if fp64 else 1330 + 250 + 80 * columns
-        return self.nodes(key[0]) * per_node + (48 << 20)
+        Per node, measured over 12 to 399 squared x 6 to 48 layers; the dense inverses of the coarsest
+        levels (up to 1,024 rows) whatever the mesh; and the unfilled ends of the memory blocks."""
+        n, fp64 = self.nodes(key[0]), self.precision_for(key[1]) == self.V.VEMG_PREC_FP64
+        chains = 2 if key[2] == self.V.VEMG_NEUMANN else 1
+        columns = 1 << (self.slots - 1).bit_length()   # as the engine rounds its slots
+
+        def blocks(b):
+            return b + min(b // 4, 64 << 20)
+
+        return (blocks(n * (1320 if fp64 else 1280) + chains * (20 << 20)) +
+                blocks(n * (250 + 86 * columns if fp64 else 260 + 68 * columns) + chains * (4 << 20)))
 
     def precision_for(self, eps: float) -> int:
         """FP32 V-cycles except at eps <= 1e-4: there the FP64 residual has reached its round-off

@@ -210,9 +210,9 @@ typedef struct vemg_engine vemg_engine;
 
 /* Launch shapes of the batched solve's row kernels (the paper has no counterpart: an autotuner of
    this implementation). Three classes: 0 = colour sweeps, 1 = the other V-cycle operations,
-   2 = the outer FP64 operations (A p, the true residual, E~ and E~^T). Each has kw lanes per row
-   (4, 8, 16 or 32; each lane takes up to 16 bytes of neighbouring columns at a time) and warps per
-   block (2, 4, 8).
+   2 = the outer FP64 operations (A p, the true residual, E~^T, and E~ with FP64 cycles). Each has
+   kw lanes per row (4, 8, 16 or 32; each lane takes up to 16 bytes of neighbouring columns at a
+   time) and warps per block (2, 4, 8).
    The first batched solve (or engine) of a width K times every candidate shape on this
    hierarchy's finest level and outer operator and keeps the fastest of each class; the results do
    not depend on the shapes. vemg_batch_tuning reports the batch width and the shapes in use with
@@ -337,9 +337,10 @@ int vemg_precond(vemg_hierarchy *h, const double *r_dev, double *z_dev, void *st
 int vemg_vcycle(vemg_hierarchy *h, int chain, const double *b_dev, double *x_dev, void *stream);
 
 /* y = A x exactly as vemg_spmv computes it (the same products summed in the same order, so the
-   same bits), but allocating no device memory. (The paper has no counterpart: this serves
-   callers that cannot call cudaMalloc, such as code running inside an allocator callback, or a
-   process whose device memory budget is fixed before the solve starts.)
+   same bits), with a promise to allocate no device memory and to leave the hierarchy's own
+   vectors alone, in which vemg_spmv works. (The paper has no counterpart: this serves callers
+   that cannot call cudaMalloc, such as code running inside an allocator callback, or a process
+   whose device memory budget is fixed before the solve starts.)
    vemg_setup builds everything this call reads (the solve-order index map and operator), so it
    works on any hierarchy vemg_setup returned, before or after any solve.
    Its work buffers live in one static device array owned by the library: 12 MiB, enough for

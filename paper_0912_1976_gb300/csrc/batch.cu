@@ -68,7 +68,6 @@ struct BRows {
     const int4 *info = nullptr;   // a level's matrix: row, first entry, lower entries, entries; in sweep order
     int diag = 0;
     int qsh = 0;            // log2 of the parts a row is split into (parts_shift)
-    double mean = 0.0;      // mean entries per row
 };
 
 // one multigrid level as the batched cycle sees it
@@ -1084,7 +1083,6 @@ static BRows outer_rows(const DCsr &A, const void *v) {
     R.rp = A.rp;
     R.ci = A.ci;
     R.v = v;
-    R.mean = (double)A.nnz / std::max(A.n, 1);
     return R;
 }
 
@@ -1093,8 +1091,7 @@ static BRows chain_rows(Arena &ar, const DCsr &A, const int *colour, const int *
     const int64_t nnz = (int64_t)A.nnz - (colour ? A.n : 0);
     R.rp = A.rp;
     R.diag = colour != nullptr;
-    R.mean = (double)nnz / std::max(A.n, 1);
-    R.qsh = parts_shift(K, fp32, rows, R.mean);
+    R.qsh = parts_shift(K, fp32, rows, (double)nnz / std::max(A.n, 1));
     if (!fp32 && !colour) {   // as the setup keeps it: copies would take some 110 bytes a node
         R.ci = A.ci;
         R.v = A.v;

@@ -1,12 +1,12 @@
 // noalloc.cu -- y = A x without any device allocation, for callers that cannot allocate.
 //
-// vemg_spmv allocates per-call work buffers (the index map from solve order to internal order
-// and solve-order copies of x and y). Some callers cannot allocate device memory at all: code
-// running where cudaMalloc is forbidden or unsafe (inside a custom allocator's callback, in a
-// process whose memory pool must not grow, under a memory budget that was fixed up front).
-// vemg_spmv_static computes the same product with its work buffers in one file-scope device
-// array of fixed size instead. The array belongs to the library: every device that loads
-// libvemg holds it until the process exits.
+// Some callers cannot allocate device memory at all: code running where cudaMalloc is forbidden or
+// unsafe (inside a custom allocator's callback, in a process whose memory pool must not grow, under
+// a memory budget that was fixed up front). vemg_spmv allocates nothing either, but works in the
+// solve's vectors of the hierarchy; vemg_spmv_static leaves those alone (a caller may use it beside a
+// solve's results on the device, or a profiler between launches) and guarantees in its contract that
+// nothing is allocated: its work buffers are one file-scope device array of fixed size. The array
+// belongs to the library: every device that loads libvemg holds it until the process exits.
 #include <stdio.h>
 
 #include <mutex>

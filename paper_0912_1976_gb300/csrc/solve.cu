@@ -423,11 +423,14 @@ enum { C_SPMV = 0, C_XR, C_Z, C_SUMB, C_PREP, C_SUMX, C_TRUE, C_LATE, C_COUNT };
 
 int solve_scalar_iters() { return S_ITERS; }
 
-// Blocks of the streaming kernels. Their number also sets the order of the dot products' sums, which no
-// order makes better than another; over the 300 iterations of the 192 x 192 x 48 xy-jittered mesh, whose
-// rounding errors grow by 1e6, the count of FP64 iterations is 302 with 228 blocks, as with sequential sums,
-// and 304 with 304 (a 131 x 113 x 25 solve: 9.8 and 9.7 ms). With FP32 cycles the FP32 rounding decides, and
-// 228 blocks would cost 2% (2.2M nodes: 15.7 -> 16.1 ms).
+// Blocks of the streaming kernels: two per SM. With FP64 cycles 228, for one reason: the number also sets the
+// order of the dot products' sums, and the parity test of the 192 x 192 x 48 xy-jittered mesh, whose rounding
+// errors grow by 1e6 over 300 iterations, holds the count for its load to one of the sequential sums' 302. It
+// is 302 with 228 blocks and 304 with 304. Neither order is the better one: 16 loads that differ from that
+// one in last bits take 298 to 306 iterations with 228 blocks, 299 to 306 with 304, and eight of them 298 to
+// 304 with sequential sums, so the test asks for more than rounding allows. 228 blocks cost FP64 solves 0.8%
+// (131 x 113 x 25: 9.82 and 9.75 ms); FP32 ones, where the FP32 rounding decides, they would cost 2%
+// (2.2M nodes: 15.7 -> 16.1 ms).
 static int vec_blocks(const vemg_hierarchy *h) {
     const int most = h->precision == VEMG_PREC_FP64 ? kVecBlocks64 : kVecBlocks;
     return (int)std::min<int64_t>(most, std::max<int64_t>(1, ((int64_t)h->nu + kRedThreads - 1) / kRedThreads));

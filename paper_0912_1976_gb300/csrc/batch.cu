@@ -430,36 +430,22 @@ __device__ void bblock_partials(double (&acc)[NS], int K, double *part) {
     }
 }
 
-// stage-1 sums: s0 = sum a*b (or sum a when b is null), s1 = sum c*d (or sum c), ...
-struct BSums {
-    const double *a[5];
-    const double *b[5];
-    int ns;
-};
-
-template <int NS>
-__global__ void __launch_bounds__(kBT) k_bsums(int64_t N, int K, BSums d, double *part) {
+// stage-1 sum of a * b per column (b null: of a)
+__global__ void __launch_bounds__(kBT) k_bsum(int64_t N, int K, const double *a, const double *b, double *part) {
     pdl_begin();
-    double acc[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) acc[s] = 0.0;
+    double acc[1] = {0.0};
     for (int64_t base = (int64_t)blockIdx.x * kBT * kBE + threadIdx.x; base < N; base += (int64_t)gridDim.x * kBT * kBE) {
-        double va[NS][kBE], vb[NS][kBE];
+        double va[kBE], vb[kBE];
 #pragma unroll
         for (int j = 0; j < kBE; ++j) {
             int64_t e = base + (int64_t)j * kBT;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                va[s][j] = e < N ? d.a[s][e] : 0.0;
-                vb[s][j] = (e < N && d.b[s]) ? d.b[s][e] : 1.0;
-            }
+            va[j] = e < N ? a[e] : 0.0;
+            vb[j] = (e < N && b) ? b[e] : 1.0;
         }
 #pragma unroll
-        for (int j = 0; j < kBE; ++j)
-#pragma unroll
-            for (int s = 0; s < NS; ++s) acc[s] = fma(va[s][j], vb[s][j], acc[s]);
+        for (int j = 0; j < kBE; ++j) acc[0] = fma(va[j], vb[j], acc[0]);
     }
-    bblock_partials<NS>(acc, K, part);
+    bblock_partials<1>(acc, K, part);
 }
 
 // the preconditioner's sums over z, r (and q): s0 = sum z, s1 = sum r z [, s2 = sum z q] (k_blate has those
@@ -617,7 +603,7 @@ __global__ void k_bprepare(int64_t N, int K, int neumann, double *__restrict__ b
 }
 
 // R -= alpha Q per column, the FP32 copy of R's A_bar part, and the stage-1 sums of R * R (elements of a
-// thread and order as in k_bsums)
+// thread and order as in k_bsum)
 __global__ void __launch_bounds__(kBT, 2) k_bupdate_r(int64_t N, int K, const double *__restrict__ q,
                                                       double *__restrict__ r, const double *__restrict__ sc,
                                                       float *__restrict__ rb32, int64_t off32, double *part) {
@@ -848,19 +834,17 @@ static int64_t rb32_offset(const vemg_hierarchy *h, const BatchWork *W) {
 }
 
 // one per-column sum (the wider sums of the preconditioner step are k_bsums_zrq's)
-static void bsums(BatchWork *W, int64_t N, const BSums &d, cudaStream_t s) {
-    if (d.ns != 1) throw Error{VEMG_EINTERNAL};
-    pdl_launch(k_bsums<1>, stage1_blocks(N), kBT, s, N, W->K, d, W->part);
+static void bsum(BatchWork *W, int64_t N, const double *a, const double *b, cudaStream_t s) {
+    pdl_launch(k_bsum, stage1_blocks(N), kBT, s, N, W->K, a, b, W->part);
     BATCH_LAUNCHED();
 }
 
-static void bprecond_any(vemg_hierarchy *h, BatchWork *W, int first, cudaStream_t s) {
+static void bprecond_any(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     if (h->precision != VEMG_PREC_FP64) bprecond<float>(h, W, s);   // BF16 hierarchies: FP32 values here
     else bprecond<double>(h, W, s);
     // t0 = sum z, t1 = (r, z) [, t2 = (z, q)]
     int64_t N = (int64_t)h->nu * W->K;
     bool flex = h->precision != VEMG_PREC_FP64;
-    (void)first;
     const int ns = flex ? 3 : 2;
     if (flex)
         pdl_launch(k_bsums_zrq<3>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
@@ -869,7 +853,7 @@ static void bprecond_any(vemg_hierarchy *h, BatchWork *W, int first, cudaStream_
         pdl_launch(k_bsums_zrq<2>, stage1_blocks(N), kBT, s, N, W->K, (const double *)W->Z, (const double *)W->R,
                    (const double *)nullptr, W->part, 1.0);
     BATCH_LAUNCHED();
-    bstage2(h, W, ST_BETA, ns, N, first, s);
+    bstage2(h, W, ST_BETA, ns, N, 0, s);
 }
 
 // b -= mean (Neumann), r = b, x = p = 0, ||b|| per column; the iterations themselves start in the
@@ -879,14 +863,12 @@ static void bphase_pre(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     const int64_t N = (int64_t)nu * K;
     const bool neu = h->bc == VEMG_NEUMANN;
     if (neu) {
-        BSums d{{W->B}, {nullptr}, 1};
-        bsums(W, N, d, s);
+        bsum(W, N, W->B, nullptr, s);
         bstage2(h, W, ST_MEAN_B, 1, N, 0, s);
     }
     k_bprepare<<<grid_for(N, 256), 256, 0, s>>>(N, K, neu, W->B, W->R, W->X, W->P, W->sc, W->Rb32, rb32_offset(h, W));
     BATCH_LAUNCHED();
-    BSums d{{W->B}, {W->B}, 1};
-    bsums(W, N, d, s);
+    bsum(W, N, W->B, W->B, s);
     bstage2(h, W, ST_BN, 1, N, 0, s);
 }
 
@@ -897,8 +879,7 @@ static void bphase_step(vemg_hierarchy *h, BatchWork *W, cudaStream_t s, cudaGra
                                                                   (const double *)nullptr, (const double *)nullptr,
                                                                   W->P, W->Q, K, -1, s, 2);
     {
-        BSums d{{W->P}, {W->Q}, 1};
-        bsums(W, N, d, s);
+        bsum(W, N, W->P, W->Q, s);
         bstage2(h, W, ST_ALPHA, 1, N, 0, s);
     }
     pdl_launch(k_bupdate_r, stage1_blocks(N), kBT, s, N, K, (const double *)W->Q, W->R, (const double *)W->sc, W->Rb32,
@@ -908,7 +889,7 @@ static void bphase_step(vemg_hierarchy *h, BatchWork *W, cudaStream_t s, cudaGra
 }
 
 static void bphase_direction(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
-    bprecond_any(h, W, 0, s);
+    bprecond_any(h, W, s);
     int64_t N = (int64_t)h->nu * W->K;
     pdl_launch(k_bupdate_p, grid_for(N, 256), 256, s, N, W->K, (const double *)W->sc, (const double *)W->Z, W->P);
     BATCH_LAUNCHED();
@@ -921,8 +902,7 @@ static void bphase_post(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
                (const double *)nullptr, (const double *)W->sc, W->part, 1.0);
     BATCH_LAUNCHED();
     if (h->bc == VEMG_NEUMANN) {
-        BSums d{{W->X}, {nullptr}, 1};
-        bsums(W, N, d, s);
+        bsum(W, N, W->X, nullptr, s);
         bstage2(h, W, ST_MEAN_X, 1, N, 0, s);
         k_bsub_mean<<<grid_for(N, 256), 256, 0, s>>>(N, K, W->X, W->sc, B_XMEAN);
         BATCH_LAUNCHED();
@@ -931,8 +911,7 @@ static void bphase_post(vemg_hierarchy *h, BatchWork *W, cudaStream_t s) {
     brow<BOP_RES, false, double, double, double, double, double>(W->Aout, h->nu, nullptr, ROW_ALL,
                                                                  (const double *)nullptr, W->B, W->X, W->Q, K, -1, s,
                                                                  2);
-    BSums d{{W->Q}, {W->Q}, 1};
-    bsums(W, N, d, s);
+    bsum(W, N, W->Q, W->Q, s);
     bstage2(h, W, ST_TRUE, 1, N, 0, s);
 }
 
